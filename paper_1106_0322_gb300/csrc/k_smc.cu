@@ -512,121 +512,6 @@ __global__ void __launch_bounds__(BLOCK, 4) k_move_mala(MoveArgs a, int64_t N, i
     }
 }
 
-// ------------------------------------------------- single-coordinate update cycle
-// The paper's own kernel (Section 4.1, "Further details"): a cycle of single-coordinate
-// random-walk Metropolis updates, j = 0..p-1 in order, each proposing beta_j' = beta_j +
-// sd * xi, repeated M times per step. One warp per particle, one launch per step.
-// eta2 = log2(e) X beta lives in shared memory (computed from X^T at the start of the step)
-// and changes by x_.j delta when an update is accepted, so an update costs O(n):
-//   delta l = delta v_j - ln 2 * sum_i [softplus2(eta2_i + x2_ij delta) - softplus2(eta2_i)]
-// with the linear half from v = X^T y. softplus2 = max(eta2, 0) + log2(1 + 2^-|eta2|); the
-// max parts are summed as differences, the log parts as the base-2 logarithm of the
-// product of their factors (each in [1, 2], SITE_CHUNK per product), and each lane keeps
-// that log for its individuals at the current state, so a trial needs one ex2 per
-// individual. The normal is Box-Muller's cosine branch on words 0 and 1 of the Philox
-// block (j, particle, t, TAG_SITE << 16 | m), word 2 the update's uniform.
-constexpr int SITE_CHUNK = 64;
-
-// Per-lane: sum over the lane's individuals r = lane + 32k of max(eta2', 0) - max(eta2, 0)
-// (dm) and log2 of the product of (1 + 2^-|eta2'|) (returned), eta2' = eta2 + x2 delta.
-__device__ __forceinline__ float site_trial(const float* __restrict__ eta, const float* __restrict__ xr, int n,
-                                            int lane, float delta, float& dm)
-{
-    float lq = 0.0f, d = 0.0f;
-    for (int k0 = 0; 32 * k0 < n; k0 += SITE_CHUNK) {
-        float prod = 1.0f;
-        const int r1 = min(n, 32 * (k0 + SITE_CHUNK));
-        for (int r = lane + 32 * k0; r < r1; r += 32) {
-            const float e0 = eta[r];
-            const float e1 = fmaf(xr[r], delta, e0);
-            d += fmaxf(e1, 0.0f) - fmaxf(e0, 0.0f);
-            prod = fmaf(prod, ex2_approx(-fabsf(e1)), prod);
-        }
-        lq += lg2_approx(prod);
-    }
-    dm = d;
-    return lq;
-}
-
-__global__ void k_move_site(SiteArgs a, int64_t N, int p, int n, PriorArgs pr, const float4* __restrict__ stepk, int t,
-                            uint32_t m0, int M, const uint64_t* __restrict__ seedp)
-{
-    extern __shared__ float site_sm[];
-    __shared__ int blk;
-    const int wpc = blockDim.x >> 5;
-    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    if (threadIdx.x == 0) blk = 0;
-    __syncthreads();
-    const float4 sk = stepk[t];
-    float* eta = site_sm + (size_t)w * (size_t)(n + p);
-    float* brow = eta + n;
-    const int64_t i = (int64_t)blockIdx.x * wpc + w;
-    if (i < N) {
-        const uint64_t seed = *seedp;
-        const float coef = sk.y, inv_ac = sk.w;
-        float* bg = a.beta + i * p;
-        for (int j = lane; j < p; j += 32) brow[j] = bg[j];
-        for (int r = lane; r < n; r += 32) eta[r] = 0.0f;
-        __syncwarp();
-        for (int j = 0; j < p; ++j) {  // eta2 = X2 beta, marker by marker (coalesced rows of X^T)
-            const float bj = brow[j];
-            const float* xr = a.XT2 + (size_t)j * n;
-            for (int r = lane; r < n; r += 32) eta[r] = fmaf(xr[r], bj, eta[r]);
-        }
-        float dm;
-        float lq = site_trial(eta, a.XT2, n, lane, 0.0f, dm);  // delta = 0: the current state
-        int nacc = 0;
-        for (int mm = 0; mm < M; ++mm) {
-            const uint32_t m = m0 + (uint32_t)mm;
-            for (int j = 0; j < p; ++j) {
-                const uint4 u = philox4x32_10(make_uint4((uint32_t)j, (uint32_t)i, (uint32_t)t, (TAG_SITE << 16) | m),
-                                              seed_key(seed));
-                float sn, cs;
-                sincospif(2.0f * u01_open_f(u.y), &sn, &cs);
-                const float delta = a.sd * (sqrtf(-2.0f * logf(u01_open_f(u.x))) * cs);
-                const float* xr = a.XT2 + (size_t)j * n;
-                const float lq1 = site_trial(eta, xr, n, lane, delta, dm);
-                const float dsp = warp_sum(dm + (lq1 - lq));
-                const float b0 = brow[j], b1 = b0 + delta;
-                const float dlp = coef * (prior_term(b1, inv_ac, pr.de) - prior_term(b0, inv_ac, pr.de));
-                const float dl = fmaf(delta, a.vy[j], -0.69314718f * dsp);
-                int acc = logf(u01_open_f(u.z)) < dl + dlp;
-                acc = __shfl_sync(0xffffffffu, acc, 0);
-                if (acc) {
-                    for (int r = lane; r < n; r += 32) eta[r] = fmaf(xr[r], delta, eta[r]);
-                    lq = lq1;
-                    if (lane == 0) brow[j] = b1;
-                    ++nacc;
-                }
-                __syncwarp();
-            }
-        }
-        for (int j = lane; j < p; j += 32) bg[j] = brow[j];
-        if (lane == 0 && nacc) atomicAdd(&blk, nacc);
-        // the MH state at the end of the step, in the units the move kernels keep it:
-        // l = beta . v - ln 2 (sum_i max(eta2_i, 0) + sum of the lanes' log products), and the
-        // log-prior term sum
-        if (a.llq) {
-            float mx = 0.0f, yd = 0.0f;
-            FSum lt;
-            for (int r = lane; r < n; r += 32) mx += fmaxf(eta[r], 0.0f);
-            for (int j = lane; j < p; j += 32) {
-                yd = fmaf(brow[j], a.vy[j], yd);
-                lt.add(prior_term(brow[j], inv_ac, pr.de));
-            }
-            const float sp2 = warp_sum(mx + lq);
-            yd = warp_sum(yd);
-            lt = warp_sum(lt);
-            if (lane == 0) {
-                a.llq[i] = make_float2((yd - 0.69314718f * sp2) * a.inv_sp_scale, 0.0f);
-                a.lpq[i] = make_float2(lt.s, lt.c);
-            }
-        }
-    }
-    __syncthreads();
-    if (threadIdx.x == 0 && blk && a.acc_count) atomicAdd(a.acc_count, (unsigned long long)blk);
-}
-
 // ------------------------------------------------------------ last move of a step
 // MH test of the pending proposals (RW, or MALA with the reverse term), then accepted
 // proposals (and their gradients) are copied into the state rows, so that between steps
@@ -1564,10 +1449,7 @@ static unsigned elem_grid(int64_t total)
 
 cudaError_t smc_init_attributes()
 {
-    cudaError_t e = cudaFuncSetAttribute(k_summaries, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SUM_STAGED_MAX);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(k_move_site, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SITE_SMEM_MAX);
-    return e;
+    return cudaFuncSetAttribute(k_summaries, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SUM_STAGED_MAX);
 }
 
 cudaError_t launch_init_prior(float* beta, int64_t N, int p, PriorArgs pr, const double* sched, int t0,
@@ -1633,25 +1515,6 @@ cudaError_t launch_move_commit(const MoveArgs& a, bool mala, int64_t N, int p, P
     }
     if (vec) return cudaLaunchKernelEx(&cfg, k_move_commit<false, true>, a, N, p, pr, stepk, t, m_prev, seed, err);
     return cudaLaunchKernelEx(&cfg, k_move_commit<false, false>, a, N, p, pr, stepk, t, m_prev, seed, err);
-}
-
-int site_warps_per_block(int64_t n, int p)
-{
-    const int64_t per = (n + p) * (int64_t)sizeof(float);
-    int64_t w = (int64_t)SITE_SMEM_MAX / (per > 0 ? per : 1);
-    if (w > 8) w = 8;
-    return (int)w;
-}
-
-cudaError_t launch_move_site(const SiteArgs& a, int64_t N, int p, int64_t n, PriorArgs pr, const float4* stepk, int t,
-                             uint32_t m0, int M, const uint64_t* seed, cudaStream_t st)
-{
-    if (M <= 0) return cudaSuccess;
-    const int wpc = site_warps_per_block(n, p);
-    if (wpc < 1) return cudaErrorInvalidValue;
-    const size_t smem = (size_t)wpc * (size_t)(n + p) * sizeof(float);
-    k_move_site<<<(unsigned)((N + wpc - 1) / wpc), 32 * wpc, smem, st>>>(a, N, p, (int)n, pr, stepk, t, m0, M, seed);
-    return cudaGetLastError();
 }
 
 cudaError_t launch_finish_loglik(const MhState& s, int64_t N, double* logw, double* ll_out, uint32_t* err,

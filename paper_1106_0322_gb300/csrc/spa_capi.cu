@@ -192,6 +192,7 @@ struct spa_ctx {
     __nv_bfloat16* GT = nullptr;  // [p][n_r] for the adjoint
     float* yv = nullptr;
     float* XT2 = nullptr;  // [p][n] X^T log2(e) for the single-coordinate kernel
+    float* XS = nullptr;   // the same in its register variant's order (allocated on first use)
     uint32_t* ybits = nullptr;  // y as a bitmask, one word per 32 individuals
     int64_t ywords = 0;
     int64_t n_r = 0;
@@ -249,6 +250,7 @@ int check_device(spa_ctx* c)
         return fail(c, SPA_EUNSUPPORTED, "the library is built for sm_103a (compute capability 10.x)");
     CK(tc_init_attributes(), "tensor-core kernel attributes");
     CK(smc_init_attributes(), "summaries kernel attributes");
+    CK(site_init_attributes(), "single-coordinate kernel attributes");
     CK(map_init_attributes(), "MAP kernel attributes");
     if (c) {
         c->device = dev;
@@ -580,6 +582,17 @@ int ensure_mala_buffers(spa_ctx* c)
     if (e == cudaSuccess && plain && !w.eta) e = dalloc(&w.eta, (size_t)(N * n + tiles * N));
     if (e == cudaSuccess && plain && !w.grad) e = dalloc(&w.grad, (size_t)(N * p));
     if (e != cudaSuccess) return cuda_fail(c, e, "MALA buffers");
+    return SPA_OK;
+}
+
+// The single-coordinate register kernel's copy of X (n small enough for that kernel).
+int ensure_site_store(spa_ctx* c)
+{
+    const int64_t count = site_xs_floats(c->n, c->p);
+    if (count == 0 || c->XS) return SPA_OK;
+    cudaError_t e = dalloc(&c->XS, (size_t)count);
+    if (e != cudaSuccess) return cuda_fail(c, e, "single-coordinate store");
+    CK(launch_store_xsite(c->XT2, c->n, c->p, c->XS, c->stream()), "store X for the single-coordinate kernel");
     return SPA_OK;
 }
 
@@ -963,7 +976,7 @@ private:
         }
         if (site_) {
             const float inv_sp = c->cfg.precision == SPA_PREC_SPLIT_BF16 ? (float)LOG2E : 1.0f;
-            const SiteArgs sa{w.beta, w.llq, w.lpq, inv_sp, c->XT2, c->colf + c->p, (float)c->cfg.site_sd, acc};
+            const SiteArgs sa{w.beta, w.llq, w.lpq, inv_sp, c->XT2, c->XS, c->colf + c->p, (float)c->cfg.site_sd, acc};
             q.ck(launch_move_site(sa, w.N, (int)c->p, c->n, c->pr, c->rb.stepk, t, m0, M_, c->rb.seed, q.st));
             st_ = after;
             return;
@@ -1043,6 +1056,7 @@ int upload_data(spa_ctx* c, const int8_t* G, const uint8_t* y)
     CK(launch_store_pack_t(c->G, c->y, n, p, c->n_r, c->GT, c->yv, st), "store pack transposed");
     CK(launch_store_ybits(c->y, n, c->ywords, c->ybits, st), "store y bits");
     CK(launch_store_xt2(c->Xf, n, p, c->XT2, st), "store X transposed");
+    if (c->XS) CK(launch_store_xsite(c->XT2, n, p, c->XS, st), "store X for the single-coordinate kernel");
     c->lip_ok = false;  // new data: the MAP solver's curvature bound is recomputed on demand
     return read_error_word(c);
 }
@@ -1055,7 +1069,7 @@ void destroy(spa_ctx* c)
     free_runbufs(c->rb);
     dfree(c->G); dfree(c->y); dfree(c->sums); dfree(c->mean); dfree(c->sd); dfree(c->v); dfree(c->unit_c); dfree(c->unit_k);
     dfree(c->l2e_s); dfree(c->mean_f); dfree(c->colf); dfree(c->Xf); dfree(c->Gbf); dfree(c->d_err); dfree(c->GT); dfree(c->yv);
-    dfree(c->ybits); dfree(c->XT2); dfree(c->lip);
+    dfree(c->ybits); dfree(c->XT2); dfree(c->XS); dfree(c->lip);
     if (c->ev_fork) cudaEventDestroy(c->ev_fork);
     if (c->ev_keys) cudaEventDestroy(c->ev_keys);
     if (c->ev_join) cudaEventDestroy(c->ev_join);
@@ -1315,6 +1329,7 @@ int batch_build(spa_batch* b, spa_ctx* const* ctxs, int32_t R, const spa_batch_a
         if (rc == SPA_OK) rc = ensure_workspace(c, N);
         if (rc == SPA_OK) rc = ensure_runbufs(c, T);
         if (rc == SPA_OK && c->cfg.move_kind == SPA_MOVE_MALA) rc = ensure_mala_buffers(c);
+        if (rc == SPA_OK && c->cfg.move_kind == SPA_MOVE_SITE) rc = ensure_site_store(c);
         if (rc == SPA_OK) {
             cudaError_t e = cudaMemcpyAsync(c->rb.sched, sched, sizeof(double) * (size_t)T, cudaMemcpyHostToDevice,
                                             c->stream());
@@ -1566,6 +1581,10 @@ static int run_common(spa_ctx* c, const double* sched, bool sched_on_device, int
     if (rc != SPA_OK) return rc;
     if (c->cfg.move_kind == SPA_MOVE_MALA) {
         rc = ensure_mala_buffers(c);
+        if (rc != SPA_OK) return rc;
+    }
+    if (c->cfg.move_kind == SPA_MOVE_SITE) {
+        rc = ensure_site_store(c);
         if (rc != SPA_OK) return rc;
     }
     cudaStream_t st = c->stream();

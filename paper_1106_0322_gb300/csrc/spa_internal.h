@@ -115,11 +115,17 @@ struct SiteArgs {
     float2* lpq;                      //   and log-prior term sum pair, as the MH state keeps them
     float inv_sp_scale;               // partial units per nat
     const float* XT2;                 // [p][n] standardised genotypes times log2(e)
+    const float* XS;                  // the same in the register kernel's order (launch_store_xsite), or NULL
     const float* vy;                  // v = X^T y (nats)
     float sd;                         // proposal standard deviation
     unsigned long long* acc_count;   // accepted coordinate updates (may be NULL)
 };
 constexpr size_t SITE_SMEM_MAX = 220 * 1024;  // eta2 and beta rows of a block's particles
+// The register kernel's copy of X^T log2(e): floats it takes (0: n is too large for that
+// kernel), and the pack from XT2 [p][n].
+int64_t site_xs_floats(int64_t n, int64_t p);
+cudaError_t launch_store_xsite(const float* XT2, int64_t n, int64_t p, float* XS, cudaStream_t st);
+cudaError_t site_init_attributes();
 // Particles per block (one warp each) for n individuals and p markers; 0 if one does not fit.
 int site_warps_per_block(int64_t n, int p);
 cudaError_t launch_move_site(const SiteArgs& a, int64_t N, int p, int64_t n, PriorArgs pr, const float4* stepk, int t,

@@ -1,0 +1,37 @@
+"""Kernel variants chosen by size, at the edges of their ranges, against the oracle."""
+import numpy as np
+import pytest
+
+import oracle
+from paper_1106_0322_gb300 import synth
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def spa():
+    import __graft_entry__
+
+    __graft_entry__.build()
+    import paper_1106_0322_gb300 as mod
+
+    return mod
+
+
+# The single-coordinate cycle keeps eta in registers for n <= 2048 (4 to 64 individuals per
+# lane, in steps of 4) and in shared memory above; updates go 32 at a time.
+@pytest.mark.parametrize("n,p,N", [(31, 1, 3), (33, 5, 64), (128, 32, 65), (129, 33, 64), (500, 20, 33), (1536, 6, 64),
+                                   (1537, 6, 64), (2048, 7, 64), (2049, 7, 64)])
+def test_site_register_and_shared_kernels_at_their_edges(spa, n, p, N):
+    """With one seed both sides draw the same Philox blocks, so the first step's updates take
+    the same decisions except where a log ratio lies within the kernels' rounding (about 1e-5)
+    of log U. A flipped update moves one of N p acceptances, and one particle's coordinate by
+    about one proposal step (0.5 sd) with its weight of order 1/N; up to two flips are allowed."""
+    reg = synth.make_region(n, p, 0.9, (0.5,), seed=1200 + n)
+    sched = synth.geometric_schedule(2, -3.0, -2.0)
+    with spa.Region(reg.G, reg.y, 1.0, config=spa.make_config(move="site", init="resample_move")) as r:
+        g = r.run(sched, N, 1, 11)
+    o = oracle.run(reg.G, reg.y, 1.0, sched, N, 1, seed=11,
+                   cfg=oracle.make_config(move="site", init="mcmc"))
+    assert abs(g["accept_rate"][0] - o["accept_rate"][0]) <= 2.0 / (N * p) + 1e-12
+    assert np.max(np.abs(g["mean"][0] - o["mean"][0])) <= 2 * 2.0 / N + 1e-4
