@@ -81,28 +81,6 @@ struct TcCfg {
     static_assert(AR != 2 || A_COL + 2 * KB_RES * 32 <= TMEM_COLS, "A_hi | A_lo must fit beside the accumulators");
 };
 
-// Sum over the first `valid` of 32 columns of softplus2(eta2) = log2(1 + 2^eta2): 32
-// independent ex2/lg2 pairs, then a tree. (Folding the logarithms into one lg2 of the
-// product of the (1 + 2^-|eta2|) factors was measured slower, both as a running product, a
-// 32-long chain, and as a depth-5 product tree: the epilogue is bound by instruction issue,
-// not by the SFU.)
-__device__ __forceinline__ float sum_sp2_32(const uint32_t (&r)[32], int valid)
-{
-    float t[32];
-    if (valid >= 32) {
-#pragma unroll
-        for (int k = 0; k < 32; ++k) t[k] = softplus2(__uint_as_float(r[k]));
-    } else {
-#pragma unroll
-        for (int k = 0; k < 32; ++k) t[k] = (k < valid) ? softplus2(__uint_as_float(r[k])) : 0.0f;
-    }
-#pragma unroll
-    for (int w = 16; w > 0; w >>= 1)
-#pragma unroll
-        for (int k = 0; k < w; ++k) t[k] += t[k + w];
-    return t[0];
-}
-
 __device__ __forceinline__ float rcp_approx(float x)
 {
     float y;
@@ -409,7 +387,7 @@ __device__ __forceinline__ void loglik_tc_body(const Src& src, uint32_t* __restr
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
     const uint32_t sbase = smem_u32(smem);
     const uint32_t stage0 = sbase + C::A_RES;  // first pipeline stage
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;  // warp-uniform
     const uint32_t bar0 = sbase + C::BAR_OFF;
     const uint32_t drain_bar = bar0 + 8 * (2 * STAGES + 4);
     const uint32_t aempty_bar = bar0 + 8 * (2 * STAGES + 5);
@@ -540,25 +518,39 @@ __device__ __forceinline__ void loglik_tc_body(const Src& src, uint32_t* __restr
         }
     } else if (warp == 1) {
         // ------------------------------------------------------------- MMA issuer
-        if (lane == 0) {
+        // The whole warp walks the loop and lane 0 alone issues: the loop, its waits and the
+        // descriptors are uniform over the warp, so the descriptors stay in uniform registers
+        // and only their low words change. In an `if (lane == 0)` the operands of every MMA were
+        // moved there one by one, and the issue (150 to 190 cycles per 128 x 256 x 16 MMA), not the
+        // tensor core (129), set the pace. RW sweep, a step of 10 moves: n = 5000, p = 500,
+        // N = 16384 1.77 -> 1.52 ms; n = 2000, p = 200, N = 8192 369 -> 347 us.
+        {
+            const uint32_t issue = lane == 0 ? 1u : 0u;
             constexpr uint32_t IDESC = idesc_bf16_f32(BM, BN);
-            uint32_t it = 0;
+            const uint32_t hi128 = sdesc_hi(128u);
+            uint32_t s = 0, ph = 0;  // stage and parity of the next k-block
             int lt = 0;
             bool ok = true;
             int64_t cur_key = -1;
             uint32_t a_par = 0;  // bit kb: the parity of AFULL(kb)'s phase to wait for next
-            int ta_epoch = 0;    // AR = 2: epochs whose A this thread has waited for
+            int ta_epoch = 0;    // AR = 2: epochs whose A this warp has waited for
+            auto wait = [&](uint32_t bar, uint32_t parity) {
+                const bool w = mbar_wait_bounded(bar, parity, err, wait_ns);
+                return __all_sync(0xffffffffu, w) != 0;
+            };
             // Injected stall (tests of the timeout path): wait first on the drain barrier,
-            // which nothing arrives at before this thread's own final commit, so the wait
+            // which nothing arrives at before this warp's own final commit, so the wait
             // runs out after wait_ns; no MMA has been issued, and the other roles give up and
             // drain as after any timeout.
-            if (stall && !mbar_wait_bounded(drain_bar, 0u, err, wait_ns)) ok = false;
+            if (stall && !wait(drain_bar, 0u)) ok = false;
             for (int64_t u = u_begin; u < u_end && ok; ++u, ++lt) {
                 const TcUnit t = src.unit(u);
                 const int kb_last = t.kblocks - 1;
+                // the last k-block's rows, and A_lo's offset in it (16-byte units)
                 const uint32_t tail_row = t.tw ? (uint32_t)(t.tw * 2) : 128u;
+                const uint32_t hi_tail = sdesc_hi(tail_row);
                 const uint32_t b = (uint32_t)(lt % C::NACC), aph = (uint32_t)((lt / C::NACC) & 1);
-                if (!mbar_wait_bounded(ACCE_BAR(b), aph ^ 1u, err, wait_ns)) {
+                if (!wait(ACCE_BAR(b), aph ^ 1u)) {
                     ok = false;
                     break;
                 }
@@ -568,7 +560,7 @@ __device__ __forceinline__ void loglik_tc_body(const Src& src, uint32_t* __restr
                     cur_key = t.key;
                 }
                 if (AR == 2 && a_first) {
-                    if (!mbar_wait_bounded(AFULL_BAR(0), (uint32_t)(ta_epoch & 1), err, wait_ns)) {
+                    if (!wait(AFULL_BAR(0), (uint32_t)(ta_epoch & 1))) {
                         ok = false;
                         break;
                     }
@@ -577,50 +569,70 @@ __device__ __forceinline__ void loglik_tc_body(const Src& src, uint32_t* __restr
                 tc_fence_after();
                 const uint32_t d = tmem_base + b * (uint32_t)BN;
                 for (int kb = 0; kb < t.kblocks; ++kb) {
-                    const uint32_t s = it % STAGES, ph = (it / STAGES) & 1u;
                     if (AR == 1 && a_first) {
-                        if (!mbar_wait_bounded(AFULL_BAR(kb), (a_par >> kb) & 1u, err, wait_ns)) {
+                        if (!wait(AFULL_BAR(kb), (a_par >> kb) & 1u)) {
                             ok = false;
                             break;
                         }
                         a_par ^= 1u << kb;
                     }
-                    if (!mbar_wait_bounded(FULL_BAR(s), ph, err, wait_ns)) {
+                    if (!wait(FULL_BAR(s), ph)) {
                         ok = false;
                         break;
                     }
                     tc_fence_after();
                     const uint32_t st = stage0 + s * C::STAGE;
-                    const uint32_t rb = (t.tw && kb == kb_last) ? tail_row : 128u;
-                    const uint64_t bg = sdesc_swz(AR ? st : st + 2 * C::A_TILE, rb);
-                    const int nks = (t.ksteps - 4 * kb) < 4 ? (t.ksteps - 4 * kb) : 4;
+                    const bool narrow = t.tw != 0 && kb == kb_last;
+                    const int nks = t.ksteps - 4 * kb;
+                    const uint32_t g_lo = sdesc_lo(AR ? st : st + 2 * C::A_TILE);
                     if (AR == 2) {
                         // A_hi of k-step g in TMEM columns A_COL + 8 g, A_lo 8 ksteps further on
                         const uint32_t ahi = tmem_base + C::A_COL + 32u * (uint32_t)kb;
                         const uint32_t alo = ahi + 8u * (uint32_t)t.ksteps;
-                        for (int ks = 0; ks < nks; ++ks)
-                            umma_bf16_ta(d, ahi + 8u * ks, bg + 2u * ks, IDESC, (kb | ks) != 0 ? 1u : 0u);
-                        for (int ks = 0; ks < nks; ++ks) umma_bf16_ta(d, alo + 8u * ks, bg + 2u * ks, IDESC, 1u);
+                        const uint32_t hi = narrow ? hi_tail : hi128;
+                        const int nk = nks < 4 ? nks : 4;
+                        for (int ks = 0; ks < nk; ++ks)
+                            umma_bf16_ta_if(issue, d, ahi + 8u * ks, sdesc_make(g_lo + 2u * ks, hi), IDESC,
+                                            (kb | ks) != 0 ? 1u : 0u);
+                        for (int ks = 0; ks < nk; ++ks)
+                            umma_bf16_ta_if(issue, d, alo + 8u * ks, sdesc_make(g_lo + 2u * ks, hi), IDESC, 1u);
                     } else {
-                        const uint32_t a = AR ? sbase + (uint32_t)(kb * 2 * C::A_TILE) : st;
-                        const uint32_t lo = (AR && (rb != 128u || kb == 3)) ? (uint32_t)C::TAIL_LO : (uint32_t)C::A_TILE;
-                        const uint64_t ahi = sdesc_swz(a, rb);
-                        const uint64_t alo = sdesc_swz(a + lo, rb);
-                        for (int ks = 0; ks < nks; ++ks)  // +32 bytes per K = 16 step inside the swizzle row
-                            umma_bf16(d, ahi + 2u * ks, bg + 2u * ks, IDESC, (kb | ks) != 0 ? 1u : 0u);
-                        for (int ks = 0; ks < nks; ++ks) umma_bf16(d, alo + 2u * ks, bg + 2u * ks, IDESC, 1u);
+                        const uint32_t lo_off =
+                            (AR && (narrow || kb == 3)) ? (uint32_t)C::TAIL_LO / 16u : (uint32_t)C::A_TILE / 16u;
+                        const uint32_t a_lo = sdesc_lo(AR ? sbase + (uint32_t)(kb * 2 * C::A_TILE) : st);
+                        if (nks >= 4) {  // +32 bytes per K = 16 step inside the swizzle row
+#pragma unroll
+                            for (int ks = 0; ks < 4; ++ks)
+                                umma_bf16_if(issue, d, sdesc_make(a_lo + 2u * ks, hi128), sdesc_make(g_lo + 2u * ks, hi128),
+                                             IDESC, (kb | ks) != 0 ? 1u : 0u);
+#pragma unroll
+                            for (int ks = 0; ks < 4; ++ks)
+                                umma_bf16_if(issue, d, sdesc_make(a_lo + lo_off + 2u * ks, hi128),
+                                             sdesc_make(g_lo + 2u * ks, hi128), IDESC, 1u);
+                        } else {
+                            const uint32_t hi = narrow ? hi_tail : hi128;
+                            for (int ks = 0; ks < nks; ++ks)
+                                umma_bf16_if(issue, d, sdesc_make(a_lo + 2u * ks, hi), sdesc_make(g_lo + 2u * ks, hi), IDESC,
+                                             (kb | ks) != 0 ? 1u : 0u);
+                            for (int ks = 0; ks < nks; ++ks)
+                                umma_bf16_if(issue, d, sdesc_make(a_lo + lo_off + 2u * ks, hi), sdesc_make(g_lo + 2u * ks, hi),
+                                             IDESC, 1u);
+                        }
                     }
-                    umma_commit(EMPTY_BAR(s));
-                    ++it;
+                    umma_commit_if(issue, EMPTY_BAR(s));
+                    if (++s == (uint32_t)STAGES) {
+                        s = 0;
+                        ph ^= 1u;
+                    }
                 }
                 if (!ok) break;
-                umma_commit(ACCF_BAR(b));
+                umma_commit_if(issue, ACCF_BAR(b));
                 // the resident A is free once this unit's MMAs are done, if the next unit
                 // belongs to another particle tile
-                if (AR && u + 1 < u_end && src.key(u + 1) != t.key) umma_commit(aempty_bar);
+                if (AR && u + 1 < u_end && src.key(u + 1) != t.key) umma_commit_if(issue, aempty_bar);
             }
-            // Wait for every MMA this thread issued before TMEM can be released.
-            umma_commit(drain_bar);
+            // Wait for every MMA this warp issued before TMEM can be released.
+            umma_commit_if(issue, drain_bar);
             mbar_drain(drain_bar, 0u, err);
         }
     } else {
@@ -788,7 +800,7 @@ __global__ void __launch_bounds__(ADJ_THREADS, 1)
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
     const uint32_t sbase = smem_u32(smem);
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;  // warp-uniform
     const uint32_t bar0 = sbase + C::BAR_OFF;
     const uint32_t drain_bar = bar0 + 8u * (uint32_t)(2 * STAGES + 4);
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + C::SLOT_OFF);
@@ -871,46 +883,52 @@ __global__ void __launch_bounds__(ADJ_THREADS, 1)
             }
         }
     } else if (warp == 1) {
-        if (lane == 0) {
-            constexpr uint32_t IDESC = idesc_bf16_f32(BM, BN2);
-            uint32_t it = 0;
-            int lt = 0;  // units with a non-empty K range, which use an accumulator buffer
-            bool ok = true;
-            for (int u = blockIdx.x; u < units && ok; u += gridDim.x) {
-                int mt, pt, kb0, kb1, ks;
-                decode(u, mt, pt, kb0, kb1, ks);
-                if (kb1 <= kb0) continue;
-                const uint32_t b = (uint32_t)(lt & 1), aph = (uint32_t)((lt >> 1) & 1);
-                if (!mbar_wait_bounded(ACCE_BAR(b), aph ^ 1u, err, wait_ns)) {
+        // the whole warp in step, lane 0 issues (as in the likelihood kernel)
+        const uint32_t issue = lane == 0 ? 1u : 0u;
+        constexpr uint32_t IDESC = idesc_bf16_f32(BM, BN2);
+        const uint32_t hi128 = sdesc_hi(128u);
+        uint32_t s = 0, ph = 0;
+        int lt = 0;  // units with a non-empty K range, which use an accumulator buffer
+        bool ok = true;
+        for (int u = blockIdx.x; u < units && ok; u += gridDim.x) {
+            int mt, pt, kb0, kb1, ks;
+            decode(u, mt, pt, kb0, kb1, ks);
+            if (kb1 <= kb0) continue;
+            const uint32_t b = (uint32_t)(lt & 1), aph = (uint32_t)((lt >> 1) & 1);
+            if (!__all_sync(0xffffffffu, mbar_wait_bounded(ACCE_BAR(b), aph ^ 1u, err, wait_ns))) {
+                ok = false;
+                break;
+            }
+            tc_fence_after();
+            const uint32_t d = tmem_base + b * C::ACC_STRIDE;
+            for (int kb = kb0; kb < kb1; ++kb) {
+                if (!__all_sync(0xffffffffu, mbar_wait_bounded(FULL_BAR(s), ph, err, wait_ns))) {
                     ok = false;
                     break;
                 }
                 tc_fence_after();
-                const uint32_t d = tmem_base + b * C::ACC_STRIDE;
-                for (int kb = kb0; kb < kb1; ++kb) {
-                    const uint32_t q = it % STAGES, ph = (it / STAGES) & 1u;
-                    if (!mbar_wait_bounded(FULL_BAR(q), ph, err, wait_ns)) {
-                        ok = false;
-                        break;
-                    }
-                    tc_fence_after();
-                    const uint32_t st = sbase + q * C::STAGE;
-                    const uint64_t ahi = sdesc_sw128(st), alo = sdesc_sw128(st + C::A_TILE);
-                    const uint64_t bg = sdesc_sw128(st + 2 * C::A_TILE);
+                const uint32_t a_lo = sdesc_lo(sbase + s * C::STAGE);
+                const uint32_t g_lo = a_lo + 2u * (uint32_t)C::A_TILE / 16u;
 #pragma unroll
-                    for (int k = 0; k < 4; ++k) umma_bf16(d, ahi + 2u * k, bg + 2u * k, IDESC, (kb > kb0 || k) ? 1u : 0u);
+                for (int k = 0; k < 4; ++k)
+                    umma_bf16_if(issue, d, sdesc_make(a_lo + 2u * k, hi128), sdesc_make(g_lo + 2u * k, hi128), IDESC,
+                                 (kb > kb0 || k) ? 1u : 0u);
 #pragma unroll
-                    for (int k = 0; k < 4; ++k) umma_bf16(d, alo + 2u * k, bg + 2u * k, IDESC, 1u);
-                    umma_commit(EMPTY_BAR(q));
-                    ++it;
+                for (int k = 0; k < 4; ++k)
+                    umma_bf16_if(issue, d, sdesc_make(a_lo + (uint32_t)C::A_TILE / 16u + 2u * k, hi128),
+                                 sdesc_make(g_lo + 2u * k, hi128), IDESC, 1u);
+                umma_commit_if(issue, EMPTY_BAR(s));
+                if (++s == (uint32_t)STAGES) {
+                    s = 0;
+                    ph ^= 1u;
                 }
-                if (!ok) break;
-                umma_commit(ACCF_BAR(b));
-                ++lt;
             }
-            umma_commit(drain_bar);
-            mbar_drain(drain_bar, 0u, err);
+            if (!ok) break;
+            umma_commit_if(issue, ACCF_BAR(b));
+            ++lt;
         }
+        umma_commit_if(issue, drain_bar);
+        mbar_drain(drain_bar, 0u, err);
     } else {
         const int quad = warp & 3;
         const int row = quad * 32 + lane;

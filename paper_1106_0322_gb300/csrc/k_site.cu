@@ -23,12 +23,6 @@ namespace {
 
 constexpr int SITE_CHUNK = 64;
 
-__device__ __forceinline__ float site_prior_term(float b, float inv_ac, int de)
-{
-    const float x = fabsf(b);
-    return de ? x : log1pf(x * inv_ac);
-}
-
 // ------------------------------------------------------------ eta2 in registers
 // Lane l's KC values eta2[l + 32 k] sit in registers as pairs (k even, odd), and X^T in the
 // order the lane reads it, four of its individuals per 16-byte load (k_store_xsite). Padding
@@ -132,7 +126,7 @@ __global__ void __launch_bounds__(32 * SITE_WARPS, site_min_blocks(KC))
                 const float lu_l = logf(u01_open_f(u.z));
                 const float b0 = in ? bg[jl] : 0.0f, v_l = in ? a.vy[jl] : 0.0f;
                 const float b1 = __fadd_rn(b0, delta_l);
-                const float dq_l = site_prior_term(b1, inv_ac, pr.de) - site_prior_term(b0, inv_ac, pr.de);
+                const float dq_l = prior_term(b1, inv_ac, pr.de) - prior_term(b0, inv_ac, pr.de);
                 const int nj = min(32, p - j0);
                 uint32_t accm = 0u;
                 const float4* xr = X + (size_t)j0 * K4 * 32;
@@ -199,7 +193,7 @@ __global__ void __launch_bounds__(32 * SITE_WARPS, site_min_blocks(KC))
             for (int j = lane; j < p; j += 32) {
                 const float b = bg[j];
                 yd = fmaf(b, a.vy[j], yd);
-                lt.add(site_prior_term(b, inv_ac, pr.de));
+                lt.add(prior_term(b, inv_ac, pr.de));
             }
             const float sp2 = warp_sum(mx + lq);
             yd = warp_sum(yd);
@@ -296,7 +290,7 @@ __global__ void k_move_site(SiteArgs a, int64_t N, int p, int n, PriorArgs pr, c
                 const float lq1 = site_trial(eta, xr, n, lane, delta, dm);
                 const float dsp = warp_sum(dm + (lq1 - lq));
                 const float b0 = brow[j], b1 = b0 + delta;
-                const float dlp = coef * (site_prior_term(b1, inv_ac, pr.de) - site_prior_term(b0, inv_ac, pr.de));
+                const float dlp = coef * (prior_term(b1, inv_ac, pr.de) - prior_term(b0, inv_ac, pr.de));
                 const float dl = fmaf(delta, a.vy[j], -0.69314718f * dsp);
                 int acc = logf(u01_open_f(u.z)) < dl + dlp;
                 acc = __shfl_sync(0xffffffffu, acc, 0);
@@ -320,7 +314,7 @@ __global__ void k_move_site(SiteArgs a, int64_t N, int p, int n, PriorArgs pr, c
             for (int r = lane; r < n; r += 32) mx += fmaxf(eta[r], 0.0f);
             for (int j = lane; j < p; j += 32) {
                 yd = fmaf(brow[j], a.vy[j], yd);
-                lt.add(site_prior_term(brow[j], inv_ac, pr.de));
+                lt.add(prior_term(brow[j], inv_ac, pr.de));
             }
             const float sp2 = warp_sum(mx + lq);
             yd = warp_sum(yd);

@@ -30,33 +30,8 @@ __device__ __forceinline__ int64_t warp_global_id()
     return ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
 }
 
-// One coordinate's term of the log prior (the -log(2c) constant dropped): Gt sums
-// log1p(|b|/(a c)) and multiplies by -(a+1); the double exponential sums |b| and
-// multiplies by -1/c.
-__device__ __forceinline__ float prior_term(float b, float inv_ac, int de)
-{
-    const float x = fabsf(b);
-    return de ? x : log1pf(x * inv_ac);
-}
+// The log prior's coefficient of its term sum (prior_term, spa_device.cuh), FP64.
 __device__ __forceinline__ double prior_coef(PriorArgs pr, double c) { return pr.de ? -1.0 / c : -((double)pr.a + 1.0); }
-
-// The Gt terms of four coordinates at once: log1p(x0) + ... + log1p(x3) with x = |b|/(a c),
-// as the logarithm of the product of the factors 1 + x_k (one logarithm instead of four).
-// Each factor and product carries a relative rounding of 2^-24, so the sum is accurate to
-// a few 1e-7 in absolute terms, about the same as four rounded log1p terms of moderate size.
-// Products beyond FP32 range (factors near 1e9) take the four logarithms instead. Every
-// kernel that forms a state's log-prior sum for the MH test (the moves, and the reweighting's
-// sum at the new scale) uses this grouping when p % 4 == 0, so that the test compares one
-// function of the state.
-__device__ __forceinline__ float prior_terms4(float4 b, float inv_ac)
-{
-    const float f0 = fmaf(fabsf(b.x), inv_ac, 1.0f), f1 = fmaf(fabsf(b.y), inv_ac, 1.0f);
-    const float f2 = fmaf(fabsf(b.z), inv_ac, 1.0f), f3 = fmaf(fabsf(b.w), inv_ac, 1.0f);
-    const float q = (f0 * f1) * (f2 * f3);
-    if (q <= FLT_MAX) return logf(q);
-    return log1pf(fabsf(b.x) * inv_ac) + log1pf(fabsf(b.y) * inv_ac) + log1pf(fabsf(b.z) * inv_ac) +
-           log1pf(fabsf(b.w) * inv_ac);
-}
 
 // The prior's gradient in MALA's drift. The drift can be any fixed function of the state:
 // the MH test evaluates the forward and reverse proposal densities with this same function,
@@ -114,12 +89,6 @@ __device__ __forceinline__ void pack_offset(__nv_bfloat16* __restrict__ Arow, in
     Arow[p] = hi;
     Arow[Kp + p] = lo;
 }
-
-__device__ __forceinline__ float4 ld4(const float* p) { return *reinterpret_cast<const float4*>(p); }
-// read-only path: per-coordinate constants no thread writes while the kernel runs
-__device__ __forceinline__ float4 ldg4(const float* p) { return __ldg(reinterpret_cast<const float4*>(p)); }
-__device__ __forceinline__ void st4(float* p, float4 v) { *reinterpret_cast<float4*>(p) = v; }
-__device__ __forceinline__ float comp(const float4& v, int k) { return k == 0 ? v.x : (k == 1 ? v.y : (k == 2 ? v.z : v.w)); }
 
 // ------------------------------------------------------------ Metropolis-Hastings test
 // The log-likelihood of particle i is sp_scale * (sum of the GEMM partials + ydq[i]), kept

@@ -17,6 +17,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <cfloat>
+
 namespace spa {
 
 // ------------------------------------------------------------------ error word bits
@@ -179,6 +181,20 @@ __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity)
     return ok != 0;
 }
 
+// Whether that phase has completed, without waiting.
+__device__ __forceinline__ bool mbar_test(uint32_t bar, uint32_t parity)
+{
+    uint32_t ok;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(ok)
+        : "r"(bar), "r"(parity)
+        : "memory");
+    return ok != 0;
+}
+
 // The default limit of a bounded wait (a context can set another, spa_set_wait_limit).
 constexpr uint64_t WAIT_LIMIT_DEFAULT_NS = 4000000000ull;
 // The limit of a drain: the wait for a CTA's own copies and MMAs in flight before it frees
@@ -272,34 +288,19 @@ __device__ __forceinline__ void tmem_dealloc(uint32_t taddr, uint32_t ncols)
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 
-// Shared-memory matrix descriptor (sm_100 format) for a K-major operand tile stored
-// with the 128-byte swizzle: rows of 64 BF16 (128 B), 8-row atoms of 1024 B.
+// Shared-memory matrix descriptor (sm_100 format) of a K-major BF16 operand tile whose rows are
+// one swizzle span of row_bytes: 128 (64 columns, 128-byte swizzle), 64 (64-byte) or 32 (32-byte):
 //   [0,14) start address >> 4, [16,30) leading byte offset >> 4 (unused here),
-//   [32,46) stride byte offset >> 4 (1024 B between 8-row groups), [46,48) = 1,
-//   [61,64) layout = 2 (128-byte swizzle). The tile base must be 1024-byte aligned.
-__device__ __forceinline__ uint64_t sdesc_sw128(uint32_t smem_addr)
+//   [32,46) stride byte offset >> 4 (8 rows), [46,48) = 1, [61,64) layout = 2, 4 or 6.
+// The tile base must be 1024-byte aligned. Kept as two words: the low one (start address)
+// advances with the operand (2 per K = 16 step), the high one is fixed by the row size.
+__device__ __forceinline__ uint32_t sdesc_lo(uint32_t smem_addr) { return ((smem_addr & 0x3FFFFu) >> 4) | (1u << 16); }
+__device__ __forceinline__ uint32_t sdesc_hi(uint32_t row_bytes)
 {
-    uint64_t d = 0;
-    d |= (uint64_t)((smem_addr & 0x3FFFFu) >> 4);
-    d |= (uint64_t)1u << 16;
-    d |= (uint64_t)(1024u >> 4) << 32;
-    d |= (uint64_t)1u << 46;
-    d |= (uint64_t)2u << 61;
-    return d;
+    const uint32_t layout = row_bytes == 128u ? 2u : (row_bytes == 64u ? 4u : 6u);
+    return ((8u * row_bytes) >> 4) | (1u << 14) | (layout << 29);
 }
-// The same for a K-major tile with rows of `row_bytes` = 64 (64-byte swizzle, layout 4) or
-// 32 (32-byte swizzle, layout 6): 8-row groups are 8 * row_bytes apart.
-__device__ __forceinline__ uint64_t sdesc_swz(uint32_t smem_addr, uint32_t row_bytes)
-{
-    if (row_bytes == 128u) return sdesc_sw128(smem_addr);
-    uint64_t d = 0;
-    d |= (uint64_t)((smem_addr & 0x3FFFFu) >> 4);
-    d |= (uint64_t)1u << 16;
-    d |= (uint64_t)((8u * row_bytes) >> 4) << 32;
-    d |= (uint64_t)1u << 46;
-    d |= (uint64_t)(row_bytes == 64u ? 4u : 6u) << 61;
-    return d;
-}
+__device__ __forceinline__ uint64_t sdesc_make(uint32_t lo, uint32_t hi) { return ((uint64_t)hi << 32) | lo; }
 
 // Instruction descriptor of kind::f16 with BF16 A and B (both K-major), FP32 accumulate:
 //   [4,6) D format = 1 (F32), [7,10) A = 1 (BF16), [10,13) B = 1 (BF16),
@@ -309,27 +310,35 @@ __host__ __device__ constexpr uint32_t idesc_bf16_f32(uint32_t M, uint32_t N)
     return (1u << 4) | (1u << 7) | (1u << 10) | ((N >> 3) << 17) | ((M >> 4) << 24);
 }
 
-// D[tmem] (+)= A[smem] * B[smem]^T for one K = 16 slice; accumulate != 0 adds to D.
-__device__ __forceinline__ void umma_bf16(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc, uint32_t idesc, uint32_t accumulate)
+// D[tmem] (+)= A[smem] * B[smem]^T for one K = 16 slice; accumulate != 0 adds to D. For a whole
+// warp in step: only the lane with `issue` set issues. With the loop and
+// its operands uniform over the warp the descriptors stay in uniform registers; inside an
+// `if (lane == 0)` each MMA first moves them there one by one, and the issue, not the tensor
+// core, sets the pace.
+__device__ __forceinline__ void umma_bf16_if(uint32_t issue, uint32_t tmem_d, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
+                                             uint32_t accumulate)
 {
     asm volatile(
-        "{\n\t.reg .pred p;\n\t"
+        "{\n\t.reg .pred p, q;\n\t"
         "setp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(tmem_d),
-        "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
+        "setp.ne.b32 q, %5, 0;\n\t"
+        "@q tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(tmem_d),
+        "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate), "r"(issue)
         : "memory");
 }
 
 // D[tmem] (+)= A[tmem] * B[smem]^T for one K = 16 slice, A read from tensor memory: row m of
 // A in lane m, K packed two BF16 per 32-bit column (even k in the low half), 8 columns per slice.
-__device__ __forceinline__ void umma_bf16_ta(uint32_t tmem_d, uint32_t tmem_a, uint64_t bdesc, uint32_t idesc,
-                                             uint32_t accumulate)
+// Issued as umma_bf16_if.
+__device__ __forceinline__ void umma_bf16_ta_if(uint32_t issue, uint32_t tmem_d, uint32_t tmem_a, uint64_t bdesc,
+                                                uint32_t idesc, uint32_t accumulate)
 {
     asm volatile(
-        "{\n\t.reg .pred p;\n\t"
+        "{\n\t.reg .pred p, q;\n\t"
         "setp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}" ::"r"(tmem_d),
-        "r"(tmem_a), "l"(bdesc), "r"(idesc), "r"(accumulate)
+        "setp.ne.b32 q, %5, 0;\n\t"
+        "@q tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}" ::"r"(tmem_d),
+        "r"(tmem_a), "l"(bdesc), "r"(idesc), "r"(accumulate), "r"(issue)
         : "memory");
 }
 
@@ -343,10 +352,16 @@ __device__ __forceinline__ void tmem_st4(uint32_t taddr, uint4 v)
 }
 __device__ __forceinline__ void tmem_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 
-// Arrive once on `bar` when every tcgen05.mma issued so far by this thread has completed.
-__device__ __forceinline__ void umma_commit(uint32_t bar)
+// Arrive once on `bar` when every tcgen05.mma issued so far by the lane with `issue` set has
+// completed (a whole warp in step).
+__device__ __forceinline__ void umma_commit_if(uint32_t issue, uint32_t bar)
 {
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
+    asm volatile(
+        "{\n\t.reg .pred q;\n\t"
+        "setp.ne.b32 q, %1, 0;\n\t"
+        "@q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}" ::"r"(bar),
+        "r"(issue)
+        : "memory");
 }
 
 // Each thread of the warp reads 32 consecutive 32-bit columns of its TMEM lane.
@@ -411,5 +426,62 @@ __device__ __forceinline__ float softplus2(float x)
 {
     return fmaxf(x, 0.0f) + lg2_approx(1.0f + ex2_approx(-fabsf(x)));
 }
+
+// Sum over the first `valid` of 32 columns of softplus2(eta2) = log2(1 + 2^eta2): 32
+// independent ex2/lg2 pairs, then a tree. (Folding the logarithms into one lg2 of the
+// product of the (1 + 2^-|eta2|) factors was measured slower, both as a running product, a
+// 32-long chain, and as a depth-5 product tree: the epilogue is bound by instruction issue,
+// not by the SFU.)
+__device__ __forceinline__ float sum_sp2_32(const uint32_t (&r)[32], int valid)
+{
+    float t[32];
+    if (valid >= 32) {
+#pragma unroll
+        for (int k = 0; k < 32; ++k) t[k] = softplus2(__uint_as_float(r[k]));
+    } else {
+#pragma unroll
+        for (int k = 0; k < 32; ++k) t[k] = (k < valid) ? softplus2(__uint_as_float(r[k])) : 0.0f;
+    }
+#pragma unroll
+    for (int w = 16; w > 0; w >>= 1)
+#pragma unroll
+        for (int k = 0; k < w; ++k) t[k] += t[k + w];
+    return t[0];
+}
+
+// ------------------------------------------------------------------- log prior
+// One coordinate's term of the log prior (the -log(2c) constant dropped): Gt sums
+// log1p(|b|/(a c)) and multiplies by -(a+1); the double exponential sums |b| and
+// multiplies by -1/c.
+__device__ __forceinline__ float prior_term(float b, float inv_ac, int de)
+{
+    const float x = fabsf(b);
+    return de ? x : log1pf(x * inv_ac);
+}
+
+// The Gt terms of four coordinates at once: log1p(x0) + ... + log1p(x3) with x = |b|/(a c),
+// as the logarithm of the product of the factors 1 + x_k (one logarithm instead of four).
+// Each factor and product carries a relative rounding of 2^-24, so the sum is accurate to
+// a few 1e-7 in absolute terms, about the same as four rounded log1p terms of moderate size.
+// Products beyond FP32 range (factors near 1e9) take the four logarithms instead. Every
+// kernel that forms a state's log-prior sum for the MH test (the moves, and the reweighting's
+// sum at the new scale) uses this grouping when p % 4 == 0, so that the test compares one
+// function of the state.
+__device__ __forceinline__ float prior_terms4(float4 b, float inv_ac)
+{
+    const float f0 = fmaf(fabsf(b.x), inv_ac, 1.0f), f1 = fmaf(fabsf(b.y), inv_ac, 1.0f);
+    const float f2 = fmaf(fabsf(b.z), inv_ac, 1.0f), f3 = fmaf(fabsf(b.w), inv_ac, 1.0f);
+    const float q = (f0 * f1) * (f2 * f3);
+    if (q <= FLT_MAX) return logf(q);
+    return log1pf(fabsf(b.x) * inv_ac) + log1pf(fabsf(b.y) * inv_ac) + log1pf(fabsf(b.z) * inv_ac) +
+           log1pf(fabsf(b.w) * inv_ac);
+}
+
+// ----------------------------------------------------------- float4 groups
+__device__ __forceinline__ float4 ld4(const float* p) { return *reinterpret_cast<const float4*>(p); }
+// read-only path: per-coordinate constants no thread writes while the kernel runs
+__device__ __forceinline__ float4 ldg4(const float* p) { return __ldg(reinterpret_cast<const float4*>(p)); }
+__device__ __forceinline__ void st4(float* p, float4 v) { *reinterpret_cast<float4*>(p) = v; }
+__device__ __forceinline__ float comp(const float4& v, int k) { return k == 0 ? v.x : (k == 1 ? v.y : (k == 2 ? v.z : v.w)); }
 
 }  // namespace spa
