@@ -81,13 +81,6 @@ struct TcCfg {
     static_assert(AR != 2 || A_COL + 2 * KB_RES * 32 <= TMEM_COLS, "A_hi | A_lo must fit beside the accumulators");
 };
 
-__device__ __forceinline__ float rcp_approx(float x)
-{
-    float y;
-    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-    return y;
-}
-
 // A 4 x 4 transpose of 16-byte chunks across each aligned group of four lanes: on entry lane
 // 4g + s holds chunks 0..3 of its own row s; on exit slot s of lane 4g + c holds chunk c of
 // row s of the group. Two butterfly exchanges, across lane bit 0 and then bit 1: in each, a
@@ -116,47 +109,13 @@ __device__ __forceinline__ void xpose4_u4(uint4 (&v)[4], int lane)
     }
 }
 
-// Residual mode: besides the softplus sum, r = y - logit^{-1}(eta) for the 32 columns of
-// this chunk is stored as BF16 hi (row of R) and lo (row + n_r) and summed into rsum.
-// eta2 = eta log2(e): with e = 2^-|eta2|, softplus2 = max(eta2, 0) + log2(1 + e) and
-// logit^{-1}(eta) = 1/(1 + e) for eta >= 0, e/(1 + e) otherwise (one ex2 shared).
-// FULL: all 32 columns are individuals (every chunk but the last of a region's row), so no
-// column needs the valid-count test. The hi | lo split is taken two columns at a time (one
-// paired conversion each for hi and lo), with the same round-to-nearest values as one at a time.
-template <bool FULL>
-__device__ __forceinline__ float resid_chunk(const float (&v)[32], int valid, uint32_t ybits,
-                                             __nv_bfloat16* __restrict__ rrow, int64_t n_r, float& rsum)
+// r's 32 hi and 32 lo values of this lane's row (resid_chunk's pairs) into R, 16 bytes a store
+// (rrow is 64-byte aligned), transposed in groups of four lanes first, so that each store
+// instruction writes eight rows' whole 64-byte segments instead of one 16-byte piece of each
+// of 32 rows.
+__device__ __forceinline__ void store_resid(const uint32_t (&hi2)[16], const uint32_t (&lo2)[16],
+                                            __nv_bfloat16* __restrict__ rrow, int64_t n_r)
 {
-    float sp[32];
-    uint32_t hi2[16], lo2[16];  // BF16 pairs, column 2q in the low half
-    float rs[32];
-#pragma unroll
-    for (int k = 0; k < 32; k += 2) {
-        float r2[2];
-#pragma unroll
-        for (int d = 0; d < 2; ++d) {
-            const int kk = k + d;
-            const float x = v[kk];
-            const bool ok = FULL || kk < valid;
-            const float e = ex2_approx(-fabsf(x));
-            const float onepe = 1.0f + e;
-            const float inv = rcp_approx(onepe);
-            const float sig = (x >= 0.0f) ? inv : e * inv;
-            const bool yk = (ybits >> kk) & 1u;
-            sp[kk] = ok ? fmaxf(x, 0.0f) + lg2_approx(onepe) : 0.0f;
-            const float r = ok ? (yk ? 1.0f : 0.0f) - sig : 0.0f;
-            rs[kk] = r;
-            r2[d] = r;
-        }
-        const __nv_bfloat162 h = __floats2bfloat162_rn(r2[0], r2[1]);
-        const float2 hf = __bfloat1622float2(h);
-        const __nv_bfloat162 l = __floats2bfloat162_rn(r2[0] - hf.x, r2[1] - hf.y);
-        hi2[k >> 1] = *reinterpret_cast<const uint32_t*>(&h);
-        lo2[k >> 1] = *reinterpret_cast<const uint32_t*>(&l);
-    }
-    // 16-byte stores of the 32 hi and 32 lo values (rrow is 64-byte aligned), transposed in
-    // groups of four lanes first, so that each store instruction writes eight rows' whole
-    // 64-byte segments instead of one 16-byte piece of each of 32 rows
     uint4 h4[4], l4[4];
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
@@ -173,15 +132,6 @@ __device__ __forceinline__ float resid_chunk(const float (&v)[32], int valid, ui
         *reinterpret_cast<uint4*>(dst) = h4[s];
         *reinterpret_cast<uint4*>(dst + n_r) = l4[s];
     }
-#pragma unroll
-    for (int w = 16; w > 0; w >>= 1)
-#pragma unroll
-        for (int k = 0; k < w; ++k) {
-            sp[k] += sp[k + w];
-            rs[k] += rs[k + w];
-        }
-    rsum = rs[0];
-    return sp[0];
 }
 
 // The units of CTA b of G. Contiguous ranges of the row-major unit order, except with a
@@ -698,15 +648,13 @@ __device__ __forceinline__ void loglik_tc_body(const Src& src, uint32_t* __restr
                     uint32_t r[32];
                     tmem_ld32_async(tbase + (uint32_t)(32 * ch), r);
                     tmem_wait_ld(r);
-                    float v[32];
-#pragma unroll
-                    for (int k = 0; k < 32; ++k) v[k] = __uint_as_float(r[k]);
                     const int64_t i0 = (int64_t)t.nt * BN + col0 + 32 * ch;
                     float rs;
+                    uint32_t hi2[16], lo2[16];
                     const uint32_t yb = __ldg(t.ybits + (i0 >> 5));
-                    __nv_bfloat16* rrow = t.R + prow * 2 * t.n_r + i0;
-                    const float sp = valid >= 32 ? resid_chunk<true>(v, valid, yb, rrow, t.n_r, rs)
-                                                 : resid_chunk<false>(v, valid, yb, rrow, t.n_r, rs);
+                    const float sp = valid >= 32 ? resid_chunk<true>(r, valid, yb, nullptr, hi2, lo2, rs)
+                                                 : resid_chunk<false>(r, valid, yb, nullptr, hi2, lo2, rs);
+                    store_resid(hi2, lo2, t.R + prow * 2 * t.n_r + i0, t.n_r);
                     partial[(gc0 + ch) * t.N_pad + prow] = -sp;
                     t.rsum_part[(gc0 + ch) * t.N_pad + prow] = rs;
                 }

@@ -40,26 +40,6 @@ constexpr int SITE_CHUNK = 64;
 constexpr float SITE_PAD = -1e30f;
 constexpr int SITE_WARPS = 4;  // particles per block
 
-__device__ __forceinline__ uint64_t pack2(float lo, float hi)
-{
-    uint64_t r;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
-    return r;
-}
-__device__ __forceinline__ float2 unpack2(uint64_t v)
-{
-    float2 r;
-    asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
-    return r;
-}
-// Two FP32 fused multiply-adds in one instruction, each rounded as fmaf rounds.
-__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c)
-{
-    uint64_t r;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
-    return r;
-}
-
 // 16-byte loads of the next update's column issued before this update's reduction: 4 where the
 // registers allow (n = 1000: 485 -> 370 us a step), none at the widest (n = 1859: 4.55 ms
 // without, 4.74 ms with).

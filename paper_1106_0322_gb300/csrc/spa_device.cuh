@@ -181,20 +181,6 @@ __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity)
     return ok != 0;
 }
 
-// Whether that phase has completed, without waiting.
-__device__ __forceinline__ bool mbar_test(uint32_t bar, uint32_t parity)
-{
-    uint32_t ok;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-        "selp.u32 %0, 1, 0, p;\n\t}"
-        : "=r"(ok)
-        : "r"(bar), "r"(parity)
-        : "memory");
-    return ok != 0;
-}
-
 // The default limit of a bounded wait (a context can set another, spa_set_wait_limit).
 constexpr uint64_t WAIT_LIMIT_DEFAULT_NS = 4000000000ull;
 // The limit of a drain: the wait for a CTA's own copies and MMAs in flight before it frees
@@ -327,6 +313,46 @@ __device__ __forceinline__ void umma_bf16_if(uint32_t issue, uint32_t tmem_d, ui
         : "memory");
 }
 
+// One lane of a converged warp. In an `if (elect_one())` block the compiler knows that a single
+// lane runs and that the block's operands are uniform: a run of unrolled MMAs there issues every
+// 47 cycles, against 71 to 77 predicated one by one (umma_bf16_if) and 92 to 103 in a loop inside
+// `if (lane == 0)` (128 x 128 x 16, measured with a stand-alone issue loop; the tensor core takes 65).
+__device__ __forceinline__ bool elect_one()
+{
+    uint32_t p;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "elect.sync _|p, 0xffffffff;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(p));
+    return p != 0;
+}
+// D[tmem] (+)= A[smem] * B[smem]^T, or A[tmem], for one K = 16 slice, issued by the calling lane.
+__device__ __forceinline__ void umma_bf16(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc, uint32_t idesc, uint32_t accumulate)
+{
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "setp.ne.b32 p, %4, 0;\n\t"
+        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(tmem_d),
+        "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
+        : "memory");
+}
+__device__ __forceinline__ void umma_bf16_ta(uint32_t tmem_d, uint32_t tmem_a, uint64_t bdesc, uint32_t idesc,
+                                             uint32_t accumulate)
+{
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "setp.ne.b32 p, %4, 0;\n\t"
+        "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}" ::"r"(tmem_d),
+        "r"(tmem_a), "l"(bdesc), "r"(idesc), "r"(accumulate)
+        : "memory");
+}
+// Arrive once on `bar` when every tcgen05.mma issued so far by the calling lane has completed.
+__device__ __forceinline__ void umma_commit(uint32_t bar)
+{
+    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
+}
+
 // D[tmem] (+)= A[tmem] * B[smem]^T for one K = 16 slice, A read from tensor memory: row m of
 // A in lane m, K packed two BF16 per 32-bit column (even k in the low half), 8 columns per slice.
 // Issued as umma_bf16_if.
@@ -427,11 +453,74 @@ __device__ __forceinline__ float softplus2(float x)
     return fmaxf(x, 0.0f) + lg2_approx(1.0f + ex2_approx(-fabsf(x)));
 }
 
+// ------------------------------------------------------- packed FP32 pairs
+// Two FP32 operations in one instruction, each rounded as its scalar form rounds.
+__device__ __forceinline__ uint64_t pack2(float lo, float hi)
+{
+    uint64_t r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+    return r;
+}
+__device__ __forceinline__ float2 unpack2(uint64_t v)
+{
+    float2 r;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
+    return r;
+}
+// Two FP32 fused multiply-adds in one instruction, each rounded as fmaf rounds.
+__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c)
+{
+    uint64_t r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+__device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b)
+{
+    uint64_t r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ uint64_t mul2(uint64_t a, uint64_t b)
+{
+    uint64_t r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+
+// A sum tree over 32 columns as 16 column pairs (2q, 2q + 1): column k is added to k + 16, then
+// k + 8, 4, 2 and 1. Pairs are produced in bit-reversed order, so that each level's two terms
+// follow each other and at most five partial sums are live; all levels but the last are
+// packed additions.
+__host__ __device__ constexpr int tree_pair(int j)
+{
+    return ((j & 1) << 3) | ((j & 2) << 1) | ((j & 4) >> 1) | ((j & 8) >> 3);
+}
+struct PairTree {
+    uint64_t part[5];
+    // the j-th pair produced (j a compile-time constant after unrolling)
+    __device__ __forceinline__ void add(int j, uint64_t v)
+    {
+        int level = 0;
+#pragma unroll
+        for (int m = j; m & 1; m >>= 1) {
+            v = add2(part[level], v);
+            ++level;
+        }
+        part[level] = v;
+    }
+    __device__ __forceinline__ float sum() const
+    {
+        const float2 r = unpack2(part[4]);
+        return r.x + r.y;
+    }
+};
+
 // Sum over the first `valid` of 32 columns of softplus2(eta2) = log2(1 + 2^eta2): 32
-// independent ex2/lg2 pairs, then a tree. (Folding the logarithms into one lg2 of the
-// product of the (1 + 2^-|eta2|) factors was measured slower, both as a running product, a
-// 32-long chain, and as a depth-5 product tree: the epilogue is bound by instruction issue,
-// not by the SFU.)
+// independent ex2/lg2 pairs, then a tree. The SFU bounds it: two operations a column, 16 lanes a
+// cycle and SM, 2.0 us per 128 x 256 tile. (Packed additions in PairTree's order save 1.5
+// instructions a column but were 1.5% slower over a sweep, n = 5000, p = 500: the independent
+// pairs keep the SFU busier. One lg2 of the product of the (1 + 2^-|eta2|) factors was slower too,
+// as a running product and as a product tree.)
 __device__ __forceinline__ float sum_sp2_32(const uint32_t (&r)[32], int valid)
 {
     float t[32];
@@ -447,6 +536,63 @@ __device__ __forceinline__ float sum_sp2_32(const uint32_t (&r)[32], int valid)
 #pragma unroll
         for (int k = 0; k < w; ++k) t[k] += t[k + w];
     return t[0];
+}
+
+__device__ __forceinline__ float rcp_approx(float x)
+{
+    float y;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+
+// The residual pass's work on a chunk of 32 individuals of one particle: the softplus sum
+// (returned), and r = y - logit^{-1}(eta) as BF16 hi and lo pairs (column 2q in the low half of
+// word q) and its sum. eta2 = eta log2(e): with e = 2^-|eta2|, softplus2 = max(eta2, 0) +
+// log2(1 + e) and logit^{-1}(eta) = 1/(1 + e) for eta >= 0, e/(1 + e) otherwise (one ex2 shared).
+// FULL: all 32 columns are individuals (every chunk but the last of a region's row), so no
+// column needs the valid-count test. YV: the phenotypes come as floats (yv, 16-byte aligned, FULL
+// only), else from the bits of ybits.
+template <bool FULL, bool YV = false>
+__device__ __forceinline__ float resid_chunk(const uint32_t (&x2)[32], int valid, uint32_t ybits, const float* yv,
+                                             uint32_t (&hi2)[16], uint32_t (&lo2)[16], float& rsum)
+{
+    const uint64_t one = pack2(1.0f, 1.0f), negone = pack2(-1.0f, -1.0f);
+    PairTree ts, tr;
+#pragma unroll
+    for (int j = 0; j < 16; ++j) {
+        const int q = tree_pair(j), k = 2 * q;
+        const float x0 = __uint_as_float(x2[k]), x1 = __uint_as_float(x2[k + 1]);
+        const float e0 = ex2_approx(-fabsf(x0)), e1 = ex2_approx(-fabsf(x1));
+        const float2 o = unpack2(add2(one, pack2(e0, e1)));
+        // sigma: the numerator is 1 or e, so the product with 1/(1 + e) rounds as the two cases do
+        const uint64_t sig = mul2(pack2(x0 >= 0.0f ? 1.0f : e0, x1 >= 0.0f ? 1.0f : e1), pack2(rcp_approx(o.x), rcp_approx(o.y)));
+        uint64_t y;
+        if (YV) {
+            const float2 yf = __ldg(reinterpret_cast<const float2*>(yv + k));
+            y = pack2(yf.x, yf.y);
+        } else {
+            y = pack2((ybits >> k) & 1u ? 1.0f : 0.0f, (ybits >> (k + 1)) & 1u ? 1.0f : 0.0f);
+        }
+        uint64_t r = fma2(sig, negone, y);
+        uint64_t sp = add2(pack2(fmaxf(x0, 0.0f), fmaxf(x1, 0.0f)), pack2(lg2_approx(o.x), lg2_approx(o.y)));
+        if (!FULL) {
+            const bool in0 = k < valid, in1 = k + 1 < valid;
+            const float2 rf = unpack2(r), sf = unpack2(sp);
+            r = pack2(in0 ? rf.x : 0.0f, in1 ? rf.y : 0.0f);
+            sp = pack2(in0 ? sf.x : 0.0f, in1 ? sf.y : 0.0f);
+        }
+        ts.add(j, sp);
+        tr.add(j, r);
+        const float2 rf = unpack2(r);
+        const __nv_bfloat162 h = __floats2bfloat162_rn(rf.x, rf.y);
+        const float2 hf = __bfloat1622float2(h);
+        const float2 lf = unpack2(fma2(pack2(hf.x, hf.y), negone, r));
+        const __nv_bfloat162 l = __floats2bfloat162_rn(lf.x, lf.y);
+        hi2[q] = *reinterpret_cast<const uint32_t*>(&h);
+        lo2[q] = *reinterpret_cast<const uint32_t*>(&l);
+    }
+    rsum = tr.sum();
+    return ts.sum();
 }
 
 // ------------------------------------------------------------------- log prior

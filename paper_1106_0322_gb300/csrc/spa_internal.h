@@ -377,6 +377,36 @@ bool adj_make_map_GT(CUtensorMap* map, const __nv_bfloat16* GT, int p, int64_t n
 cudaError_t launch_adjoint_tc(const CUtensorMap& mapR, const CUtensorMap& mapGT, const AdjPlan& a, int p, float* gpart,
                               int64_t N_pad, uint32_t* err, cudaStream_t st, uint64_t wait_ns = 0, int max_ctas = 0,
                               bool r_last_use_hint = false);
+// The residual likelihood pass and the adjoint GEMM in one kernel, without R in memory
+// (p <= 255; k_grad_tc.cu): softplus partials, residual sums and gpart, the same bits as
+// launch_loglik_tc's residual mode and launch_adjoint_tc give. max_ctas caps the grid.
+struct GradPlan {
+    int ksteps, kblocks, tw, N2, c_bufs, stages, grid;
+    uint32_t a_bytes, t_bytes, smem;
+};
+struct GradMaps {
+    CUtensorMap B, Bt, T;  // G in 128-row boxes (64 columns; narrow last k-block), G^T in N2-row boxes
+};
+struct GradArgs {
+    const uint32_t* ybits;
+    const float* yv;  // the phenotypes as floats
+    float *partial, *rsum_part, *gpart;
+    int64_t N_pad;
+    int n, p, Kp;
+    uint32_t* err;
+    uint64_t wait_ns;
+    int stall;
+    // from the plans (filled by the launcher)
+    int m_tiles, ksplit, kb_n, ksteps, kblocks, tw, N2, c_bufs, stages;
+    uint32_t a_bytes, t_bytes;
+};
+bool grad_tc_plan(GradPlan& pl, int64_t n, int p, const AdjPlan& adj, int max_ctas);
+bool grad_tc_make_maps(GradMaps& m, const __nv_bfloat16* Gbf, const __nv_bfloat16* GT, int64_t n, int p, int Kp, int64_t n_r,
+                       const GradPlan& pl);
+cudaError_t grad_tc_init_attributes();
+cudaError_t launch_grad_tc(const CUtensorMap& A, const CUtensorMap& At, const GradMaps& m, const GradPlan& pl,
+                           const AdjPlan& adj, GradArgs g, cudaStream_t st);
+
 cudaError_t launch_grad_finish(const float* gpart, int ksplit, const float* rsum_part, int n_parts, int64_t N_pad,
                                int64_t N, int p, const float* mean_f, const float* inv_sd, const float* B, PriorArgs pr,
                                double c, float* grad, cudaStream_t st);

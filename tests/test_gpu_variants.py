@@ -35,3 +35,22 @@ def test_site_register_and_shared_kernels_at_their_edges(spa, n, p, N):
                    cfg=oracle.make_config(move="site", init="mcmc"))
     assert abs(g["accept_rate"][0] - o["accept_rate"][0]) <= 2.0 / (N * p) + 1e-12
     assert np.max(np.abs(g["mean"][0] - o["mean"][0])) <= 2 * 2.0 / N + 1e-4
+
+
+# A MALA sweep evaluates likelihood and gradient in one kernel when p <= 255; a batch's regions
+# run the residual pass and the adjoint as two kernels. Edges: k-blocks (p + 1 mod 64, narrow last
+# ones), marker tiles (16, 128, 208, 255), 32-, 64- and 128-individual tiles, K-splits 1 to 8.
+@pytest.mark.parametrize("n,p,N", [(31, 1, 5), (63, 15, 130), (64, 16, 300), (65, 31, 1100), (127, 32, 700),
+                                   (128, 63, 900), (129, 64, 2600), (191, 95, 3000), (257, 127, 520), (640, 128, 5000),
+                                   (700, 129, 1000), (900, 191, 390), (1000, 207, 2100), (1100, 208, 260),
+                                   (600, 223, 640), (513, 224, 770), (2111, 255, 1500), (96, 40, 20000)])
+def test_gradient_kernel_gives_the_two_kernels_bits(spa, n, p, N):
+    reg = synth.make_region(n, p, 0.9, (0.4, -0.3), seed=1300 + n)
+    sched = synth.geometric_schedule(3, -4.0, -1.0)
+    with spa.Region(reg.G, reg.y, 2.0, config=spa.make_config(move="mala")) as r:
+        one = r.run(sched, N, 2, 5)
+        b = spa.Batch([r], [sched], [N], [2], [5])
+        (two,) = b.run()
+        b.close()
+        for k in one:
+            assert np.array_equal(one[k], two[k]), k
