@@ -12,6 +12,7 @@ hand-written adjoint (``spa_grad_device``).
 from __future__ import annotations
 
 import ctypes as C
+import functools
 import math
 import os
 import threading
@@ -548,6 +549,7 @@ def prior_sample(seed: int, nu: float, c: float, N: int, p: int) -> np.ndarray:
 
 
 # ---------------------------------------------------------- autograd wrapper
+@functools.lru_cache(maxsize=None)
 def _torch_loglik_function():
     import torch
 

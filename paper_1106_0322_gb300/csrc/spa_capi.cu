@@ -199,6 +199,7 @@ struct spa_ctx {
     CUtensorMap mapGT;
     int mapGT_BN = 0;
     uint32_t* d_err = nullptr;
+    uint32_t* h_err = nullptr;  // pinned: where the error word is copied to
     Workspace ws;
     RunBufs rb;
     cudaGraphExec_t gexec = nullptr;
@@ -213,6 +214,7 @@ struct spa_ctx {
     uint64_t wait_ns = 0;      // limit of the tensor-core kernels' bounded waits (0: the default)
     int tile_cfg = -1;         // likelihood tile configuration fixed by spa_set_tile_config (-1: tuned)
     int fault = 0;             // faults injected into the current sweep graph (SPA_FAULT)
+    bool own_busy = true;      // work may still run on own_stream (nothing waited for it yet)
 
     cudaStream_t stream() const { return cfg.stream ? static_cast<cudaStream_t>(cfg.stream) : own_stream; }
 };
@@ -270,13 +272,39 @@ int map_device_error(spa_ctx* c, uint32_t e)
     return fail(c, SPA_ECUDA, "unknown device error");
 }
 
-int read_error_word(spa_ctx* c)
+// Wait for the work on stream st and report (and clear) the device error word.
+int read_error_word(spa_ctx* c, cudaStream_t st)
 {
-    uint32_t e = 0;
-    CK(cudaMemcpyAsync(&e, c->d_err, sizeof(e), cudaMemcpyDeviceToHost, c->stream()), "read error word");
-    CK(cudaStreamSynchronize(c->stream()), "stream synchronize");
-    CK(cudaMemsetAsync(c->d_err, 0, sizeof(uint32_t), c->stream()), "reset error word");
+    // into pinned memory: one copy and one wait (a pageable copy is staged and waited for by itself)
+    CK(cudaMemcpyAsync(c->h_err, c->d_err, sizeof(uint32_t), cudaMemcpyDeviceToHost, st), "read error word");
+    CK(cudaStreamSynchronize(st), "stream synchronize");
+    const uint32_t e = *reinterpret_cast<volatile uint32_t*>(c->h_err);
+    if (e != 0) {
+        CK(cudaMemsetAsync(c->d_err, 0, sizeof(uint32_t), st), "reset error word");
+        CK(cudaStreamSynchronize(st), "stream synchronize");
+    }
+    if (st == c->stream()) c->own_busy = false;
     return map_device_error(c, e);
+}
+int read_error_word(spa_ctx* c) { return read_error_word(c, c->stream()); }
+
+// Before an entry point works on a caller's stream: the context's stream is done with the
+// workspace. Its own stream needs the wait only if something was left running on it.
+int settle_stream(spa_ctx* c, cudaStream_t st)
+{
+    if (st == c->stream() || (!c->cfg.stream && !c->own_busy)) return SPA_OK;
+    CK(cudaStreamSynchronize(c->stream()), "sync context stream");
+    c->own_busy = false;
+    return SPA_OK;
+}
+
+// Whether the likelihood entry points can read the caller's device particles in place: rows
+// read 16 bytes at a time are aligned, and nothing the call writes overlaps them.
+bool particles_in_place(const float* B, int64_t N, int64_t p, const void* out, size_t out_bytes)
+{
+    const uintptr_t b = reinterpret_cast<uintptr_t>(B), o = reinterpret_cast<uintptr_t>(out);
+    if ((p & 3) == 0 && (b & 15u) != 0) return false;
+    return !out || o + out_bytes <= b || b + sizeof(float) * (size_t)(N * p) <= o;
 }
 
 void free_workspace(Workspace& w)
@@ -493,6 +521,7 @@ int ensure_workspace(spa_ctx* c, int64_t N)
 {
     Workspace& w = c->ws;
     if (w.N == N) return SPA_OK;
+    c->own_busy = true;
     drop_graph(c);
     free_workspace(w);
     const int64_t p = c->p;
@@ -547,6 +576,7 @@ int ensure_adjoint_buffers(spa_ctx* c)
 {
     Workspace& w = c->ws;
     if (w.R) return SPA_OK;
+    c->own_busy = true;
     const AdjPlan a = adj_plan((int)c->p, c->n, w.N_pad, c->num_sms);
     const TcPlan plan = tc_plan(c->n, (int)c->p, w.N_pad, c->num_sms);
     cudaError_t e = dalloc(&w.R, (size_t)(w.N_pad * 2 * a.n_r));
@@ -591,6 +621,7 @@ int ensure_site_store(spa_ctx* c)
 {
     const int64_t count = site_xs_floats(c->n, c->p);
     if (count == 0 || c->XS) return SPA_OK;
+    c->own_busy = true;
     cudaError_t e = dalloc(&c->XS, (size_t)count);
     if (e != cudaSuccess) return cuda_fail(c, e, "single-coordinate store");
     CK(launch_store_xsite(c->XT2, c->n, c->p, c->XS, c->stream()), "store X for the single-coordinate kernel");
@@ -1098,6 +1129,7 @@ void destroy(spa_ctx* c)
     dfree(c->G); dfree(c->y); dfree(c->sums); dfree(c->mean); dfree(c->sd); dfree(c->v); dfree(c->unit_c); dfree(c->unit_k);
     dfree(c->l2e_s); dfree(c->mean_f); dfree(c->colf); dfree(c->Xf); dfree(c->Gbf); dfree(c->d_err); dfree(c->GT); dfree(c->yv);
     dfree(c->ybits); dfree(c->XT2); dfree(c->XS); dfree(c->lip);
+    if (c->h_err) cudaFreeHost(c->h_err);
     if (c->ev_fork) cudaEventDestroy(c->ev_fork);
     if (c->ev_keys) cudaEventDestroy(c->ev_keys);
     if (c->ev_join) cudaEventDestroy(c->ev_join);
@@ -1504,6 +1536,7 @@ int spa_create(const int8_t* G, const uint8_t* y, int64_t n, int64_t p, double n
     CA(ybits, c->ywords);
     CA(d_err, 1);
 #undef CA
+    if (e == cudaSuccess) e = cudaHostAlloc(reinterpret_cast<void**>(&c->h_err), sizeof(uint32_t), cudaHostAllocDefault);
     if (e != cudaSuccess) {
         set_thread_error_str(std::string("device allocation: ") + cudaGetErrorString(e));
         destroy(c);
@@ -1616,6 +1649,7 @@ static int run_common(spa_ctx* c, const double* sched, bool sched_on_device, int
         if (rc != SPA_OK) return rc;
     }
     cudaStream_t st = c->stream();
+    c->own_busy = true;
     CK(cudaMemcpyAsync(c->rb.sched, sched, sizeof(double) * (size_t)T,
                        sched_on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, st),
        "copy schedule");
@@ -1810,11 +1844,16 @@ static int loglik_impl(spa_ctx* c, const float* B, bool B_dev, int64_t N, double
     Workspace& w = c->ws;
     const int64_t p = c->p;
     const bool tc = c->cfg.precision == SPA_PREC_SPLIT_BF16;
-    if (st_user) CK(cudaStreamSynchronize(c->stream()), "sync context stream");
-    CK(cudaMemcpyAsync(w.beta, B, sizeof(float) * (size_t)(N * p), B_dev ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice,
-                       st),
-       "copy B");
-    const MoveArgs a = move_args(c, nullptr);
+    rc = settle_stream(c, st);
+    if (rc != SPA_OK) return rc;
+    MoveArgs a = move_args(c, nullptr);
+    if (B_dev && particles_in_place(B, N, p, ll_dev ? ll : nullptr, sizeof(double) * (size_t)N)) {
+        a.beta = const_cast<float*>(B);  // packed with noise = 0: read only
+    } else {
+        CK(cudaMemcpyAsync(w.beta, B, sizeof(float) * (size_t)(N * p),
+                           B_dev ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, st),
+           "copy B");
+    }
     CK(launch_move_rw(a, false, N, (int)p, c->pr, c->unit_k, 0, 0u, 0u, nullptr, 0, c->d_err, st), "pack");
     if (tc) {
         CK(launch_loglik_tc(maps_of(c), plan_of(c), c->n, c->Kp, c->ybits, w.partial, w.N_pad, c->d_err, st, nullptr,
@@ -1825,8 +1864,7 @@ static int loglik_impl(spa_ctx* c, const float* B, bool B_dev, int64_t N, double
     }
     CK(launch_finish_loglik(a.mh, N, nullptr, ll_dev ? ll : w.ll, c->d_err, st), "finish loglik");
     if (!ll_dev) CK(cudaMemcpyAsync(ll, w.ll, sizeof(double) * (size_t)N, cudaMemcpyDeviceToHost, st), "copy ll");
-    if (st != c->stream()) CK(cudaStreamSynchronize(st), "sync");
-    return read_error_word(c);
+    return read_error_word(c, st);
 }
 
 int spa_loglik_repeat(spa_ctx* c, int64_t N, int32_t reps, void* stream)
@@ -1834,6 +1872,7 @@ int spa_loglik_repeat(spa_ctx* c, int64_t N, int32_t reps, void* stream)
     if (!c) return fail(nullptr, SPA_EINVAL, "ctx is NULL");
     if (c->ws.N != N || N < 1 || reps < 0) return fail(c, SPA_EINVAL, "no workspace of N particles");
     cudaStream_t st = stream ? static_cast<cudaStream_t>(stream) : c->stream();
+    c->own_busy = true;
     Workspace& w = c->ws;
     for (int32_t k = 0; k < reps; ++k) {
         if (c->cfg.precision == SPA_PREC_SPLIT_BF16) {
@@ -1856,6 +1895,7 @@ int spa_grad_repeat(spa_ctx* c, int64_t N, int32_t reps, void* stream)
     Enq q;
     q.c = c;
     q.st = stream ? static_cast<cudaStream_t>(stream) : c->stream();
+    c->own_busy = true;
     Workspace& w = c->ws;
     for (int32_t k = 0; k < reps && q.e == cudaSuccess; ++k) enq_grad_tc(q, w.gl_p, w.beta_p, 0.0, w.N);
     if (q.e != cudaSuccess) return cuda_fail(c, q.e, "gradient kernels");
@@ -2014,24 +2054,29 @@ static int grad_impl(spa_ctx* c, const float* B, bool dev, int64_t N, double cs,
             if (e != cudaSuccess) return cuda_fail(c, e, "gradient buffer");
         }
         cudaStream_t st = st_user ? st_user : c->stream();
-        if (st_user) CK(cudaStreamSynchronize(c->stream()), "sync context stream");
-        CK(cudaMemcpyAsync(w.beta, B, sizeof(float) * (size_t)(N * p),
-                           dev ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, st),
-           "copy B");
+        rc = settle_stream(c, st);
+        if (rc != SPA_OK) return rc;
         Enq q;
         q.c = c;
         q.st = st;
-        const MoveArgs a = move_args(c, nullptr);
+        MoveArgs a = move_args(c, nullptr);
+        if (dev && particles_in_place(B, N, p, grad, sizeof(float) * (size_t)(N * p)) &&
+            particles_in_place(B, N, p, ll, sizeof(double) * (size_t)N)) {
+            a.beta = const_cast<float*>(B);  // packed with noise = 0: read only
+        } else {
+            CK(cudaMemcpyAsync(w.beta, B, sizeof(float) * (size_t)(N * p),
+                               dev ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, st),
+               "copy B");
+        }
         q.ck(launch_move_rw(a, false, N, (int)p, c->pr, c->unit_k, 0, 0u, 0u, nullptr, 0, c->d_err, st));
-        enq_grad_tc(q, dev ? grad : w.grad, w.beta, cs, N);
+        enq_grad_tc(q, dev ? grad : w.grad, a.beta, cs, N);
         q.ck(launch_finish_loglik(a.mh, N, nullptr, (dev && ll) ? ll : w.ll, c->d_err, st));
         if (q.e != cudaSuccess) return cuda_fail(c, q.e, "gradient (tensor cores)");
         if (!dev) {
             CK(cudaMemcpyAsync(grad, w.grad, sizeof(float) * (size_t)(N * p), cudaMemcpyDeviceToHost, st), "copy grad");
             if (ll) CK(cudaMemcpyAsync(ll, w.ll, sizeof(double) * (size_t)N, cudaMemcpyDeviceToHost, st), "copy ll");
         }
-        CK(cudaStreamSynchronize(st), "sync");
-        return read_error_word(c);
+        return read_error_word(c, st);
     }
     if (!w.eta) {
         const int64_t tiles = (n + SIMT_TILE_N - 1) / SIMT_TILE_N;
@@ -2040,7 +2085,8 @@ static int grad_impl(spa_ctx* c, const float* B, bool dev, int64_t N, double cs,
         if (e != cudaSuccess) return cuda_fail(c, e, "gradient scratch");
     }
     cudaStream_t st = st_user ? st_user : c->stream();
-    if (st_user) CK(cudaStreamSynchronize(c->stream()), "sync context stream");
+    rc = settle_stream(c, st);
+    if (rc != SPA_OK) return rc;
     CK(cudaMemcpyAsync(w.beta, B, sizeof(float) * (size_t)(N * p), dev ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, st),
        "copy B");
     CK(launch_grad_simt(w.beta, c->Xf, c->y, N, n, (int)p, w.eta, dev ? grad : w.grad, dev ? ll : (ll ? w.ll : nullptr),
@@ -2050,8 +2096,7 @@ static int grad_impl(spa_ctx* c, const float* B, bool dev, int64_t N, double cs,
         CK(cudaMemcpyAsync(grad, w.grad, sizeof(float) * (size_t)(N * p), cudaMemcpyDeviceToHost, st), "copy grad");
         if (ll) CK(cudaMemcpyAsync(ll, w.ll, sizeof(double) * (size_t)N, cudaMemcpyDeviceToHost, st), "copy ll");
     }
-    CK(cudaStreamSynchronize(st), "sync");
-    return read_error_word(c);
+    return read_error_word(c, st);
 }
 
 int spa_grad(spa_ctx* c, const float* B, int64_t N, double cs, double* ll_out, float* grad_out)
