@@ -173,6 +173,24 @@ __device__ __forceinline__ bool mh_decide(const MhState& s, const PartSlices& sh
 }
 
 
+// A step's first move after a resampling: the gather left particle i's row in beta_p (and its
+// gradient in gl_p), so the move reads it there and writes it back as the state, as it does with
+// an accepted proposal; here its MH state and the uniform weights follow. Returns whether the
+// step resampled.
+__device__ __forceinline__ bool take_resampled(const MoveArgs& a, int64_t i, int lane)
+{
+    if (!a.rs.flag || *a.rs.flag == 0) return false;
+    if (lane == 0) {
+        a.mh.llq[i] = a.rs.llq_tmp[i];
+        a.mh.lpq[i] = a.rs.lpq_tmp[i];
+        a.rs.w.logw[i] = a.rs.lw;
+        a.rs.w.W[i] = a.rs.wi;
+        a.rs.w.Wf[i] = (float)a.rs.wi;
+        a.rs.w.wfix[i] = a.rs.wf;
+    }
+    return true;
+}
+
 // ------------------------------------------------------------ RW move kernel
 // One warp per particle. With DECIDE, the warp first runs the MH test of the proposal
 // left by the previous move (its log-likelihood partials are complete, the GEMM having run
@@ -287,10 +305,13 @@ __global__ void __launch_bounds__(BLOCK, 5) k_move_rw(MoveArgs a, int64_t N, int
     const float4 sk = stepk[t];
     const int64_t i = warp_global_id();
     const int lane = threadIdx.x & 31;
-    bool acc = false;
+    bool acc = false;  // the state is the row in beta_p: an accepted proposal, or a resampled particle
     if (i < N) {
         const uint64_t seed = (noise || DECIDE) ? *seedp : 0ull;
-        if (DECIDE) acc = mh_decide(a.mh, parts, i, lane, sk.y, 0.0f, m_prev, err);
+        if (DECIDE)
+            acc = mh_decide(a.mh, parts, i, lane, sk.y, 0.0f, m_prev, err);
+        else
+            acc = take_resampled(a, i, lane);
         const float* src = (acc ? a.beta_p : a.beta) + i * p;
         float* dst = a.beta_p + i * p;
         float* cur = a.beta + i * p;
@@ -391,6 +412,8 @@ __global__ void __launch_bounds__(BLOCK, 4) k_move_mala(MoveArgs a, int64_t N, i
             const float2 fw = a.fwd[i];
             const float extra = -((bwd.s - fw.x) + (bwd.c - fw.y)) / (2.0f * h * h);
             acc = mh_decide(a.mh, parts, i, lane, sk.y, extra, m_prev, err);
+        } else {
+            acc = take_resampled(a, i, lane);
         }
         const float* src = (acc ? a.beta_p : a.beta) + i * p;
         const float* gsrc = (acc ? a.gl_p : a.gl) + i * p;
@@ -486,6 +509,37 @@ __global__ void __launch_bounds__(BLOCK, 4) k_move_mala(MoveArgs a, int64_t N, i
 // proposals (and their gradients) are copied into the state rows, so that between steps
 // beta and gl hold the particles.
 template <bool MALA, bool VEC>
+__device__ __forceinline__ bool commit_test(const MoveArgs& a, const PartSlices& parts, int64_t i, int p, int lane, PriorArgs pr,
+                                            float4 sk, uint32_t m_prev, uint32_t* err)
+{
+    float extra = 0.0f;
+    if (MALA) {
+        const float ac = sk.x, a1 = pr.a + 1.0f, inv_c = sk.z;
+        const float h = *a.h, h2 = 0.5f * h * h;
+        const FSum bwd = warp_sum(mala_reverse<VEC>(a, i, p, lane, h2, a1, ac, inv_c, pr.de));
+        const float2 fw = a.fwd[i];
+        extra = -((bwd.s - fw.x) + (bwd.c - fw.y)) / (2.0f * h * h);
+    }
+    return mh_decide(a.mh, parts, i, lane, sk.y, extra, m_prev, err);
+}
+
+template <bool MALA, bool VEC>
+__device__ __forceinline__ void commit_row(const MoveArgs& a, int64_t i, int p, int lane)
+{
+    const float* src = a.beta_p + i * p;
+    float* dst = a.beta + i * p;
+    if (VEC) {
+        for (int j = 4 * lane; j < p; j += 128) st4(dst + j, ld4(src + j));
+        if (MALA)
+            for (int j = 4 * lane; j < p; j += 128) st4(a.gl + i * p + j, ld4(a.gl_p + i * p + j));
+    } else {
+        for (int j = lane; j < p; j += 32) dst[j] = src[j];
+        if (MALA)
+            for (int j = lane; j < p; j += 32) a.gl[i * p + j] = a.gl_p[i * p + j];
+    }
+}
+
+template <bool MALA, bool VEC>
 __global__ void __launch_bounds__(BLOCK) k_move_commit(MoveArgs a, int64_t N, int p, PriorArgs pr,
                                                       const float4* __restrict__ stepk, int t, uint32_t m_prev,
                                                       const uint64_t* __restrict__ seedp, uint32_t* err)
@@ -500,28 +554,8 @@ __global__ void __launch_bounds__(BLOCK) k_move_commit(MoveArgs a, int64_t N, in
     const int lane = threadIdx.x & 31;
     bool acc = false;
     if (i < N) {
-        float extra = 0.0f;
-        if (MALA) {
-            const float ac = sk.x, a1 = pr.a + 1.0f, inv_c = sk.z;
-            const float h = *a.h, h2 = 0.5f * h * h;
-            const FSum bwd = warp_sum(mala_reverse<VEC>(a, i, p, lane, h2, a1, ac, inv_c, pr.de));
-            const float2 fw = a.fwd[i];
-            extra = -((bwd.s - fw.x) + (bwd.c - fw.y)) / (2.0f * h * h);
-        }
-        acc = mh_decide(a.mh, parts, i, lane, sk.y, extra, m_prev, err);
-        if (acc) {
-            const float* src = a.beta_p + i * p;
-            float* dst = a.beta + i * p;
-            if (VEC) {
-                for (int j = 4 * lane; j < p; j += 128) st4(dst + j, ld4(src + j));
-                if (MALA)
-                    for (int j = 4 * lane; j < p; j += 128) st4(a.gl + i * p + j, ld4(a.gl_p + i * p + j));
-            } else {
-                for (int j = lane; j < p; j += 32) dst[j] = src[j];
-                if (MALA)
-                    for (int j = lane; j < p; j += 32) a.gl[i * p + j] = a.gl_p[i * p + j];
-            }
-        }
+        acc = commit_test<MALA, VEC>(a, parts, i, p, lane, pr, sk, m_prev, err);
+        if (acc) commit_row<MALA, VEC>(a, i, p, lane);
     }
     if (lane == 0) accw[threadIdx.x >> 5] = acc ? 1 : 0;
     count_warps(a.mh.acc_count, accw);
@@ -558,6 +592,37 @@ __global__ void __launch_bounds__(BLOCK) k_finish_loglik(MhState s, int64_t N, d
 constexpr int RW_PER_BLOCK = 8;
 constexpr int RW_THREADS = 32 * RW_PER_BLOCK;
 
+// The row sums of particle i (row b): the incremental weight's and the log-prior's at c_t.
+__device__ __forceinline__ void reweight_row(const float* b, int p, PriorArgs pr, const ReweightK& rk, int lane, FSum& sdiff,
+                                             FSum& snew)
+{
+    const float k1 = rk.k1, kc = rk.kc, kac = rk.kac, inv_ac = rk.inv_ac;
+    const bool grouped = (p & 3) == 0 && !pr.de;  // the moves' four-coordinate prior term
+    for (int j = lane; j < p; j += 32) {
+        const float x = fabsf(b[j]);
+        sdiff.add(pr.de ? x : log1pf(x * k1 / (kc * (kac + x))));
+        if (!grouped) snew.add(prior_term(x, inv_ac, pr.de));
+    }
+    if (grouped)
+        for (int g = lane; 4 * g < p; g += 32) snew.add(prior_terms4(ld4(b + 4 * g), inv_ac));
+}
+
+// The block's particles' log-weights from the row sums (warp 0, one particle per lane, FP64).
+__device__ __forceinline__ void reweight_finish(const float4* sums, int64_t base, int64_t N, PriorArgs pr, const ReweightK& rk,
+                                                double* __restrict__ logw, float2* __restrict__ lpq, uint32_t* err)
+{
+    const int lane = threadIdx.x;
+    if (lane >= RW_PER_BLOCK || base + lane >= N) return;
+    const int64_t i = base + lane;
+    const float4 s = sums[lane];
+    const double sd = (double)s.x + (double)s.y;
+    const double d = pr.de ? rk.lbase - sd * rk.dinv : rk.lbase - ((double)pr.a + 1.0) * sd;
+    const double nl = logw[i] + d;
+    if (!isfinite(nl)) atomicOr(err, DERR_NONFINITE);
+    logw[i] = nl;
+    lpq[i] = make_float2(s.z, s.w);
+}
+
 __global__ void __launch_bounds__(RW_THREADS) k_reweight(const float* __restrict__ beta, double* __restrict__ logw,
                                                    float2* __restrict__ lpq, int64_t N, int p, PriorArgs pr,
                                                    const ReweightK* __restrict__ rkp, int t, uint32_t* __restrict__ err)
@@ -567,141 +632,198 @@ __global__ void __launch_bounds__(RW_THREADS) k_reweight(const float* __restrict
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int64_t base = (int64_t)blockIdx.x * RW_PER_BLOCK;
     const ReweightK rk = rkp[t];
-    const float k1 = rk.k1, kc = rk.kc, kac = rk.kac, inv_ac = rk.inv_ac;
-    {
-        const int q = w;
-        const int64_t i = base + q;
-        FSum sdiff, snew;
-        if (i < N) {
-            const bool grouped = (p & 3) == 0 && !pr.de;  // the moves' four-coordinate prior term
-            for (int j = lane; j < p; j += 32) {
-                const float x = fabsf(beta[i * p + j]);
-                sdiff.add(pr.de ? x : log1pf(x * k1 / (kc * (kac + x))));
-                if (!grouped) snew.add(prior_term(x, inv_ac, pr.de));
-            }
-            if (grouped)
-                for (int g = lane; 4 * g < p; g += 32)
-                    snew.add(prior_terms4(*reinterpret_cast<const float4*>(beta + i * p + 4 * g), inv_ac));
-        }
-        sdiff = warp_sum(sdiff);
-        snew = warp_sum(snew);
-        if (lane == 0) sums[q] = make_float4(sdiff.s, sdiff.c, snew.s, snew.c);
-    }
+    FSum sdiff, snew;
+    if (base + w < N) reweight_row(beta + (base + w) * p, p, pr, rk, lane, sdiff, snew);
+    sdiff = warp_sum(sdiff);
+    snew = warp_sum(snew);
+    if (lane == 0) sums[w] = make_float4(sdiff.s, sdiff.c, snew.s, snew.c);
     __syncthreads();
-    if (w == 0 && lane < RW_PER_BLOCK) {
-        const int64_t i = base + lane;
-        if (i < N) {
-            const float4 s = sums[lane];
-            const double sd = (double)s.x + (double)s.y;
-            const double d = pr.de ? rk.lbase - sd * rk.dinv : rk.lbase - ((double)pr.a + 1.0) * sd;
-            const double nl = logw[i] + d;
-            if (!isfinite(nl)) atomicOr(err, DERR_NONFINITE);
-            logw[i] = nl;
-            lpq[i] = make_float2(s.z, s.w);
-        }
+    reweight_finish(sums, base, N, pr, rk, logw, lpq, err);
+}
+
+// The step's last MH test with its commit (k_move_commit), then the reweighting to the next
+// scale of the row just settled, in one launch: one kernel boundary less a step, and the row is
+// read once.
+template <bool MALA, bool VEC>
+__global__ void __launch_bounds__(BLOCK) k_commit_reweight(MoveArgs a, int64_t N, int p, PriorArgs pr,
+                                                          const float4* __restrict__ stepk, int t, uint32_t m_prev,
+                                                          double* __restrict__ logw, const ReweightK* __restrict__ rkp,
+                                                          uint32_t* err)
+{
+    static_assert(RW_PER_BLOCK == WARPS, "one warp per particle in both halves");
+    __shared__ int accw[BLOCK / 32];
+    __shared__ PartSlices parts;
+    __shared__ float4 sums[RW_PER_BLOCK];
+    grid_dependency_wait();
+    gather_partials(a.mh, N, parts);
+    __syncthreads();
+    const float4 sk = stepk[t];
+    const ReweightK rk = rkp[t + 1];
+    const int64_t i = warp_global_id();
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    bool acc = false;
+    FSum sdiff, snew;
+    if (i < N) {
+        acc = commit_test<MALA, VEC>(a, parts, i, p, lane, pr, sk, m_prev, err);
+        if (acc) commit_row<MALA, VEC>(a, i, p, lane);
+        reweight_row((acc ? a.beta_p : a.beta) + i * p, p, pr, rk, lane, sdiff, snew);
     }
+    sdiff = warp_sum(sdiff);
+    snew = warp_sum(snew);
+    if (lane == 0) {
+        sums[w] = make_float4(sdiff.s, sdiff.c, snew.s, snew.c);
+        accw[w] = acc ? 1 : 0;
+    }
+    count_warps(a.mh.acc_count, accw);  // a block barrier first
+    reweight_finish(sums, (int64_t)blockIdx.x * RW_PER_BLOCK, N, pr, rk, logw, a.mh.lpq, err);
 }
 
 // ---------------------------------------------------------- log-sum-exp and ESS
-__device__ double block_max_f64(double v, double* sh)
+// Order-preserving integer of a double (NaN apart): the maximum runs on the integer units, where an
+// FP64 comparison costs a warp 16 issue cycles.
+__device__ __forceinline__ long long f64_key(double x)
 {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v = fmax(v, __shfl_xor_sync(0xffffffffu, v, o));
-    __syncthreads();
-    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = v;
-    __syncthreads();
-    double r = sh[0];
-    for (int k = 1; k < (int)(blockDim.x >> 5); ++k) r = fmax(r, sh[k]);
-    return r;
+    const long long b = __double_as_longlong(x);
+    return b ^ ((b >> 63) & 0x7fffffffffffffffll);
 }
-__device__ double block_sum_f64(double v, double* sh)
+__device__ __forceinline__ double key_f64(long long k)
+{
+    return __longlong_as_double(k ^ ((k >> 63) & 0x7fffffffffffffffll));
+}
+__device__ __forceinline__ long long warp_max(long long v)
 {
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    __syncthreads();
-    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = v;
-    __syncthreads();
-    double r = sh[0];
-    for (int k = 1; k < (int)(blockDim.x >> 5); ++k) r += sh[k];
-    return r;
+    for (int o = 16; o > 0; o >>= 1) v = max(v, __shfl_xor_sync(0xffffffffu, v, o));
+    return v;
 }
 
-// Each block: (m_b, sum e^{x - m_b}, sum e^{2(x - m_b)}) over its elements. The last block
-// to finish combines the blocks in block order and publishes LSE, ESS, log Z and the flag.
+// Each block: (m_b, sum e^{x - m_b}, sum e^{2(x - m_b)}) over its elements, combined by
+// k_normalise. FP64 latency bounds it: one exp (about 40 dependent operations) and two sums whose
+// trees run side by side.
 constexpr int LSE_THREADS = 128;  // one weight per thread up to 128 x LSE_BLOCKS particles
 
 __global__ void __launch_bounds__(LSE_THREADS) k_lse_partial(const double* __restrict__ logw, int64_t N,
-                                                      double* __restrict__ scratch, unsigned int* __restrict__ counter,
-                                                      int t, int mode, double ess_frac, double* __restrict__ ess_out,
-                                                      double* __restrict__ logz_out, uint8_t* __restrict__ res_out,
-                                                      int* __restrict__ flag, uint32_t* __restrict__ err)
+                                                      double* __restrict__ scratch)
 {
     grid_dependency_wait();
-    __shared__ double sh[BLOCK / 32];
-    __shared__ bool last;
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    double mx = -DBL_MAX;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < N; i += stride) mx = fmax(mx, logw[i]);
-    const double mb = block_max_f64(mx, sh);
+    constexpr int W = LSE_THREADS / 32;
+    __shared__ long long shm[W];
+    __shared__ double sh1[W], sh2[W];
+    const int w = threadIdx.x >> 5;
+    const int64_t stride = (int64_t)gridDim.x * LSE_THREADS, i0 = (int64_t)blockIdx.x * LSE_THREADS + threadIdx.x;
+    const double x0 = i0 < N ? logw[i0] : -DBL_MAX;
+    long long mk = max(f64_key(x0), f64_key(-DBL_MAX));
+    for (int64_t i = i0 + stride; i < N; i += stride) mk = max(mk, f64_key(logw[i]));
+    mk = warp_max(mk);
+    if ((threadIdx.x & 31) == 0) shm[w] = mk;
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < W; ++k) mk = max(mk, shm[k]);
+    const double mb = key_f64(mk);
     double s1 = 0.0, s2 = 0.0;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < N; i += stride) {
-        const double e = exp(logw[i] - mb);
+    for (int64_t i = i0; i < N; i += stride) {
+        const double e = exp((i == i0 ? x0 : logw[i]) - mb);
         s1 += e;
         s2 += e * e;
     }
-    s1 = block_sum_f64(s1, sh);
-    s2 = block_sum_f64(s2, sh);
-    const int B = gridDim.x;
-    if (threadIdx.x == 0) {
-        scratch[blockIdx.x] = mb;
-        scratch[B + blockIdx.x] = s1;
-        scratch[2 * B + blockIdx.x] = s2;
-        __threadfence();
-        last = (atomicAdd(counter, 1u) == (unsigned)(B - 1));
-    }
-    __syncthreads();
-    if (!last || threadIdx.x >= 32) return;
-    __threadfence();
-    // combine the block partials: lane l takes blocks l, l+32, ... (fixed order), then a
-    // fixed-order warp tree
-    const int lane = threadIdx.x;
-    double m = -DBL_MAX;
-    for (int b = lane; b < B; b += 32) m = fmax(m, scratch[b]);
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
-    double S1 = 0.0, S2 = 0.0;
-    for (int b = lane; b < B; b += 32) {
-        const double f = (scratch[B + b] > 0.0) ? exp(scratch[b] - m) : 0.0;
-        S1 += scratch[B + b] * f;
-        S2 += scratch[2 * B + b] * f * f;
-    }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
-        S1 += __shfl_xor_sync(0xffffffffu, S1, o);
-        S2 += __shfl_xor_sync(0xffffffffu, S2, o);
+        const double v1 = __shfl_xor_sync(0xffffffffu, s1, o), v2 = __shfl_xor_sync(0xffffffffu, s2, o);
+        s1 += v1;
+        s2 += v2;
     }
-    if (lane != 0) return;
-    const double lse = m + log(S1);
-    const double ess = (S1 * S1) / S2;
-    scratch[3 * B] = lse;
-    *counter = 0u;
-    if (!isfinite(lse) || !(ess >= 1.0 - 1e-9)) atomicOr(err, !isfinite(lse) ? DERR_NONFINITE : DERR_ESS);
-    const int res = (mode == 2) ? 1 : (ess < ess_frac * (double)N);
-    *flag = res;
-    if (logz_out) logz_out[t] = (mode == 0) ? lse : lse - log((double)N);
-    if (mode != 2) {
-        if (ess_out) ess_out[t] = ess;
-        if (res_out) res_out[t] = (uint8_t)res;
+    if ((threadIdx.x & 31) == 0) {
+        sh1[w] = s1;
+        sh2[w] = s2;
     }
+    __syncthreads();
+    if (threadIdx.x != 0) return;
+    s1 = sh1[0];
+    s2 = sh2[0];
+#pragma unroll
+    for (int k = 1; k < W; ++k) {
+        s1 += sh1[k];
+        s2 += sh2[k];
+    }
+    const int B = gridDim.x;
+    scratch[blockIdx.x] = mb;
+    scratch[B + blockIdx.x] = s1;
+    scratch[2 * B + blockIdx.x] = s2;
+}
+
+// lambda exp(acceptance - 0.574), the acceptance being acc of denom proposals.
+__device__ __forceinline__ double adapted_lambda(double lam, unsigned long long acc, double denom)
+{
+    return denom > 0.0 ? lam * exp((double)acc / denom - 0.574) : lam;
 }
 
 __device__ __forceinline__ uint32_t weight_fix(double W) { return (uint32_t)__double2ull_rn(W * 2147483648.0); }
 
-__global__ void k_normalise(WeightArrays w, int64_t N, const double* __restrict__ lse_ptr)
+// The log-sum-exp of B <= LSE_BLOCKS block partials and the weights normalised by it. Every block
+// combines the partials itself, lane l of warp 0 taking blocks l, l + 32, ... and then a
+// fixed-order warp tree; block 0 publishes ESS, log Z and the resampling flag, from another warp
+// while warp 0 takes the logarithm. A combining last block of the first kernel (a fence, a
+// counter, a second read) and this pass took 12 + 5 us cold at N = 4096 as at N = 8192.
+// With lam (MALA), block 0 also adapts the step size to the last block of moves' acceptance.
+constexpr int NORM_THREADS = 64;
+
+__global__ void __launch_bounds__(NORM_THREADS) k_normalise(WeightArrays w, int64_t N, const double* __restrict__ scratch, int B,
+                                                            LseOut o, double* __restrict__ lam,
+                                                            const unsigned long long* __restrict__ acc, double denom)
 {
     grid_dependency_wait();
-    const double lse = *lse_ptr;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < N; i += (int64_t)gridDim.x * blockDim.x) {
+    __shared__ double sh_lse;
+    const int lane = threadIdx.x & 31;
+    double m, S1 = 0.0, S2 = 0.0;
+    {
+        constexpr int K = LSE_BLOCKS / 32;
+        double x[K], a[K], c[K];
+        long long mk = f64_key(-DBL_MAX);
+#pragma unroll
+        for (int k = 0; k < K; ++k) {
+            const int b = lane + 32 * k;
+            const bool in = b < B;
+            x[k] = in ? scratch[b] : -DBL_MAX;
+            a[k] = in ? scratch[B + b] : 0.0;
+            c[k] = in ? scratch[2 * B + b] : 0.0;
+            mk = max(mk, f64_key(x[k]));
+        }
+        m = key_f64(warp_max(mk));
+#pragma unroll
+        for (int k = 0; k < K; ++k) {
+            if (lane + 32 * k >= B) break;
+            const double f = (a[k] > 0.0) ? exp(x[k] - m) : 0.0;
+            S1 += a[k] * f;
+            S2 += c[k] * f * f;
+        }
+#pragma unroll
+        for (int s = 16; s > 0; s >>= 1) {
+            const double v1 = __shfl_xor_sync(0xffffffffu, S1, s), v2 = __shfl_xor_sync(0xffffffffu, S2, s);
+            S1 += v1;
+            S2 += v2;
+        }
+    }
+    if (threadIdx.x == 0) {
+        const double lse = m + log(S1);
+        sh_lse = lse;
+        if (blockIdx.x == 0) {
+            if (!isfinite(lse)) atomicOr(o.err, DERR_NONFINITE);
+            if (o.logz) o.logz[o.t] = (o.mode == 0) ? lse : lse - log((double)N);
+            if (lam) *lam = adapted_lambda(*lam, *acc, denom);
+        }
+    } else if (threadIdx.x == 32 && blockIdx.x == 0) {
+        const double ess = (S1 * S1) / S2;
+        if (!(ess >= 1.0 - 1e-9)) atomicOr(o.err, isfinite(S1) && S1 > 0.0 ? DERR_ESS : DERR_NONFINITE);
+        const int res = (o.mode == 2) ? 1 : (ess < o.ess_frac * (double)N);
+        *o.flag = res;
+        if (o.mode != 2) {
+            if (o.ess) o.ess[o.t] = ess;
+            if (o.resampled) o.resampled[o.t] = (uint8_t)res;
+        }
+    }
+    __syncthreads();
+    const double lse = sh_lse;
+    for (int64_t i = (int64_t)blockIdx.x * NORM_THREADS + threadIdx.x; i < N; i += (int64_t)gridDim.x * NORM_THREADS) {
         const double l = w.logw[i] - lse;
         const double W = exp(l);
         w.logw[i] = l;
@@ -764,7 +886,18 @@ __global__ void __launch_bounds__(RS_LOCAL_THREADS) k_resample_local(const doubl
             const int cl = (len - c0 < RS_BLOCK) ? (int)(len - c0) : RS_BLOCK;
             double* row = rs_sm + c * RS_PAD;
             double local = 0.0;
-            for (int k = 0; k < cl; ++k) {
+            int k = 0;
+            for (; k + 16 <= cl; k += 16) {  // 16 loads ahead of the chain of additions
+                double v[16];
+#pragma unroll
+                for (int q = 0; q < 16; ++q) v[q] = row[k + q];
+#pragma unroll
+                for (int q = 0; q < 16; ++q) {
+                    local = __dadd_rn(local, v[q]);
+                    row[k + q] = local;
+                }
+            }
+            for (; k < cl; ++k) {
                 local = __dadd_rn(local, row[k]);
                 row[k] = local;
             }
@@ -874,6 +1007,75 @@ __global__ void __launch_bounds__(BLOCK) k_gather(const int32_t* __restrict__ id
     }
 }
 
+// The same from the local sums alone, for N <= RG_MAX_BLOCKS blocks of 256: every block of the
+// gather forms the carries itself (one thread, in block order), and every warp finds its ancestor
+// by a 32-way search, the smallest i with C_i > (k + u)/N as in k_resample_search. Two kernel
+// boundaries less than carries, search and gather apart. The line lies at 16384 particles: at
+// 30000 every block's 118 additions cost more than the boundaries (a sweep 1.60 against 1.50 ms).
+constexpr int RG_MAX_BLOCKS = 64;
+
+template <bool VEC>
+__global__ void __launch_bounds__(BLOCK) k_resample_gather(const double* __restrict__ cum, int t,
+                                                          const uint64_t* __restrict__ seedp, const float* __restrict__ beta,
+                                                          float* __restrict__ beta_tmp, const float2* __restrict__ llq,
+                                                          const float2* __restrict__ lpq, float2* __restrict__ llq_tmp,
+                                                          float2* __restrict__ lpq_tmp, const float* __restrict__ g,
+                                                          float* __restrict__ g_tmp, int64_t N, int p, const int* __restrict__ flag)
+{
+    grid_dependency_wait();
+    if (*flag == 0) return;
+    __shared__ double tot[RG_MAX_BLOCKS], carry[RG_MAX_BLOCKS], us;
+    const int nblk = (int)((N + RS_BLOCK - 1) / RS_BLOCK);
+    if ((int)threadIdx.x < nblk) tot[threadIdx.x] = cum[N + threadIdx.x];
+    if (threadIdx.x == 32) {
+        const uint4 x = philox4x32_10(make_uint4(0u, 0u, (uint32_t)t, TAG_RESAMPLE << 16), seed_key(*seedp));
+        us = u01_d(x.x);
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        double run = 0.0;
+        for (int b = 0; b < nblk; ++b) {
+            carry[b] = run;
+            run = __dadd_rn(run, tot[b]);
+        }
+    }
+    __syncthreads();
+    const int64_t k = warp_global_id();
+    const int lane = threadIdx.x & 31;
+    if (k >= N) return;
+    const long long target = __double_as_longlong(__ddiv_rn(__dadd_rn((double)k, us), (double)N));
+    int lo = 0, hi = (int)N;  // the answer is in [lo, hi), or hi = N if no C_i exceeds the target
+    while (hi - lo > 1) {
+        const int step = (hi - lo + 31) / 32;
+        const int i = min(lo + (lane + 1) * step, hi) - 1;
+        const double c = (i < RS_BLOCK) ? cum[i] : __dadd_rn(carry[i / RS_BLOCK], cum[i]);
+        const unsigned int gt = __ballot_sync(0xffffffffu, __double_as_longlong(c) > target);
+        if (gt == 0u) {  // only in the first round: rounding left C below the target
+            lo = (int)N - 1;
+            break;
+        }
+        const int f = __ffs(gt) - 1;
+        hi = min(lo + (f + 1) * step, hi);
+        lo = min(lo + f * step, hi - 1);
+    }
+    const int64_t a = lo;
+    const float* src = beta + a * p;
+    float* dst = beta_tmp + k * p;
+    if (VEC) {
+        for (int j = 4 * lane; j < p; j += 128) st4(dst + j, ld4(src + j));
+        if (g)
+            for (int j = 4 * lane; j < p; j += 128) st4(g_tmp + k * p + j, ld4(g + a * p + j));
+    } else {
+        for (int j = lane; j < p; j += 32) dst[j] = src[j];
+        if (g)
+            for (int j = lane; j < p; j += 32) g_tmp[k * p + j] = g[a * p + j];
+    }
+    if (lane == 0) {
+        llq_tmp[k] = llq[a];
+        lpq_tmp[k] = lpq[a];
+    }
+}
+
 // The resampled particles back into the state, with uniform weights (log(1/N), 1/N and
 // round(2^31/N), formed on the host).
 template <bool VEC>
@@ -912,10 +1114,14 @@ __global__ void __launch_bounds__(BLOCK) k_copyback(float* __restrict__ beta, co
 // -------------------------------------------------------------- column moments
 constexpr int CS_ROWS = 8;
 
-__global__ void k_colstats_partial(const float* __restrict__ beta, const float* __restrict__ Wf, int64_t N, int p,
-                                   float4* __restrict__ part)
+// With rs_flag set (a step that resampled, its rows still in beta_rs): those rows, weights wi.
+__global__ void k_colstats_partial(const float* __restrict__ beta_state, const float* __restrict__ Wf, int64_t N, int p,
+                                   float4* __restrict__ part, const float* __restrict__ beta_rs,
+                                   const int* __restrict__ rs_flag, float wi)
 {
     grid_dependency_wait();
+    const bool rs = rs_flag && *rs_flag != 0;
+    const float* __restrict__ beta = rs ? beta_rs : beta_state;
     __shared__ float4 sh[CS_ROWS][32];
     const int tx = threadIdx.x, ty = threadIdx.y;
     const int j = blockIdx.x * 32 + tx;
@@ -928,7 +1134,7 @@ __global__ void k_colstats_partial(const float* __restrict__ beta, const float* 
 #pragma unroll
             for (int u = 0; u < 4; ++u) {
                 b[u] = beta[(i + u * step) * p + j];
-                wv[u] = Wf[i + u * step];
+                wv[u] = rs ? wi : Wf[i + u * step];
             }
 #pragma unroll
             for (int u = 0; u < 4; ++u) {
@@ -939,7 +1145,7 @@ __global__ void k_colstats_partial(const float* __restrict__ beta, const float* 
         }
         for (; i < N; i += step) {
             const float b = beta[i * p + j];
-            const float wb = Wf[i] * b;
+            const float wb = (rs ? wi : Wf[i]) * b;
             s1.add(wb);
             s2.add(wb * b);
         }
@@ -960,7 +1166,7 @@ __global__ void k_colstats_partial(const float* __restrict__ beta, const float* 
 
 // One warp per coordinate: lane s takes split s (fixed order), then a warp tree.
 __global__ void k_colstats_finish(const float4* __restrict__ part, int p, int splits, float* __restrict__ scale_out,
-                                  int kind, double lam_const, const double* __restrict__ lam_dev, double sd_floor,
+                                  int kind, double rw_factor, const double* __restrict__ lam_dev, double sd_floor,
                                   const double* __restrict__ sched, int t, float* __restrict__ h_out, double p_pow)
 {
     grid_dependency_wait();
@@ -979,12 +1185,11 @@ __global__ void k_colstats_finish(const float4* __restrict__ part, int p, int sp
         s2 += __shfl_xor_sync(0xffffffffu, s2, o);
     }
     if (lane != 0) return;
-    const double lam = lam_dev ? *lam_dev : lam_const;
-    if (j == 0 && h_out) *h_out = (float)(lam * p_pow);
+    if (j == 0 && h_out) *h_out = (float)(*lam_dev * p_pow);
     const double var = fmax(s2 - s1 * s1, 0.0);
     const double fl = sd_floor * sched[t];
     if (kind == 0) {
-        scale_out[j] = (float)(lam / sqrt((double)p) * fmax(sqrt(var), fl));
+        scale_out[j] = (float)(rw_factor * fmax(sqrt(var), fl));
     } else {
         // MALA's D_j, and beside it sqrt(D_j) and 1/D_j for the proposal and its densities
         const double D = fmax(var, fl * fl);
@@ -1319,7 +1524,7 @@ __global__ void k_accept_rate(const unsigned long long* acc, int T, double denom
 
 __global__ void k_adapt_lambda(double* lam, const unsigned long long* acc, double denom)
 {
-    if (threadIdx.x == 0 && denom > 0.0) *lam *= exp((double)*acc / denom - 0.574);
+    if (threadIdx.x == 0) *lam = adapted_lambda(*lam, *acc, denom);
 }
 
 __global__ void k_set_f64(double* ptr, double v)
@@ -1408,6 +1613,11 @@ static cudaError_t launch_pdl(void (*kern)(KArgs...), dim3 grid, dim3 block, siz
     return cudaLaunchKernelEx(&cfg, kern, args...);
 }
 
+static int64_t lse_blocks(int64_t N)
+{
+    const int64_t blocks = (N + LSE_THREADS - 1) / LSE_THREADS;
+    return blocks < LSE_BLOCKS ? blocks : LSE_BLOCKS;
+}
 static unsigned warps_grid(int64_t N) { return (unsigned)((N + WARPS - 1) / WARPS); }
 static unsigned elem_grid(int64_t total)
 {
@@ -1493,6 +1703,18 @@ cudaError_t launch_finish_loglik(const MhState& s, int64_t N, double* logw, doub
     return cudaGetLastError();
 }
 
+cudaError_t launch_commit_reweight(const MoveArgs& a, bool mala, int64_t N, int p, PriorArgs pr, const float4* stepk, int t,
+                                   uint32_t m_prev, double* logw, const ReweightK* rk, uint32_t* err, cudaStream_t st)
+{
+    const bool vec = (p & 3) == 0;
+    const dim3 grid(warps_grid(N)), block(BLOCK);
+    if (mala)
+        return vec ? launch_pdl(k_commit_reweight<true, true>, grid, block, (size_t)0, st, a, N, p, pr, stepk, t, m_prev, logw, rk, err)
+                   : launch_pdl(k_commit_reweight<true, false>, grid, block, (size_t)0, st, a, N, p, pr, stepk, t, m_prev, logw, rk, err);
+    return vec ? launch_pdl(k_commit_reweight<false, true>, grid, block, (size_t)0, st, a, N, p, pr, stepk, t, m_prev, logw, rk, err)
+               : launch_pdl(k_commit_reweight<false, false>, grid, block, (size_t)0, st, a, N, p, pr, stepk, t, m_prev, logw, rk, err);
+}
+
 cudaError_t launch_reweight(const float* beta, double* logw, float2* lpq, int64_t N, int p, PriorArgs pr,
                             const ReweightK* rk, int t, uint32_t* err, cudaStream_t st)
 {
@@ -1501,27 +1723,19 @@ cudaError_t launch_reweight(const float* beta, double* logw, float2* lpq, int64_
     return cudaGetLastError();
 }
 
-cudaError_t launch_lse_ess(const WeightArrays& w, int64_t N, double* scratch, unsigned int* counter, int t, int mode,
-                           double ess_frac, double* ess_out, double* logz_out, uint8_t* resampled_out, int* flag,
-                           uint32_t* err, cudaStream_t st, bool pdl)
+cudaError_t launch_lse(const double* logw, int64_t N, double* scratch, cudaStream_t st)
 {
-    int64_t blocks = (N + LSE_THREADS - 1) / LSE_THREADS;
-    if (blocks > LSE_BLOCKS) blocks = LSE_BLOCKS;
-    if (pdl) {
-        const cudaError_t e_ = launch_pdl(k_lse_partial, dim3((unsigned)blocks), dim3(LSE_THREADS), (size_t)(0), st,
-                                          w.logw, N, scratch, counter, t, mode, ess_frac, ess_out, logz_out,
-                                          resampled_out, flag, err);
-        if (e_ != cudaSuccess) return e_;
-    } else {  // after a wait on another stream's event
-        k_lse_partial<<<(unsigned)blocks, LSE_THREADS, 0, st>>>(w.logw, N, scratch, counter, t, mode, ess_frac, ess_out,
-                                                               logz_out, resampled_out, flag, err);
-    }
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    // one FP64 exp per weight: blocks of 64 spread them over the SMs' FP64 units
-    const unsigned nb = (unsigned)std::min<int64_t>((N + 63) / 64, 8192);
-    { const cudaError_t e_ = launch_pdl(k_normalise, dim3(nb), dim3(64), (size_t)(0), st, w, N, scratch + 3 * blocks); if (e_ != cudaSuccess) return e_; }
-    return cudaGetLastError();
+    return launch_pdl(k_lse_partial, dim3((unsigned)lse_blocks(N)), dim3(LSE_THREADS), (size_t)0, st, logw, N, scratch);
+}
+
+cudaError_t launch_normalise(const WeightArrays& w, int64_t N, const double* scratch, const LseOut& out, double* lam,
+                             const unsigned long long* acc, double denom, cudaStream_t st)
+{
+    // one FP64 exp per weight: blocks of 64 spread them over the SMs' FP64 units; no more blocks than
+    // fill them, since each combines the partials first
+    const unsigned nb = (unsigned)std::min<int64_t>((N + NORM_THREADS - 1) / NORM_THREADS, 1024);
+    return launch_pdl(k_normalise, dim3(nb), dim3(NORM_THREADS), (size_t)0, st, w, N, scratch, (int)lse_blocks(N), out, lam, acc,
+                      denom);
 }
 
 cudaError_t launch_weight_forms(const double* W, int64_t N, float* Wf, uint32_t* wfix, cudaStream_t st)
@@ -1552,6 +1766,24 @@ cudaError_t launch_resample_index(const double* W, int64_t N, double* cum, int32
     return cudaGetLastError();
 }
 
+bool resample_gather_fits(int64_t N) { return (N + RS_BLOCK - 1) / RS_BLOCK <= RG_MAX_BLOCKS; }
+
+cudaError_t launch_resample_gather(const double* W, int64_t N, double* cum, const int* flag, int t, const uint64_t* seed,
+                                   const float* beta, float* beta_tmp, const float2* llq, const float2* lpq, float2* llq_tmp,
+                                   float2* lpq_tmp, const float* g, float* g_tmp, int p, cudaStream_t st)
+{
+    const int64_t chunks = (N + RS_BLOCK - 1) / RS_BLOCK;
+    const cudaError_t e = launch_pdl(k_resample_local, dim3((unsigned)((chunks + RS_CHUNKS - 1) / RS_CHUNKS)),
+                                     dim3(RS_LOCAL_THREADS), RS_LOCAL_SMEM, st, W, N, cum, flag);
+    if (e != cudaSuccess) return e;
+    const dim3 grid(warps_grid(N)), block(BLOCK);
+    if ((p & 3) == 0)
+        return launch_pdl(k_resample_gather<true>, grid, block, (size_t)0, st, cum, t, seed, beta, beta_tmp, llq, lpq, llq_tmp,
+                          lpq_tmp, g, g_tmp, N, p, flag);
+    return launch_pdl(k_resample_gather<false>, grid, block, (size_t)0, st, cum, t, seed, beta, beta_tmp, llq, lpq, llq_tmp,
+                      lpq_tmp, g, g_tmp, N, p, flag);
+}
+
 cudaError_t launch_gather(const int32_t* idx, const float* beta, float* beta_tmp, const float2* llq, const float2* lpq,
                           float2* llq_tmp, float2* lpq_tmp, const float* g, float* g_tmp, int64_t N, int p,
                           const int* flag, cudaStream_t st)
@@ -1565,14 +1797,20 @@ cudaError_t launch_gather(const int32_t* idx, const float* beta, float* beta_tmp
     return cudaGetLastError();
 }
 
+// uniform weights after resampling: log(1/N), 1/N and round(2^31 / N), formed on the host
+UniformWeights uniform_weights(int64_t N)
+{
+    const double wi = 1.0 / (double)N;
+    return UniformWeights{-std::log((double)N), wi, (uint32_t)std::llrint(wi * 2147483648.0)};
+}
+
 cudaError_t launch_copyback(float* beta, const float* beta_tmp, float2* llq, float2* lpq, const float2* llq_tmp,
                             const float2* lpq_tmp, float* g, const float* g_tmp, const WeightArrays& w, int64_t N, int p,
                             const int* flag, cudaStream_t st)
 {
-    // uniform weights after resampling: log(1/N), 1/N and round(2^31 / N), formed on the host
-    const double wi = 1.0 / (double)N;
-    const uint32_t wf = (uint32_t)std::llrint(wi * 2147483648.0);
-    const double lw = -std::log((double)N);
+    const UniformWeights u = uniform_weights(N);
+    const double wi = u.wi, lw = u.lw;
+    const uint32_t wf = u.wf;
     if ((p & 3) == 0)
         { const cudaError_t e_ = launch_pdl(k_copyback<true>, dim3(warps_grid(N)), dim3(BLOCK), (size_t)(0), st, beta, beta_tmp, llq, lpq, llq_tmp, lpq_tmp, g, g_tmp, w, N, p,
                                                           flag, lw, wi, wf); if (e_ != cudaSuccess) return e_; }
@@ -1584,15 +1822,17 @@ cudaError_t launch_copyback(float* beta, const float* beta_tmp, float2* llq, flo
 
 cudaError_t launch_colstats(const float* beta, const float* Wf, int64_t N, int p, float4* part, float* scale_out,
                             int kind, double lam_const, const double* lam_dev, double sd_floor, const double* sched,
-                            int t, float* h_out, cudaStream_t st)
+                            int t, float* h_out, cudaStream_t st, const float* beta_rs, const int* rs_flag)
 {
+    const float wi = (float)uniform_weights(N).wi;
+    const double rw_factor = lam_const / std::sqrt((double)p);  // the same FP64 quotient on the host
     dim3 block(32, CS_ROWS);
     dim3 grid((unsigned)((p + 31) / 32), COLSTAT_SPLITS);
-    { const cudaError_t e_ = launch_pdl(k_colstats_partial, dim3(grid), dim3(block), (size_t)(0), st, beta, Wf, N, p, part); if (e_ != cudaSuccess) return e_; }
+    { const cudaError_t e_ = launch_pdl(k_colstats_partial, dim3(grid), dim3(block), (size_t)(0), st, beta, Wf, N, p, part, beta_rs, rs_flag, wi); if (e_ != cudaSuccess) return e_; }
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     // one warp (and block) per coordinate: its FP64 sums and square roots on their own SM
-    { const cudaError_t e_ = launch_pdl(k_colstats_finish, dim3((unsigned)p), dim3(32), (size_t)(0), st, part, p, COLSTAT_SPLITS, scale_out, kind, lam_const,
+    { const cudaError_t e_ = launch_pdl(k_colstats_finish, dim3((unsigned)p), dim3(32), (size_t)(0), st, part, p, COLSTAT_SPLITS, scale_out, kind, rw_factor,
                                                                lam_dev, sd_floor, sched, t, h_out,
                                                                std::pow((double)p, -1.0 / 6.0)); if (e_ != cudaSuccess) return e_; }
     return cudaGetLastError();

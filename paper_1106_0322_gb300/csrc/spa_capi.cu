@@ -99,12 +99,11 @@ struct Workspace {
     double *ll = nullptr, *logw = nullptr, *W = nullptr;  // ll: FP64 log-likelihood output of the entry points
     float* Wf = nullptr;
     uint32_t* wfix = nullptr;
-    double *cum = nullptr, *lambda = nullptr, *lse_scratch = nullptr;
+    double *cum = nullptr, *lambda = nullptr, *lse_scratch = nullptr;  // lse_scratch: block partials
     uint32_t* keysT = nullptr;  // [p][N] order-preserving keys of beta for the summaries
     float* lu = nullptr;        // [2][N_pad] log U of the pending proposals' MH tests
     float* WfS = nullptr;       // the weights the summaries of a step read, copied beside the keys
     uint32_t* wfixS = nullptr;
-    unsigned int* lse_counter = nullptr;
     float4* colpart = nullptr;
     float* h = nullptr;  // MALA step h = lambda p^(-1/6)
     float* partial = nullptr;
@@ -312,7 +311,7 @@ void free_workspace(Workspace& w)
     dfree(w.beta); dfree(w.beta_p); dfree(w.scale); dfree(w.A);
     dfree(w.lpt_p); dfree(w.ydq); dfree(w.llq); dfree(w.lpq); dfree(w.llq_tmp); dfree(w.lpq_tmp);
     dfree(w.ll); dfree(w.logw); dfree(w.W); dfree(w.Wf); dfree(w.wfix); dfree(w.cum); dfree(w.keysT); dfree(w.WfS); dfree(w.wfixS); dfree(w.lu); dfree(w.colpart); dfree(w.lambda); dfree(w.h);
-    dfree(w.lse_scratch); dfree(w.lse_counter);
+    dfree(w.lse_scratch);
     dfree(w.partial); dfree(w.idx); dfree(w.flag); dfree(w.eta); dfree(w.grad);
     dfree(w.gl); dfree(w.gl_p); dfree(w.fwd); dfree(w.R); dfree(w.rsum); dfree(w.gpart);
     w.N = w.N_pad = 0;
@@ -547,7 +546,6 @@ int ensure_workspace(spa_ctx* c, int64_t N)
     WA(lambda, 1);
     WA(h, 1);
     WA(lse_scratch, LSE_SCRATCH);
-    WA(lse_counter, 1);
     WA(partial, parts * N_pad);
     WA(idx, N);
     WA(flag, 1);
@@ -560,7 +558,6 @@ int ensure_workspace(spa_ctx* c, int64_t N)
     CK(cudaMemsetAsync(w.A, 0, sizeof(__nv_bfloat16) * (size_t)(N_pad * 2 * c->Kp), c->stream()), "memset A");
     CK(cudaMemsetAsync(w.partial, 0, sizeof(float) * (size_t)(parts * N_pad), c->stream()), "memset partial");
     CK(cudaMemsetAsync(w.flag, 0, sizeof(int), c->stream()), "memset flag");
-    CK(cudaMemsetAsync(w.lse_counter, 0, sizeof(unsigned int), c->stream()), "memset counter");
     if (!tc_make_map_A(&w.mapA, w.A, N_pad, c->Kp) || !tc_make_map_A_tail(&w.mapAt, w.A, N_pad, c->Kp, plan.tw)) {
         free_workspace(w);
         return fail(c, SPA_ECUDA, "cuTensorMapEncodeTiled failed for the particle operand");
@@ -806,27 +803,52 @@ MoveArgs move_args(spa_ctx* c, unsigned long long* acc)
     return a;
 }
 
-void enq_resample(Enq& q, int t)
+// Resample if the step's flag is set. fold: leave the rows in beta_p, for the step's proposal
+// scales and first move to take from there (resampled_state); else copy them back.
+void enq_resample(Enq& q, int t, bool fold)
 {
     spa_ctx* c = q.c;
     Workspace& w = c->ws;
-    q.ck(launch_resample_index(w.W, w.N, w.cum, w.idx, w.flag, t, c->rb.seed, 0.0, q.st));
-    q.launches += 2;  // local sums, carries and search
     const bool mala = c->cfg.move_kind == SPA_MOVE_MALA;
-    q.ck(launch_gather(w.idx, w.beta, w.beta_p, w.llq, w.lpq, w.llq_tmp, w.lpq_tmp, mala ? w.gl : nullptr,
-                       mala ? w.gl_p : nullptr, w.N, (int)c->p, w.flag, q.st));
+    float *g = mala ? w.gl : nullptr, *g_tmp = mala ? w.gl_p : nullptr;
+    if (resample_gather_fits(w.N)) {
+        q.ck(launch_resample_gather(w.W, w.N, w.cum, w.flag, t, c->rb.seed, w.beta, w.beta_p, w.llq, w.lpq, w.llq_tmp,
+                                    w.lpq_tmp, g, g_tmp, (int)c->p, q.st));
+        ++q.launches;  // local sums, gather
+    } else {
+        q.ck(launch_resample_index(w.W, w.N, w.cum, w.idx, w.flag, t, c->rb.seed, 0.0, q.st));
+        q.launches += 2;  // local sums, carries and search
+        q.ck(launch_gather(w.idx, w.beta, w.beta_p, w.llq, w.lpq, w.llq_tmp, w.lpq_tmp, g, g_tmp, w.N, (int)c->p, w.flag,
+                           q.st));
+    }
+    if (fold) return;
     WeightArrays wa{w.logw, w.W, w.Wf, w.wfix};
-    q.ck(launch_copyback(w.beta, w.beta_p, w.llq, w.lpq, w.llq_tmp, w.lpq_tmp, mala ? w.gl : nullptr,
-                         mala ? w.gl_p : nullptr, wa, w.N, (int)c->p, w.flag, q.st));
+    q.ck(launch_copyback(w.beta, w.beta_p, w.llq, w.lpq, w.llq_tmp, w.lpq_tmp, g, g_tmp, wa, w.N, (int)c->p, w.flag, q.st));
 }
 
-void enq_colstats(Enq& q, int t)
+ResampledState resampled_state(spa_ctx* c)
+{
+    Workspace& w = c->ws;
+    const UniformWeights u = uniform_weights(w.N);
+    ResampledState r;
+    r.flag = w.flag;
+    r.llq_tmp = w.llq_tmp;
+    r.lpq_tmp = w.lpq_tmp;
+    r.w = WeightArrays{w.logw, w.W, w.Wf, w.wfix};
+    r.lw = u.lw;
+    r.wi = u.wi;
+    r.wf = u.wf;
+    return r;
+}
+
+void enq_colstats(Enq& q, int t, bool fold)
 {
     spa_ctx* c = q.c;
     Workspace& w = c->ws;
     const int kind = c->cfg.move_kind == SPA_MOVE_MALA ? 1 : 0;
     q.ck(launch_colstats(w.beta, w.Wf, w.N, (int)c->p, w.colpart, w.scale, kind, c->cfg.rw_scale,
-                         kind ? w.lambda : nullptr, c->cfg.sd_floor, c->rb.sched, t, kind ? w.h : nullptr, q.st));
+                         kind ? w.lambda : nullptr, c->cfg.sd_floor, c->rb.sched, t, kind ? w.h : nullptr, q.st,
+                         fold ? w.beta_p : nullptr, fold ? w.flag : nullptr));
     ++q.launches;  // two kernels
 }
 
@@ -914,11 +936,11 @@ public:
                 q.ck(launch_finish_loglik(mh_state(c, nullptr), w.N, w.logw, nullptr, c->d_err, q.st));
                 if (c->fault & FAULT_NAN_WEIGHT) q.ck(launch_set_f64(w.logw, std::nan(""), q.st));
                 const bool rm = cfg.init_mode == SPA_INIT_RESAMPLE_MOVE;
-                q.ck(launch_lse_ess(wa, w.N, w.lse_scratch, w.lse_counter, 0, rm ? 2 : 1, cfg.ess_frac, r.ess, r.logz,
-                                    r.res, w.flag, c->d_err, q.st));
-                ++q.launches;  // log-sum-exp is two kernels
+                q.ck(launch_lse(w.logw, w.N, w.lse_scratch, q.st));
+                const LseOut lo{r.ess, r.logz, r.res, w.flag, c->d_err, 0, rm ? 2 : 1, cfg.ess_frac};
+                q.ck(launch_normalise(wa, w.N, w.lse_scratch, lo, nullptr, nullptr, 0.0, q.st));
                 if (rm) {
-                    enq_resample(q, 0);
+                    enq_resample(q, 0, false);
                     b_ = 0;
                     st_ = BURN_BEGIN;
                 } else {
@@ -936,8 +958,8 @@ public:
                 }
                 unsigned long long* scratch = r.acc + T_;
                 if (q.e == cudaSuccess) q.e = cudaMemsetAsync(scratch, 0, sizeof(unsigned long long), q.st);
-                if (!site_) enq_colstats(q, 0);
-                begin_moves(q, 0, m_base_, scratch, BURN_MOVE, BURN_END);
+                if (!site_) enq_colstats(q, 0, false);
+                begin_moves(q, 0, m_base_, scratch, BURN_MOVE, BURN_END, false);
                 break;
             }
             case BURN_END: {
@@ -957,29 +979,39 @@ public:
                 }
                 const int t = (int)t_;
                 if (t > 0) {
-                    q.ck(launch_reweight(w.beta, w.logw, w.lpq, w.N, p, c->pr, r.rk, t, c->d_err, q.st));
+                    if (!reweighted_) q.ck(launch_reweight(w.beta, w.logw, w.lpq, w.N, p, c->pr, r.rk, t, c->d_err, q.st));
+                    q.ck(launch_lse(w.logw, w.N, w.lse_scratch, q.st));
                     // the previous step's transpose has read beta and the weights (forked runs)
                     if (fork_sum_ && q.e == cudaSuccess) q.e = cudaStreamWaitEvent(q.st, c->ev_keys, 0);
-                    q.ck(launch_lse_ess(wa, w.N, w.lse_scratch, w.lse_counter, t, 0, cfg.ess_frac, r.ess, r.logz, r.res,
-                                        w.flag, c->d_err, q.st));
-                    ++q.launches;
+                    const LseOut lo{r.ess, r.logz, r.res, w.flag, c->d_err, t, 0, cfg.ess_frac};
+                    q.ck(launch_normalise(wa, w.N, w.lse_scratch, lo, mala_ && M_ > 0 ? w.lambda : nullptr, r.acc + t - 1,
+                                          denom_, q.st));
                 }
-                enq_resample(q, t);
-                if (!site_) enq_colstats(q, t);
-                begin_moves(q, t, t == 0 ? m_base_ : 0u, r.acc + t, STEP_MOVE, STEP_END);
+                // a first move follows that can take the resampled rows where the gather leaves them
+                const bool fold = !site_ && M_ > 0;
+                enq_resample(q, t, fold);
+                if (!site_) enq_colstats(q, t, fold);
+                begin_moves(q, t, t == 0 ? m_base_ : 0u, r.acc + t, STEP_MOVE, STEP_END, fold);
                 break;
             }
             case BURN_MOVE:
             case STEP_MOVE: {
                 if (mm_ == M_) {
-                    // the last MH test of the block, with the commit of its accepted rows
+                    // the last MH test of the block, with the commit of its accepted rows; with the
+                    // next step's reweighting unless the best particle of this one is recorded first
                     const MoveArgs a = move_args(c, acc_);
-                    q.ck(launch_move_commit(a, mala_, w.N, p, c->pr, r.stepk, mt_, m0_ + (uint32_t)(M_ - 1), r.seed,
+                    reweighted_ = st_ == STEP_MOVE && t_ + 1 < T_ && !cfg.map_path;
+                    if (reweighted_)
+                        q.ck(launch_commit_reweight(a, mala_, w.N, p, c->pr, r.stepk, mt_, m0_ + (uint32_t)(M_ - 1), w.logw,
+                                                    r.rk, c->d_err, q.st));
+                    else
+                        q.ck(launch_move_commit(a, mala_, w.N, p, c->pr, r.stepk, mt_, m0_ + (uint32_t)(M_ - 1), r.seed,
                                             c->d_err, q.st));
                     st_ = after_moves_;
                     break;
                 }
-                const MoveArgs a = move_args(c, acc_);
+                MoveArgs a = move_args(c, acc_);
+                if (mm_ == 0 && fold_) a.rs = resampled_state(c);
                 const uint32_t m = m0_ + (uint32_t)mm_;
                 if (mala_)
                     q.ck(launch_move_mala(a, mm_ > 0, w.N, p, c->pr, r.stepk, mt_, m, m - 1u, r.seed, c->d_err, q.st));
@@ -1009,8 +1041,7 @@ public:
                 }
                 if (cfg.map_path)
                     q.ck(launch_best_particle(mh_state(c, nullptr), w.beta, w.N, p, c->pr, r.sched, t, r.best, q.st));
-                if (mala_) q.ck(launch_adapt_lambda(w.lambda, r.acc + t, denom_, q.st));
-                ++t_;
+                ++t_;  // (MALA's step size is adapted with the next step's weights)
                 st_ = STEP_BEGIN;
                 break;
             }
@@ -1025,7 +1056,8 @@ private:
 
     // M moves at step t with move indices m0 .. m0+M-1 (all M cycles in one launch for the
     // single-coordinate kernel, which needs no likelihood evaluations), then `after`.
-    void begin_moves(Enq& q, int t, uint32_t m0, unsigned long long* acc, Stage moves, Stage after)
+    // fold: the first one takes the step's resampled rows from where the gather left them.
+    void begin_moves(Enq& q, int t, uint32_t m0, unsigned long long* acc, Stage moves, Stage after, bool fold)
     {
         spa_ctx* c = c_;
         Workspace& w = c->ws;
@@ -1044,6 +1076,7 @@ private:
         m0_ = m0;
         acc_ = acc;
         mm_ = 0;
+        fold_ = fold;
         after_moves_ = after;
         st_ = moves;
     }
@@ -1060,6 +1093,8 @@ private:
     uint32_t m_base_ = 0;
     // the current block of moves
     int mt_ = 0, mm_ = 0;
+    bool fold_ = false;
+    bool reweighted_ = false;  // the next step's reweighting ran with this step's commit
     uint32_t m0_ = 0;
     unsigned long long* acc_ = nullptr;
     Stage after_moves_ = STEP_END;
@@ -2256,19 +2291,19 @@ int spa_lse_ess(const double* logw, int64_t N, double* lse, double* ess)
     float* dWf = s.get<float>(N);
     uint32_t* dFix = s.get<uint32_t>(N);
     double* dS = s.get<double>(LSE_SCRATCH);
-    unsigned int* dC = s.get<unsigned int>(1);
     double* dOut = s.get<double>(2);
     uint8_t* dR = s.get<uint8_t>(1);
     int* dF = s.get<int>(1);
     uint32_t* dE = s.get<uint32_t>(1);
-    if (!dL || !dW || !dWf || !dFix || !dS || !dC || !dOut || !dR || !dF || !dE)
+    if (!dL || !dW || !dWf || !dFix || !dS || !dOut || !dR || !dF || !dE)
         return fail(nullptr, SPA_ENOMEM, "device allocation");
     cudaStream_t st = cudaStreamPerThread;
     const WeightArrays wa{dL, dW, dWf, dFix};
     cudaError_t e = cudaMemcpyAsync(dL, logw, sizeof(double) * (size_t)N, cudaMemcpyHostToDevice, st);
     if (e == cudaSuccess) e = cudaMemsetAsync(dE, 0, sizeof(uint32_t), st);
-    if (e == cudaSuccess) e = cudaMemsetAsync(dC, 0, sizeof(unsigned int), st);
-    if (e == cudaSuccess) e = launch_lse_ess(wa, N, dS, dC, 0, 0, 0.0, dOut + 1, dOut, dR, dF, dE, st);
+    if (e == cudaSuccess) e = launch_lse(dL, N, dS, st);
+    const LseOut lo{dOut + 1, dOut, dR, dF, dE, 0, 0, 0.0};
+    if (e == cudaSuccess) e = launch_normalise(wa, N, dS, lo, nullptr, nullptr, 0.0, st);
     double h[2] = {0.0, 0.0};
     if (e == cudaSuccess) e = cudaMemcpyAsync(h, dOut, sizeof(h), cudaMemcpyDeviceToHost, st);
     int rc = finish_free(e, "lse/ess");

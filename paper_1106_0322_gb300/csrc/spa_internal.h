@@ -87,6 +87,22 @@ struct MhState {
     int64_t ld_lu;
 };
 
+// What a step's resampling leaves for its first move (and the proposal scales before it) when the
+// rows are not copied back first: with *flag set, the resampled rows are in beta_p (gradients in
+// gl_p), their MH state in llq_tmp / lpq_tmp, and the weights become uniform.
+struct UniformWeights {
+    double lw, wi;  // log(1/N), 1/N
+    uint32_t wf;    // round(2^31 / N)
+};
+UniformWeights uniform_weights(int64_t N);
+struct ResampledState {
+    const int* flag = nullptr;  // NULL: the state rows are the particles
+    const float2 *llq_tmp = nullptr, *lpq_tmp = nullptr;
+    WeightArrays w{};
+    double lw = 0.0, wi = 0.0;
+    uint32_t wf = 0;
+};
+
 struct MoveArgs {
     float* beta;                 // particle states
     float* beta_p;               // proposals
@@ -106,6 +122,7 @@ struct MoveArgs {
     const float* gl_p;           // grad l of the proposals
     float2* fwd;                 // forward-move residual sum of the proposals
     const float* h;              // step size
+    ResampledState rs;           // a step's first move only
 };
 
 // The paper's single-coordinate cycle (move kind 2): M cycles over j = 0..p-1 per launch.
@@ -160,19 +177,33 @@ cudaError_t launch_finish_loglik(const MhState& s, int64_t N, double* logw, doub
 cudaError_t launch_adapt_lambda(double* lam, const unsigned long long* acc, double denom, cudaStream_t st);
 cudaError_t launch_set_f64(double* ptr, double v, cudaStream_t st);
 
+// launch_move_commit at step t, then launch_reweight to step t + 1, in one kernel.
+cudaError_t launch_commit_reweight(const MoveArgs& a, bool mala, int64_t N, int p, PriorArgs pr, const float4* stepk, int t,
+                                   uint32_t m_prev, double* logw, const ReweightK* rk, uint32_t* err, cudaStream_t st);
+
 // logw += log p(beta | c_t) - log p(beta | c_{t-1}); the log-prior pair lpq refreshed at c_t.
 cudaError_t launch_reweight(const float* beta, double* logw, float2* lpq, int64_t N, int p, PriorArgs pr,
                             const ReweightK* rk, int t, uint32_t* err, cudaStream_t st);
 
-// Log-sum-exp and ESS of logw (per-CTA partial (max, sum e, sum e^2) combined in block order
-// by the last CTA), then normalisation into W, Wf, wfix.
+// Log-sum-exp of logw: partial (max, sum e, sum e^2) per block into scratch [LSE_SCRATCH], then
+// launch_normalise combines them in block order, publishes LSE, ESS and the resampling flag (LseOut)
+// and forms the weights W, Wf, wfix.
 // mode 0: step t >= 1 (log_z[t] = LSE); 1: prior-IS start (log_z[0] = LSE - log N);
 // 2: resample-move start (log_z[0] = LSE - log N, resampling forced, ESS not recorded).
 constexpr int LSE_BLOCKS = 128;
-constexpr int LSE_SCRATCH = 3 * LSE_BLOCKS + 4;  // doubles
-cudaError_t launch_lse_ess(const WeightArrays& w, int64_t N, double* scratch, unsigned int* counter, int t, int mode,
-                           double ess_frac, double* ess_out, double* logz_out, uint8_t* resampled_out, int* flag,
-                           uint32_t* err, cudaStream_t st, bool pdl = true);
+constexpr int LSE_SCRATCH = 3 * LSE_BLOCKS;  // doubles
+struct LseOut {
+    double *ess, *logz;   // [T] (may be NULL)
+    uint8_t* resampled;   // [T] (may be NULL)
+    int* flag;
+    uint32_t* err;
+    int t, mode;
+    double ess_frac;
+};
+cudaError_t launch_lse(const double* logw, int64_t N, double* scratch, cudaStream_t st);
+// lam != NULL (MALA): lambda *= exp(acceptance - 0.574) as well, acceptance = *acc / denom.
+cudaError_t launch_normalise(const WeightArrays& w, int64_t N, const double* scratch, const LseOut& out, double* lam,
+                             const unsigned long long* acc, double denom, cudaStream_t st);
 // Wf and wfix from a given W (for the summaries entry point).
 cudaError_t launch_weight_forms(const double* W, int64_t N, float* Wf, uint32_t* wfix, cudaStream_t st);
 
@@ -184,6 +215,12 @@ cudaError_t launch_mark_uniform(int64_t N, int t, double* ess_out, uint8_t* resa
 // N + ceil(N/256) + 1 doubles (local sums, carries, u).
 cudaError_t launch_resample_index(const double* W, int64_t N, double* cum, int32_t* idx, const int* flag,
                                   int t, const uint64_t* seed, double u_override, cudaStream_t st);
+// The same, index and gather in two kernels, for N that fits (local sums; then carries, search
+// and gather): same ancestors.
+bool resample_gather_fits(int64_t N);
+cudaError_t launch_resample_gather(const double* W, int64_t N, double* cum, const int* flag, int t, const uint64_t* seed,
+                                   const float* beta, float* beta_tmp, const float2* llq, const float2* lpq, float2* llq_tmp,
+                                   float2* lpq_tmp, const float* g, float* g_tmp, int p, cudaStream_t st);
 cudaError_t launch_gather(const int32_t* idx, const float* beta, float* beta_tmp, const float2* llq, const float2* lpq,
                           float2* llq_tmp, float2* lpq_tmp, const float* g, float* g_tmp, int64_t N, int p,
                           const int* flag, cudaStream_t st);
@@ -195,10 +232,12 @@ cudaError_t launch_copyback(float* beta, const float* beta_tmp, float2* llq, flo
 // sigma_j = lam/sqrt(p) max(sd_j, floor c) into scale_out [p]; kind 1 (MALA):
 // D_j = max(var_j, (floor c)^2), sqrt(D_j) and 1/D_j into scale_out [3p].
 constexpr int COLSTAT_SPLITS = 128;
-// With lam_dev (MALA) it also writes h = lambda p^{-1/6} to h_out.
+// With lam_dev (MALA) it also writes h = lambda p^{-1/6} to h_out. With rs_flag != NULL and *rs_flag
+// set, the particles are beta_rs with uniform weights (ResampledState).
 cudaError_t launch_colstats(const float* beta, const float* Wf, int64_t N, int p, float4* part, float* scale_out,
                             int kind, double lam_const, const double* lam_dev, double sd_floor,
-                            const double* sched, int t, float* h_out, cudaStream_t st);
+                            const double* sched, int t, float* h_out, cudaStream_t st, const float* beta_rs = nullptr,
+                            const int* rs_flag = nullptr);
 
 // Per-scale summaries of Section 5 for step t.
 struct SummaryArgs {
