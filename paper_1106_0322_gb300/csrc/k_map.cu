@@ -10,7 +10,8 @@
 // loss's curvature bound), Nesterov momentum, and the gradient-based restart of
 // O'Donoghue and Candes (2015): momentum is dropped whenever (z - beta') . (beta' - beta) > 0.
 // Each step is two FP32 matrix-vector products with the standardised X, both from X^T
-// log2(e) in [p][n] layout (coalesced columns for X z, coalesced rows for X^T r).
+// log2(e) in [p][n] layout (coalesced columns for X z, coalesced rows for X^T r); for small
+// problems the first takes it from registers.
 //
 // Along a sweep (Section 4.1): at step t the EM starts from the particle with the highest
 // posterior density and from the previous step's MAP, and keeps the mode with the higher
@@ -32,6 +33,7 @@ namespace spa {
 namespace {
 
 constexpr int MAP_THREADS = 512;
+constexpr int MAP_REG_P = 64;  // markers a thread can hold of its individual (load_x)
 constexpr int MAP_MAX_INNER = 4000;  // proximal-gradient steps per EM step
 
 __device__ __forceinline__ float block_sum_f(float v, float* red)
@@ -69,6 +71,12 @@ __device__ __forceinline__ double block_sum_d(double v, double* red)
     return r;
 }
 
+__device__ __forceinline__ float sigmoid_f(float x)
+{
+    const float e = __expf(-fabsf(x));
+    return x >= 0.0f ? 1.0f / (1.0f + e) : e / (1.0f + e);
+}
+
 // eta = X z, one thread per individual: it walks column j of X^T log2(e) (consecutive
 // threads read consecutive individuals, so every load is coalesced; a row of X would put
 // each thread on its own cache line), z from shared memory, scaled back by ln 2
@@ -101,12 +109,6 @@ __device__ void gemv_xt(const MapData& d, const float* r, float* g)
     }
 }
 
-__device__ __forceinline__ float sigmoid_f(float x)
-{
-    const float e = __expf(-fabsf(x));
-    return x >= 0.0f ? 1.0f / (1.0f + e) : e / (1.0f + e);
-}
-
 // log p(b | a, c) of one coordinate, FP64 (the constant -log 2c included)
 __device__ __forceinline__ double logprior1_d(PriorArgs pr, double c, float b)
 {
@@ -125,9 +127,9 @@ struct MapSmem {
 __device__ MapSmem map_smem(float* base, int64_t n, int p)
 {
     MapSmem m;
-    m.beta = base;
-    m.z = m.beta + p;
-    m.prev = m.z + p;
+    m.z = base;  // 16-byte aligned, room for MAP_REG_P
+    m.beta = m.z + (p > MAP_REG_P ? p : MAP_REG_P);
+    m.prev = m.beta + p;
     m.w = m.prev + p;
     m.g = m.w + p;
     m.eta = m.g + p;
@@ -137,14 +139,162 @@ __device__ MapSmem map_smem(float* base, int64_t n, int p)
     return m;
 }
 
+// The weighted-L1 problem at the weights m.w from m.z = m.beta: proximal gradient steps until no
+// coordinate moves by more than tol_in.
+__device__ __forceinline__ void map_inner(const MapData& d, float invL, float tol_in, const MapSmem& m)
+{
+    const int p = d.p;
+    float tk = 1.0f;
+    for (int it = 0; it < MAP_MAX_INNER; ++it) {
+        gemv_x(d, m.z, m.eta);
+        __syncthreads();
+        for (int64_t i = threadIdx.x; i < d.n; i += blockDim.x)
+            m.eta[i] = (d.y[i] ? 1.0f : 0.0f) - sigmoid_f(m.eta[i]);
+        __syncthreads();
+        gemv_xt(d, m.eta, m.g);
+        __syncthreads();
+        float dot = 0.0f, diff = 0.0f;
+        for (int j = threadIdx.x; j < p; j += blockDim.x) {
+            const float u = fmaf(m.g[j], invL, m.z[j]), k = m.w[j] * invL;
+            const float bn = u > k ? u - k : (u < -k ? u + k : 0.0f);
+            dot += (m.z[j] - bn) * (bn - m.beta[j]);
+            diff = fmaxf(diff, fabsf(bn - m.beta[j]));
+            m.g[j] = bn;  // the new point
+        }
+        dot = block_sum_f(dot, m.red);
+        diff = block_max_f(diff, m.red);
+        const bool restart = dot > 0.0f;
+        const float tn = restart ? 1.0f : 0.5f * (1.0f + sqrtf(fmaf(4.0f * tk, tk, 1.0f)));
+        const float mom = restart ? 0.0f : (tk - 1.0f) / tn;
+        for (int j = threadIdx.x; j < p; j += blockDim.x) {
+            const float bn = m.g[j];
+            m.z[j] = fmaf(mom, bn - m.beta[j], bn);
+            m.beta[j] = bn;
+        }
+        tk = tn;
+        __syncthreads();
+        if (diff < tol_in) break;
+    }
+}
+
+// gemv_xt with K >= ceil(p / W) markers a warp at once, so that their chains of additions and their
+// warp sums overlap; each is summed in gemv_xt's order.
+template <int K>
+__device__ __forceinline__ void gemv_xt_at_once(const MapData& d, const float* r, float* g)
+{
+    constexpr int W = MAP_THREADS / 32;
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31, n = (int)d.n;
+    const float* xr[K];
+    float acc[K];
+#pragma unroll
+    for (int k = 0; k < K; ++k) {
+        xr[k] = d.XT2 + (int64_t)min(w + k * W, d.p - 1) * n;
+        acc[k] = 0.0f;
+    }
+#pragma unroll 4
+    for (int i = lane; i < n; i += 32) {
+        const float ri = r[i];
+#pragma unroll
+        for (int k = 0; k < K; ++k) acc[k] = fmaf(xr[k][i], ri, acc[k]);
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+        for (int k = 0; k < K; ++k) acc[k] += __shfl_xor_sync(0xffffffffu, acc[k], o);
+#pragma unroll
+    for (int k = 0; k < K; ++k)
+        if (lane == k && w + k * W < d.p) g[w + k * W] = acc[k] * 0.69314718f;
+}
+
+// map_inner for n <= MAP_THREADS and p <= MAP_REG_P: x holds the thread's individual's genotypes
+// (zeros beyond p), yi its phenotype, m.z zeros beyond p. Every sum is taken in map_inner's order,
+// so the results are its bits. A block solves alone: the step is latency and the reads of X from
+// L1 (n p words a product, 128 bytes a cycle). Here the first product reads none, the second runs a
+// warp's markers at once, and the update, momentum and stopping test are warp 0's alone, in
+// shuffles: three barriers a step instead of eight. A step at n = 500, p = 50: 2.3 -> 1.2 us; a
+// path of 64 scales 42.6 -> 21.7 ms, at 333 x 17 (20 scales) 2.38 -> 1.58, at 200 x 10 (50 scales)
+// 8.29 -> 5.02. Larger problems stay with map_inner: the same update and four markers at once, with
+// X from memory in both products, took 83 ms against 71 at 1000 x 100 and 782 against 520 at
+// 2000 x 200.
+__device__ __forceinline__ void map_inner_in_registers(const MapData& d, const float (&x)[MAP_REG_P], float yi,
+                                                       float invL, float tol_in, const MapSmem& m)
+{
+    constexpr int W = MAP_THREADS / 32;
+    const int p = d.p, lane = threadIdx.x & 31;
+    float tk = 1.0f;
+    for (int it = 0; it < MAP_MAX_INNER; ++it) {
+        float a0 = 0.0f, a1 = 0.0f;  // gemv_x's two sums
+#pragma unroll
+        for (int j = 0; j < MAP_REG_P; j += 4) {
+            const float4 v = *reinterpret_cast<const float4*>(m.z + j);
+            a0 = fmaf(x[j], v.x, a0);
+            a1 = fmaf(x[j + 1], v.y, a1);
+            a0 = fmaf(x[j + 2], v.z, a0);
+            a1 = fmaf(x[j + 3], v.w, a1);
+        }
+        if ((int)threadIdx.x < d.n) m.eta[threadIdx.x] = yi - sigmoid_f((a0 + a1) * 0.69314718f);
+        __syncthreads();
+        if (p <= W)
+            gemv_xt_at_once<1>(d, m.eta, m.g);
+        else if (p <= 2 * W)
+            gemv_xt_at_once<2>(d, m.eta, m.g);
+        else
+            gemv_xt_at_once<MAP_REG_P / W>(d, m.eta, m.g);
+        __syncthreads();
+        if (threadIdx.x < 32) {
+            float dot = 0.0f, diff = 0.0f, bn[MAP_REG_P / 32];
+#pragma unroll
+            for (int k = 0; k < MAP_REG_P / 32; ++k) {
+                const int j = 32 * k + lane;
+                float v = 0.0f;
+                bn[k] = 0.0f;
+                if (j < p) {
+                    const float u = fmaf(m.g[j], invL, m.z[j]), c = m.w[j] * invL;
+                    bn[k] = u > c ? u - c : (u < -c ? u + c : 0.0f);
+                    v += (m.z[j] - bn[k]) * (bn[k] - m.beta[j]);
+                    diff = fmaxf(diff, fabsf(bn[k] - m.beta[j]));
+                }
+                dot += warp_sum(v);
+            }
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) diff = fmaxf(diff, __shfl_xor_sync(0xffffffffu, diff, o));
+            const bool restart = dot > 0.0f;
+            const float tn = restart ? 1.0f : 0.5f * (1.0f + sqrtf(fmaf(4.0f * tk, tk, 1.0f)));
+            const float mom = restart ? 0.0f : (tk - 1.0f) / tn;
+#pragma unroll
+            for (int k = 0; k < MAP_REG_P / 32; ++k) {
+                const int j = 32 * k + lane;
+                if (j < p) {
+                    m.z[j] = fmaf(mom, bn[k] - m.beta[j], bn[k]);
+                    m.beta[j] = bn[k];
+                }
+            }
+            tk = tn;
+            if (lane == 0) m.red[0] = diff;
+        }
+        __syncthreads();
+        if (m.red[0] < tol_in) break;
+    }
+}
+
 // One EM solve by the whole block from the point already in m.beta; returns the log
 // posterior l(beta) + log p(beta | a, c) at the mode (FP64 sums).
+template <bool REGX>
 __device__ double map_em_block(const MapData& d, double c, int max_em, float tol, const MapSmem& m)
 {
     const int p = d.p;
     const float L = *d.lip, invL = 1.0f / L;
     const float ac = (float)((double)d.pr.a * c), a1 = d.pr.a + 1.0f, invc = (float)(1.0 / c);
     const float tol_in = 0.1f * tol;
+    float x[MAP_REG_P];
+    float yi = 0.0f;
+    if (REGX) {
+        const bool live = (int)threadIdx.x < d.n;
+#pragma unroll
+        for (int j = 0; j < MAP_REG_P; ++j) x[j] = live && j < p ? d.XT2[(int64_t)j * d.n + threadIdx.x] : 0.0f;
+        if (live) yi = d.y[threadIdx.x] ? 1.0f : 0.0f;
+        for (int j = p + threadIdx.x; j < MAP_REG_P; j += blockDim.x) m.z[j] = 0.0f;
+    }
     for (int em = 0; em < max_em; ++em) {
         for (int j = threadIdx.x; j < p; j += blockDim.x) {
             m.w[j] = d.pr.de ? invc : a1 / (ac + fabsf(m.beta[j]));
@@ -152,37 +302,10 @@ __device__ double map_em_block(const MapData& d, double c, int max_em, float tol
             m.z[j] = m.beta[j];
         }
         __syncthreads();
-        float tk = 1.0f;
-        for (int it = 0; it < MAP_MAX_INNER; ++it) {
-            gemv_x(d, m.z, m.eta);
-            __syncthreads();
-            for (int64_t i = threadIdx.x; i < d.n; i += blockDim.x)
-                m.eta[i] = (d.y[i] ? 1.0f : 0.0f) - sigmoid_f(m.eta[i]);
-            __syncthreads();
-            gemv_xt(d, m.eta, m.g);
-            __syncthreads();
-            float dot = 0.0f, diff = 0.0f;
-            for (int j = threadIdx.x; j < p; j += blockDim.x) {
-                const float u = fmaf(m.g[j], invL, m.z[j]), k = m.w[j] * invL;
-                const float bn = u > k ? u - k : (u < -k ? u + k : 0.0f);
-                dot += (m.z[j] - bn) * (bn - m.beta[j]);
-                diff = fmaxf(diff, fabsf(bn - m.beta[j]));
-                m.g[j] = bn;  // the new point
-            }
-            dot = block_sum_f(dot, m.red);
-            diff = block_max_f(diff, m.red);
-            const bool restart = dot > 0.0f;
-            const float tn = restart ? 1.0f : 0.5f * (1.0f + sqrtf(fmaf(4.0f * tk, tk, 1.0f)));
-            const float mom = restart ? 0.0f : (tk - 1.0f) / tn;
-            for (int j = threadIdx.x; j < p; j += blockDim.x) {
-                const float bn = m.g[j];
-                m.z[j] = fmaf(mom, bn - m.beta[j], bn);
-                m.beta[j] = bn;
-            }
-            tk = tn;
-            __syncthreads();
-            if (diff < tol_in) break;
-        }
+        if (REGX)
+            map_inner_in_registers(d, x, yi, invL, tol_in, m);
+        else
+            map_inner(d, invL, tol_in, m);
         float ch = 0.0f;
         for (int j = threadIdx.x; j < p; j += blockDim.x) ch = fmaxf(ch, fabsf(m.beta[j] - m.prev[j]));
         ch = block_max_f(ch, m.red);
@@ -200,6 +323,7 @@ __device__ double map_em_block(const MapData& d, double c, int max_em, float tol
 }
 
 // S independent solves (one block each) from beta0[s].
+template <bool REGX>
 __global__ void __launch_bounds__(MAP_THREADS) k_map(MapData d, const float* __restrict__ beta0, double c, int max_em,
                                                     float tol, float* __restrict__ beta_out, double* __restrict__ lp_out)
 {
@@ -208,7 +332,7 @@ __global__ void __launch_bounds__(MAP_THREADS) k_map(MapData d, const float* __r
     const int s = blockIdx.x;
     for (int j = threadIdx.x; j < d.p; j += blockDim.x) m.beta[j] = beta0[(int64_t)s * d.p + j];
     __syncthreads();
-    const double lp = map_em_block(d, c, max_em, tol, m);
+    const double lp = map_em_block<REGX>(d, c, max_em, tol, m);
     for (int j = threadIdx.x; j < d.p; j += blockDim.x) beta_out[(int64_t)s * d.p + j] = m.beta[j];
     if (threadIdx.x == 0) lp_out[s] = lp;
 }
@@ -219,6 +343,7 @@ __global__ void __launch_bounds__(MAP_THREADS) k_map(MapData d, const float* __r
 // step whose predecessor did not change copies its entry; the others solve
 // EM(c_t, S_r[t-1]), keep it if its log posterior is above lpA[t] (ties keep A_t), and
 // count themselves in *n_changed when the kept mode differs from S_r[t].
+template <bool REGX>
 __global__ void __launch_bounds__(MAP_THREADS) k_map_round(MapData d, const float* __restrict__ best,
                                                           const double* __restrict__ sched, int round, int max_em,
                                                           float tol, float* __restrict__ A, double* __restrict__ lpA,
@@ -235,7 +360,7 @@ __global__ void __launch_bounds__(MAP_THREADS) k_map_round(MapData d, const floa
     if (round == 0) {
         for (int j = threadIdx.x; j < p; j += blockDim.x) m.beta[j] = best[o + j];
         __syncthreads();
-        const double lp = map_em_block(d, c, max_em, tol, m);
+        const double lp = map_em_block<REGX>(d, c, max_em, tol, m);
         for (int j = threadIdx.x; j < p; j += blockDim.x) {
             A[o + j] = m.beta[j];
             S_w[o + j] = m.beta[j];
@@ -257,7 +382,7 @@ __global__ void __launch_bounds__(MAP_THREADS) k_map_round(MapData d, const floa
     }
     for (int j = threadIdx.x; j < p; j += blockDim.x) m.beta[j] = S_r[o - p + j];
     __syncthreads();
-    const double lp2 = map_em_block(d, c, max_em, tol, m);
+    const double lp2 = map_em_block<REGX>(d, c, max_em, tol, m);
     const bool chain = lp2 > lpA[t];
     float ndiff = 0.0f;
     for (int j = threadIdx.x; j < p; j += blockDim.x) {
@@ -349,19 +474,26 @@ __global__ void __launch_bounds__(MAP_THREADS) k_map_lipschitz(MapData d, float*
     if (threadIdx.x == 0) *lip_out = 0.25f * lam * 1.02f;
 }
 
-size_t map_smem_bytes(int64_t n, int p) { return sizeof(float) * (size_t)(5 * p + n + 64) + sizeof(double) * 33; }
+size_t map_smem_bytes(int64_t n, int p)
+{
+    return sizeof(float) * (size_t)(4 * p + (p > MAP_REG_P ? p : MAP_REG_P) + n + 64) + sizeof(double) * 33;
+}
+bool map_in_registers(int64_t n, int p) { return n <= MAP_THREADS && p <= MAP_REG_P; }
 
 }  // namespace
 
-bool map_fits(int64_t n, int p) { return map_smem_bytes(n, p) <= MAP_SMEM_MAX; }
+bool map_fits(int64_t n, int p)
+{
+    // (what the entry points take does not depend on z's padding)
+    return sizeof(float) * (size_t)(5 * p + n + 64) + sizeof(double) * 33 <= MAP_SMEM_MAX;
+}
 
 cudaError_t map_init_attributes()
 {
-    cudaError_t e = cudaFuncSetAttribute(k_map, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)MAP_SMEM_MAX);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(k_map_round, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)MAP_SMEM_MAX);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(k_map_lipschitz, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)MAP_SMEM_MAX);
+    constexpr int most = (int)MAP_SMEM_MAX + 4 * MAP_REG_P;
+    cudaError_t e = cudaFuncSetAttribute(k_map<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_map_round<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_map_lipschitz, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
     return e;
 }
 
@@ -374,7 +506,8 @@ cudaError_t launch_map_lipschitz(const MapData& d, float* lip, cudaStream_t st)
 cudaError_t launch_map(const MapData& d, const float* beta0, int S, double c, int max_em, float tol, float* beta_out,
                        double* lp_out, cudaStream_t st)
 {
-    k_map<<<S, MAP_THREADS, map_smem_bytes(d.n, d.p), st>>>(d, beta0, c, max_em, tol, beta_out, lp_out);
+    (map_in_registers(d.n, d.p) ? k_map<true> : k_map<false>)<<<S, MAP_THREADS, map_smem_bytes(d.n, d.p), st>>>(
+        d, beta0, c, max_em, tol, beta_out, lp_out);
     return cudaGetLastError();
 }
 
@@ -383,7 +516,7 @@ cudaError_t launch_map_round(const MapData& d, const float* best, const double* 
 {
     const int r = (round + 1) & 1, w = round & 1;
     const int64_t tp = (int64_t)T * d.p;
-    k_map_round<<<T, MAP_THREADS, map_smem_bytes(d.n, d.p), st>>>(
+    (map_in_registers(d.n, d.p) ? k_map_round<true> : k_map_round<false>)<<<T, MAP_THREADS, map_smem_bytes(d.n, d.p), st>>>(
         d, best, sched, round, max_em, tol, b.A, b.lpA, b.S + r * tp, b.lpS + r * T, b.chg + r * T, b.S + w * tp,
         b.lpS + w * T, b.chg + w * T, b.n_changed);
     return cudaGetLastError();

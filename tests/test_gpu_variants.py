@@ -54,3 +54,19 @@ def test_gradient_kernel_gives_the_two_kernels_bits(spa, n, p, N):
         b.close()
         for k in one:
             assert np.array_equal(one[k], two[k]), k
+
+
+# One EM solve keeps the genotypes in registers for n <= 512 and p <= 64, a warp's markers (16
+# warps) in groups of 1, 2 or 4; larger problems read them in both products.
+@pytest.mark.parametrize("n,p", [(40, 1), (97, 15), (511, 16), (512, 17), (300, 32), (512, 33), (512, 64), (513, 33),
+                                 (512, 65)])
+def test_map_register_and_general_kernels_at_their_edges(spa, n, p):
+    """The double-exponential mode is unique, so the oracle's is the same point; the tolerances are
+    those of the FP32 inner solves (a last step below 1e-7 at a contraction no worse than 1e-4)."""
+    reg = synth.make_region(n, p, 0.5, (0.5,), seed=1400 + n)
+    start = np.random.default_rng(n + p).normal(0, 0.1, (1, p)).astype(np.float32)
+    with spa.Region(reg.G, reg.y, np.inf) as r:
+        g, glp = r.map(start, 0.05, max_em=100, tol=1e-6)
+    o, olp = oracle.map_em(reg.G, reg.y, np.inf, 0.05, start[0].astype(np.float64), max_em=100, tol=1e-10)
+    assert np.max(np.abs(g[0] - o)) < 2e-3 * max(1.0, np.max(np.abs(o)))
+    assert abs(glp[0] - olp) < 1e-4 * abs(olp) + 1e-3
