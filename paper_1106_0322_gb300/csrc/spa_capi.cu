@@ -254,6 +254,7 @@ int check_device(spa_ctx* c)
     CK(grad_tc_init_attributes(), "gradient kernel attributes");
     CK(site_init_attributes(), "single-coordinate kernel attributes");
     CK(map_init_attributes(), "MAP kernel attributes");
+    CK(simt_init_attributes(), "plain FP32 kernel attributes");
     if (c) {
         c->device = dev;
         c->num_sms = prop.multiProcessorCount;
@@ -751,7 +752,7 @@ void enq_loglik(Enq& q)
         q.ck(launch_loglik_tc(maps_of(c), plan_of(c), c->n, c->Kp, c->ybits, w.partial, w.N_pad, c->d_err, q.st,
                               nullptr, c->wait_ns, c->fault & FAULT_STALL));
     } else {
-        q.ck(launch_loglik_simt(w.beta_p, c->Xf, c->y, w.N, c->n, (int)c->p, w.partial, w.N_pad, q.st));
+        q.ck(launch_loglik_simt(w.beta_p, c->Xf, c->y, w.N, c->n, (int)c->p, w.partial, w.N_pad, plan_sm_count(c), q.st));
     }
 }
 
@@ -873,7 +874,8 @@ void enq_likelihood(Enq& q, const LikPoint& lp)
     }
     enq_loglik(q);
     if (mala) {
-        q.ck(launch_grad_simt(src, c->Xf, c->y, w.N, c->n, (int)c->p, w.eta, out, nullptr, c->pr, 0.0, q.st));
+        q.ck(launch_grad_simt(src, c->Xf, c->y, w.N, c->n, (int)c->p, w.eta, out, nullptr, c->pr, 0.0,
+                              plan_sm_count(c), q.st));
         ++q.launches;  // the plain adjoint is two kernels
     }
 }
@@ -1895,7 +1897,7 @@ static int loglik_impl(spa_ctx* c, const float* B, bool B_dev, int64_t N, double
                             c->wait_ns, fault_mask() & FAULT_STALL),
            "loglik tc");
     } else {
-        CK(launch_loglik_simt(w.beta_p, c->Xf, c->y, N, c->n, (int)p, w.partial, w.N_pad, st), "loglik simt");
+        CK(launch_loglik_simt(w.beta_p, c->Xf, c->y, N, c->n, (int)p, w.partial, w.N_pad, c->num_sms, st), "loglik simt");
     }
     CK(launch_finish_loglik(a.mh, N, nullptr, ll_dev ? ll : w.ll, c->d_err, st), "finish loglik");
     if (!ll_dev) CK(cudaMemcpyAsync(ll, w.ll, sizeof(double) * (size_t)N, cudaMemcpyDeviceToHost, st), "copy ll");
@@ -1915,7 +1917,7 @@ int spa_loglik_repeat(spa_ctx* c, int64_t N, int32_t reps, void* stream)
                             c->wait_ns),
                "loglik tc");
         } else {
-            CK(launch_loglik_simt(w.beta_p, c->Xf, c->y, N, c->n, (int)c->p, w.partial, w.N_pad, st), "loglik simt");
+            CK(launch_loglik_simt(w.beta_p, c->Xf, c->y, N, c->n, (int)c->p, w.partial, w.N_pad, c->num_sms, st), "loglik simt");
         }
     }
     return SPA_OK;
@@ -2125,7 +2127,7 @@ static int grad_impl(spa_ctx* c, const float* B, bool dev, int64_t N, double cs,
     CK(cudaMemcpyAsync(w.beta, B, sizeof(float) * (size_t)(N * p), dev ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, st),
        "copy B");
     CK(launch_grad_simt(w.beta, c->Xf, c->y, N, n, (int)p, w.eta, dev ? grad : w.grad, dev ? ll : (ll ? w.ll : nullptr),
-                        c->pr, cs, st),
+                        c->pr, cs, c->num_sms, st),
        "gradient");
     if (!dev) {
         CK(cudaMemcpyAsync(grad, w.grad, sizeof(float) * (size_t)(N * p), cudaMemcpyDeviceToHost, st), "copy grad");

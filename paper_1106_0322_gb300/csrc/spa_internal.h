@@ -453,12 +453,14 @@ cudaError_t launch_grad_finish(const float* gpart, int ksplit, const float* rsum
 // Plain FP32 SIMT path: partial[nt * N_pad + i] = -sum over 64-individual tile nt of
 // softplus(eta_r) (natural units; the linear half beta . v is added by the move kernels).
 constexpr int SIMT_TILE_N = 64;
+cudaError_t simt_init_attributes();
 cudaError_t launch_loglik_simt(const float* beta_p, const float* Xf, const uint8_t* y, int64_t N, int64_t n, int p,
-                               float* partial, int64_t N_pad, cudaStream_t st);
+                               float* partial, int64_t N_pad, int num_sms, cudaStream_t st);
 
-// Plain FP32 gradient: eta = B X^T materialised, r = y - logit^{-1}(eta); grad = r X
+// Plain FP32 gradient: r = y - logit^{-1}(B X^T) materialised; grad = r X
 // (+ prior gradient at c when c > 0); ll = sum y eta - softplus(eta).
 cudaError_t launch_grad_simt(const float* B, const float* Xf, const uint8_t* y, int64_t N, int64_t n, int p,
-                             float* eta_scratch, float* grad, double* ll, PriorArgs pr, double c, cudaStream_t st);
+                             float* eta_scratch, float* grad, double* ll, PriorArgs pr, double c, int num_sms,
+                             cudaStream_t st);
 
 }  // namespace spa

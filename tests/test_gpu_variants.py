@@ -70,3 +70,22 @@ def test_map_register_and_general_kernels_at_their_edges(spa, n, p):
     o, olp = oracle.map_em(reg.G, reg.y, np.inf, 0.05, start[0].astype(np.float64), max_em=100, tol=1e-10)
     assert np.max(np.abs(g[0] - o)) < 2e-3 * max(1.0, np.max(np.abs(o)))
     assert abs(glp[0] - olp) < 1e-4 * abs(olp) + 1e-3
+
+
+# The plain FP32 products run in tiles of 32 x 64, 64 x 64 or 128 x 128 (particles by individuals,
+# then particles by markers), 16 of the summed dimension at a time.
+@pytest.mark.parametrize("n,p,N", [(31, 1, 3), (64, 16, 32), (65, 17, 33), (129, 15, 64), (641, 33, 1030),
+                                   (1000, 100, 4096), (999, 101, 4095), (300, 500, 8191)])
+def test_plain_fp32_tiles_at_their_edges(spa, n, p, N):
+    """FP32 sums of at most 1000 terms: 1e-5 of the log-likelihood, 1e-5 of sum_i |x_ij| for the
+    gradient (FP32 rounding 6e-8 a term, and r's error of a quarter of eta's)."""
+    reg = synth.make_region(n, p, 0.9, (0.4,), seed=1500 + n)
+    B = synth.random_particles(N, p, 0.05, seed=p)
+    with spa.Region(reg.G, reg.y, 1.0, config=spa.make_config(precision="fp32")) as r:
+        l = r.loglik(B)
+        ll, g = r.grad(B, 0.0)
+    o_ll, o_g = oracle.loglik_grad(reg.G, reg.y, B.astype(np.float64))
+    assert np.all(np.abs(l - o_ll) <= 1e-5 * np.abs(o_ll))
+    assert np.all(np.abs(ll - o_ll) <= 1e-5 * np.abs(o_ll))
+    scale = np.abs((reg.G - reg.G.mean(0)) / reg.G.std(0)).sum(0)
+    assert np.all(np.abs(g - o_g) <= 1e-5 * scale[None, :])
