@@ -296,6 +296,13 @@ __global__ void __launch_bounds__(BLOCK, 5) k_move_rw(MoveArgs a, int64_t N, int
 {
     __shared__ int accw[BLOCK / 32];
     __shared__ PartSlices parts;
+    const int64_t i = warp_global_id();
+    const int lane = threadIdx.x & 31, groups = (p + 3) >> 2;
+    // The first group's normals depend on nothing that the previous kernel writes: drawn by blocks that
+    // are resident before it ends. RW step of 10 moves at n = 2000, p = 200, N = 8192: 331 -> 328 us;
+    // 5 moves at n = 1859, p = 183, N = 5003: 190 -> 187.
+    float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (noise && i < N && lane < groups) z = normals4(*seedp, (uint32_t)lane, (uint32_t)i, (uint32_t)t, m);
     grid_dependency_wait();  // the previous kernel (the likelihood GEMM) has finished
     grid_launch_dependents();
     if (DECIDE) {
@@ -303,8 +310,6 @@ __global__ void __launch_bounds__(BLOCK, 5) k_move_rw(MoveArgs a, int64_t N, int
         __syncthreads();
     }
     const float4 sk = stepk[t];
-    const int64_t i = warp_global_id();
-    const int lane = threadIdx.x & 31;
     bool acc = false;  // the state is the row in beta_p: an accepted proposal, or a resampled particle
     if (i < N) {
         const uint64_t seed = (noise || DECIDE) ? *seedp : 0ull;
@@ -318,10 +323,8 @@ __global__ void __launch_bounds__(BLOCK, 5) k_move_rw(MoveArgs a, int64_t N, int
         __nv_bfloat16* Arow = a.A ? a.A + i * (int64_t)a.ldA : nullptr;
         FSum lt;
         float yd = 0.0f, off = 0.0f;
-        const int groups = (p + 3) >> 2;
         for (int g = lane; g < groups; g += 32) {
-            float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
-            if (noise) z = normals4(seed, (uint32_t)g, (uint32_t)i, (uint32_t)t, m);
+            if (noise && g >= 32) z = normals4(seed, (uint32_t)g, (uint32_t)i, (uint32_t)t, m);
             rw_group<VEC>(a, p, g, true, acc, noise, z, sk.w, pr.de, src, dst, cur, Arow, lt, yd, off);
         }
         lt = warp_sum(lt);
@@ -392,6 +395,10 @@ __global__ void __launch_bounds__(BLOCK, 4) k_move_mala(MoveArgs a, int64_t N, i
 {
     __shared__ int accw[BLOCK / 32];
     __shared__ PartSlices parts;
+    const int64_t i = warp_global_id();
+    const int lane = threadIdx.x & 31, groups = (p + 3) >> 2;
+    float4 z4 = make_float4(0.f, 0.f, 0.f, 0.f);  // (as in k_move_rw)
+    if (VEC && i < N && lane < groups) z4 = normals4(*seedp, (uint32_t)lane, (uint32_t)i, (uint32_t)t, m);
     grid_dependency_wait();  // the previous kernel (the gradient finish, or the step's proposal scales) has finished
     grid_launch_dependents();
     if (DECIDE) {
@@ -399,8 +406,6 @@ __global__ void __launch_bounds__(BLOCK, 4) k_move_mala(MoveArgs a, int64_t N, i
         __syncthreads();
     }
     const float4 sk = stepk[t];
-    const int64_t i = warp_global_id();
-    const int lane = threadIdx.x & 31;
     bool acc = false;
     if (i < N) {
         const uint64_t seed = *seedp;
@@ -423,13 +428,12 @@ __global__ void __launch_bounds__(BLOCK, 4) k_move_mala(MoveArgs a, int64_t N, i
         __nv_bfloat16* Arow = a.A ? a.A + i * (int64_t)a.ldA : nullptr;
         FSum lt, fw;
         float yd = 0.0f, off = 0.0f;
-        const int groups = (p + 3) >> 2;
         const bool grouped = (p & 3) == 0 && !pr.de;  // the four-coordinate prior term
         if (VEC) {
             // p % 4 == 0: the same per-coordinate arithmetic on float4 groups, the state's and
             // the gradient's rows read and written 16 bytes at a time, the GEMM row 8
             for (int g = lane; g < groups; g += 32) {
-                const float4 z4 = normals4(seed, (uint32_t)g, (uint32_t)i, (uint32_t)t, m);
+                if (g >= 32) z4 = normals4(seed, (uint32_t)g, (uint32_t)i, (uint32_t)t, m);
                 const int j0 = 4 * g;
                 const float4 x0 = ld4(src + j0), g0 = ld4(gsrc + j0);
                 if (acc) {
