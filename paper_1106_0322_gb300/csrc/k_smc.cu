@@ -1212,7 +1212,6 @@ __global__ void k_colstats_finish(const float4* __restrict__ part, int p, int sp
 // round(W 2^31), so every cumulative sum is exact and independent of the order of the
 // atomic additions.
 constexpr int SUM_THREADS = 512;
-constexpr size_t SUM_STAGED_MAX = 200 * 1024;  // dynamic shared memory of the staged variant
 
 __device__ __forceinline__ uint32_t float_key(float f)
 {
@@ -1235,6 +1234,7 @@ __device__ int warp_find_bin(const uint32_t* hist, int nbins, unsigned long long
     const int per = nbins / 32;
     const uint32_t* mine_p = hist + lane * per;
     unsigned long long mine = 0;
+#pragma unroll 16
     for (int k = 0; k < per; ++k) mine += mine_p[(k + lane) & (per - 1)];
     unsigned long long incl = mine;
 #pragma unroll
@@ -1311,23 +1311,47 @@ __global__ void k_keys_transpose(const float* __restrict__ beta, int64_t N, int 
     }
 }
 
-constexpr int SUM_SUB = 4;     // sub-histograms of the first radix digit (by warp % 4)
+// Two compensated sums at once, in packed operations (each rounds as its scalar form).
+struct FSum2 {
+    static __device__ __forceinline__ void add(FSum& a, FSum& b, float xa, float xb)
+    {
+        const uint64_t neg = pack2(-1.0f, -1.0f);
+        const uint64_t s = pack2(a.s, b.s), x = pack2(xa, xb);
+        const uint64_t t = add2(s, x);
+        const uint64_t z = fma2(s, neg, t);                                       // t - s
+        const uint64_t e = add2(fma2(fma2(z, neg, t), neg, s), fma2(z, neg, x));  // (s - (t - z)) + (x - z)
+        const uint64_t c = add2(pack2(a.c, b.c), e);
+        const float2 t2 = unpack2(t), c2 = unpack2(c);
+        a.s = t2.x;
+        b.s = t2.y;
+        a.c = c2.x;
+        b.c = c2.y;
+    }
+};
+
+constexpr int SUM_SUB = 4;     // sub-histograms of the first radix digit (by lane % 4)
 constexpr int SUM_BINS = 2048;  // bins of an 11-bit digit
 
 // Per coordinate j (one CTA): the weighted mean and the concentrations (compensated FP32
 // sums), and the weighted quantiles by an exact radix select on the fixed-point weights
 // round(W 2^31) over the order-preserving integer keys of the values: digits of 11, 11 and
 // 10 bits from the top. The first digit's histogram is built while the values are loaded,
-// in SUM_SUB copies that are merged before the search (particles cluster in a few
-// top-digit bins, and one copy per warp group spreads their atomics).
+// in SUM_SUB copies that are merged before the search: particles cluster in a few top-digit
+// bins, and neighbouring copies in neighbouring banks spread a warp's atomics. The later digits'
+// passes read the keys again (from L2), and the weights of those in a selected bin only: kept in
+// shared memory instead, keys and weights took 8 N bytes, one CTA an SM from N = 12000 on.
+// At most NQ levels and ND thresholds; the usual few take less work a value. Bound by instructions
+// and the latency of the reads; it runs beside the next step and keeps the likelihood kernel off the
+// SMs it holds. n = 2000, p = 200, N = 8192: 34 -> 20 us, a RW step of 10 moves 333 -> 328;
+// n = 5000, p = 500, N = 16384: 143 -> 56 us, step 1479 -> 1395.
+template <int NQ, int ND>
 __global__ void __launch_bounds__(SUM_THREADS, 2) k_summaries(const uint32_t* __restrict__ keysT, const float* __restrict__ Wf,
                                                                const uint32_t* __restrict__ wfix, int64_t N, int p,
                                                                SummaryArgs sa, int t, double* __restrict__ mean,
-                                                               double* __restrict__ quant, double* __restrict__ conc,
-                                                               int staged)
+                                                               double* __restrict__ quant, double* __restrict__ conc)
 {
     grid_dependency_wait();
-    extern __shared__ uint32_t sm[];
+    extern __shared__ __align__(16) uint32_t hist[];  // max(SUM_SUB, nq) * SUM_BINS words
     __shared__ float red_s[SUM_THREADS / 32][9], red_c[SUM_THREADS / 32][9];
     __shared__ unsigned long long shu[SUM_THREADS / 32];
     __shared__ uint32_t shk[SUM_THREADS / 32];
@@ -1336,42 +1360,52 @@ __global__ void __launch_bounds__(SUM_THREADS, 2) k_summaries(const uint32_t* __
     const int j = blockIdx.x;
     const int tid = threadIdx.x, w = tid >> 5, lane = tid & 31;
     const int nq = (quant && sa.nq > 0) ? sa.nq : 0, nd = sa.nd;
-    uint32_t* keys = sm;
-    uint32_t* wts = sm + (staged ? N : 0);
-    uint32_t* hist = sm + (staged ? 2 * N : 0);  // max(SUM_SUB, nq) * SUM_BINS words
     if (nq > 0) {
-        for (int e = tid; e < SUM_SUB * SUM_BINS; e += SUM_THREADS) hist[e] = 0u;
+        for (int e = tid; e < SUM_SUB * SUM_BINS / 4; e += SUM_THREADS)
+            reinterpret_cast<uint4*>(hist)[e] = make_uint4(0u, 0u, 0u, 0u);
         if (tid < 8) below[tid] = 0ull;
         __syncthreads();
     }
-    uint32_t* hsub = hist + (w & (SUM_SUB - 1)) * SUM_BINS;
-    // ---- load: stage keys and weights; mean, concentrations, top-digit histogram
+    uint32_t* hsub = hist + (lane & (SUM_SUB - 1));
+    // ---- mean, concentrations, top-digit histogram
     FSum msum;
-    FSum cs[8];
+    FSum cs[ND];
     uint32_t kmax = 0;
     unsigned long long tot = 0;
     const uint32_t* kcol = keysT + (int64_t)j * N;
-    for (int64_t i = tid; i < N; i += SUM_THREADS) {
-        const uint32_t k = kcol[i];
+    auto take = [&](uint32_t k, uint32_t wv, float wf) {
         const float b = key_float(k);
-        const uint32_t wv = wfix[i];
-        const float wf = Wf[i];
-        if (staged) {
-            keys[i] = k;
-            wts[i] = wv;
-        }
         msum.add(wf * b);
+        if (ND == 2) {  // a zero term leaves a compensated sum as it is
+            FSum2::add(cs[0], cs[1], fabsf(b) < sa.dthr[0] ? wf : 0.0f, fabsf(b) < sa.dthr[1] ? wf : 0.0f);
+        } else {
 #pragma unroll
-        for (int d = 0; d < 8; ++d)
-            if (d < nd && fabsf(b) < sa.dthr[d]) cs[d].add(wf);
+            for (int d = 0; d < ND; ++d)
+                if (d < nd && fabsf(b) < sa.dthr[d]) cs[d].add(wf);
+        }
         kmax = k > kmax ? k : kmax;
         tot += wv;
-        if (nq > 0 && wv != 0u) atomicAdd(&hsub[k >> 21], wv);
+        if (nq > 0 && wv != 0u) atomicAdd(&hsub[(k >> 21) * SUM_SUB], wv);
+    };
+    constexpr int U = 4;  // elements a thread has in flight
+    int64_t i = tid;
+    for (; i + (U - 1) * SUM_THREADS < N; i += U * SUM_THREADS) {
+        uint32_t k[U], wv[U];
+        float wf[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            k[u] = kcol[i + u * SUM_THREADS];
+            wv[u] = wfix[i + u * SUM_THREADS];
+            wf[u] = Wf[i + u * SUM_THREADS];
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u) take(k[u], wv[u], wf[u]);
     }
+    for (; i < N; i += SUM_THREADS) take(kcol[i], wfix[i], Wf[i]);
     // ---- one block reduction for every scalar
     msum = warp_sum(msum);
 #pragma unroll
-    for (int d = 0; d < 8; ++d)
+    for (int d = 0; d < ND; ++d)
         if (d < nd) cs[d] = warp_sum(cs[d]);
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
@@ -1382,7 +1416,7 @@ __global__ void __launch_bounds__(SUM_THREADS, 2) k_summaries(const uint32_t* __
         red_s[w][0] = msum.s;
         red_c[w][0] = msum.c;
 #pragma unroll
-        for (int d = 0; d < 8; ++d)
+        for (int d = 0; d < ND; ++d)
             if (d < nd) {
                 red_s[w][1 + d] = cs[d].s;
                 red_c[w][1 + d] = cs[d].c;
@@ -1414,13 +1448,17 @@ __global__ void __launch_bounds__(SUM_THREADS, 2) k_summaries(const uint32_t* __
         tot += shu[k];
         kmax = max(kmax, shk[k]);
     }
-    // merge the top-digit copies into copy 0
-    for (int b = tid; b < SUM_BINS; b += SUM_THREADS) {
-        uint32_t v = hist[b];
+    // merge the top-digit copies: bin b's in words SUM_SUB b .., their sum in word b
+    static_assert(SUM_SUB == 4 && SUM_BINS % SUM_THREADS == 0, "one uint4 a bin");
+    uint32_t merged[SUM_BINS / SUM_THREADS];
 #pragma unroll
-        for (int s2 = 1; s2 < SUM_SUB; ++s2) v += hist[s2 * SUM_BINS + b];
-        hist[b] = v;
+    for (int u = 0; u < SUM_BINS / SUM_THREADS; ++u) {
+        const uint4 v = reinterpret_cast<const uint4*>(hist)[tid + u * SUM_THREADS];
+        merged[u] = v.x + v.y + v.z + v.w;
     }
+    __syncthreads();
+#pragma unroll
+    for (int u = 0; u < SUM_BINS / SUM_THREADS; ++u) hist[tid + u * SUM_THREADS] = merged[u];
     __syncthreads();
     // ---- digit searches: the top digit on the merged histogram, then bits 10..20 and 0..9
     // of the keys that share the selected prefix, one histogram per quantile level
@@ -1429,26 +1467,36 @@ __global__ void __launch_bounds__(SUM_THREADS, 2) k_summaries(const uint32_t* __
         const int shift = (pass == 0) ? 21 : ((pass == 1) ? 10 : 0);
         const int nb = 1 << bits;
         if (pass > 0) {
-            uint32_t want[8];
-            bool on[8];
+            uint32_t want[NQ];  // (no key has the prefix ~0)
 #pragma unroll
-            for (int q = 0; q < 8; ++q) {
-                on[q] = q < nq && bins[q][0] >= 0;
-                want[q] = on[q] ? ((pass == 1) ? (uint32_t)bins[q][0] : (((uint32_t)bins[q][0] << 11) | (uint32_t)bins[q][1]))
-                                : 0u;
-            }
+            for (int q = 0; q < NQ; ++q)
+                want[q] = q < nq && bins[q][0] >= 0
+                              ? ((pass == 1) ? (uint32_t)bins[q][0] : (((uint32_t)bins[q][0] << 11) | (uint32_t)bins[q][1]))
+                              : ~0u;
             for (int e = tid; e < nq * nb; e += SUM_THREADS) hist[e] = 0u;
             __syncthreads();
-            for (int64_t i = tid; i < N; i += SUM_THREADS) {
-                const uint32_t k = staged ? keys[i] : kcol[i];
-                const uint32_t wv = staged ? wts[i] : wfix[i];
-                if (wv == 0u) continue;
-                const uint32_t dig = (k >> shift) & (uint32_t)(nb - 1);
+            auto look = [&](uint32_t k, int64_t at) {
                 const uint32_t pre = k >> (shift + bits);
+                bool any = false;
 #pragma unroll
-                for (int q = 0; q < 8; ++q)
-                    if (on[q] && pre == want[q]) atomicAdd(&hist[q * nb + dig], wv);
+                for (int q = 0; q < NQ; ++q) any |= pre == want[q];
+                if (!any) return;
+                const uint32_t wv = wfix[at];
+                if (wv == 0u) return;
+                const uint32_t dig = (k >> shift) & (uint32_t)(nb - 1);
+#pragma unroll
+                for (int q = 0; q < NQ; ++q)
+                    if (pre == want[q]) atomicAdd(&hist[q * nb + dig], wv);
+            };
+            int64_t at = tid;
+            for (; at + (2 * U - 1) * SUM_THREADS < N; at += 2 * U * SUM_THREADS) {
+                uint32_t k[2 * U];
+#pragma unroll
+                for (int u = 0; u < 2 * U; ++u) k[u] = kcol[at + u * SUM_THREADS];
+#pragma unroll
+                for (int u = 0; u < 2 * U; ++u) look(k[u], at + u * SUM_THREADS);
             }
+            for (; at < N; at += SUM_THREADS) look(kcol[at], at);
             __syncthreads();
         }
         if (w < nq) {
@@ -1632,7 +1680,8 @@ static unsigned elem_grid(int64_t total)
 
 cudaError_t smc_init_attributes()
 {
-    return cudaFuncSetAttribute(k_summaries, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SUM_STAGED_MAX);
+    return cudaFuncSetAttribute(k_summaries<8, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                8 * SUM_BINS * (int)sizeof(uint32_t));
 }
 
 cudaError_t launch_init_prior(float* beta, int64_t N, int p, PriorArgs pr, const double* sched, int t0,
@@ -1865,14 +1914,12 @@ cudaError_t launch_summaries_keys(const uint32_t* keysT, const float* Wf, const 
     }
     for (int q = 0; q < 8; ++q) a.target[q] = (unsigned long long)std::ceil(a.q[q] * 2147483648.0);
     const int nh = (quant && s.nq > 0) ? (s.nq > SUM_SUB ? s.nq : SUM_SUB) : 0;
-    const size_t hist_bytes = (size_t)nh * SUM_BINS * sizeof(uint32_t);
-    const size_t staged_bytes = (size_t)N * 2 * sizeof(uint32_t) + hist_bytes;
-    const int staged = staged_bytes <= SUM_STAGED_MAX ? 1 : 0;
-    const size_t bytes = staged ? staged_bytes : hist_bytes;
+    const size_t bytes = (size_t)nh * SUM_BINS * sizeof(uint32_t);
+    auto* kern = (s.nq <= 4 && s.nd <= 2) ? k_summaries<4, 2> : k_summaries<8, 8>;
     if (pdl)
-        return launch_pdl(k_summaries, dim3((unsigned)p), dim3(SUM_THREADS), bytes, st, keysT, Wf, wfix, N, p, a, t, mean,
-                          quant, conc, staged);
-    k_summaries<<<(unsigned)p, SUM_THREADS, bytes, st>>>(keysT, Wf, wfix, N, p, a, t, mean, quant, conc, staged);
+        return launch_pdl(kern, dim3((unsigned)p), dim3(SUM_THREADS), bytes, st, keysT, Wf, wfix, N, p, a, t, mean, quant,
+                          conc);
+    kern<<<(unsigned)p, SUM_THREADS, bytes, st>>>(keysT, Wf, wfix, N, p, a, t, mean, quant, conc);
     return cudaGetLastError();
 }
 

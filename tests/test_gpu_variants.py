@@ -89,3 +89,22 @@ def test_plain_fp32_tiles_at_their_edges(spa, n, p, N):
     assert np.all(np.abs(ll - o_ll) <= 1e-5 * np.abs(o_ll))
     scale = np.abs((reg.G - reg.G.mean(0)) / reg.G.std(0)).sum(0)
     assert np.all(np.abs(g - o_g) <= 1e-5 * scale[None, :])
+
+
+# The summaries kernel is compiled for up to 4 quantile levels and 2 thresholds, and for 8 and 8;
+# 512 threads read 4 (then 8) values each at a time.
+@pytest.mark.parametrize("N", [1, 31, 511, 513, 2048, 2051, 4096, 5003])
+def test_summary_kernels_give_the_same_values(spa, N):
+    reg = synth.make_region(150, 6, 0.9, (0.5,), seed=1600)
+    sched = synth.geometric_schedule(3, -4.0, -1.0)
+    few, many = dict(quantiles=(0.05, 0.5, 0.95), deltas=(0.05, 0.1)), dict(
+        quantiles=(0.01, 0.05, 0.25, 0.5, 0.75, 0.95, 0.99, 0.999), deltas=(0.01, 0.05, 0.1, 0.2))
+    out = []
+    for cfg in (few, many):
+        with spa.Region(reg.G, reg.y, 1.0, config=spa.make_config(move="rw", **cfg)) as r:
+            out.append(r.run(sched, N, 1, 4))
+    assert np.array_equal(out[0]["mean"], out[1]["mean"])
+    assert np.array_equal(out[0]["quantile"], out[1]["quantile"][:, :, [1, 3, 5]])
+    assert np.array_equal(out[0]["conc"], out[1]["conc"][:, :, 1:3])
+    q = out[1]["quantile"]
+    assert np.all(np.diff(q, axis=2) >= 0.0)
