@@ -859,84 +859,126 @@ __global__ void k_mark_uniform(int64_t N, int t, double* ess_out, uint8_t* res_o
 // The cumulative sum C of W in the specified order: a running sum inside each 256-block
 // in index order, a running sum of the block totals, C_i = carry(block) + local_i. cum holds
 // N + ceil(N/256) + 1 doubles: the block-local running sums, then one carry per block, then u.
-// Three kernels spread it over the SMs: the local sums (16 blocks of 256 per CTA, staged in
-// shared memory with coalesced loads and stores; lane l of warp 0 runs block l's additions),
-// the carries (one thread, in block order), and the search, which forms C_i = carry + local_i
-// as it reads it. The association order, and so every bit of C, is that of the definition.
-constexpr int RS_BLOCK = 256;         // cumulative-sum block of the specified association order
-constexpr int RS_CHUNKS = 16;         // 256-blocks per CTA of the local pass (33 KB of shared memory)
-constexpr int RS_PAD = RS_BLOCK + 1;  // shared-memory row of one 256-block (odd stride: no bank conflicts)
-constexpr int RS_LOCAL_THREADS = 256;
-constexpr size_t RS_LOCAL_SMEM = sizeof(double) * RS_CHUNKS * RS_PAD;
-constexpr int RS_CARRY_THREADS = 1024;
-constexpr int RS_TOT = 4096;  // block totals staged per pass of the carry kernel
+// Three kernels spread it over the SMs: the local sums (a warp per block), the carries (one
+// warp, in block order), and the search, which forms C_i = carry + local_i as it reads it.
+// Every bit of C is that of additions in the definition's order (running_sums).
+constexpr int RS_BLOCK = 256;  // cumulative-sum block of the specified association order
+constexpr int RS_CHUNKS = 4;   // 256-blocks (warps) per CTA of the local pass
+constexpr int RS_CARRY_GROUPS = 8;  // block totals a lane of the carry kernel reads ahead
 
-__global__ void __launch_bounds__(RS_LOCAL_THREADS) k_resample_local(const double* __restrict__ W, int64_t N,
-                                                                     double* __restrict__ cum,
-                                                                     const int* __restrict__ flag)
+// The 32 running sums S + w_0, (S + w_0) + w_1, ... of a warp's values, each rounded as that chain
+// of FP64 additions rounds; lane l's in r, the last returned.
+//
+// The chain itself is 32 additions of about 110 cycles, one after the other. But as long as the sum
+// keeps its exponent e, an addition adds to its 53-bit integer mantissa M the addend's mantissa
+// shifted right, rounded to nearest, a tie to the even sum: M + d0 if M is even, M + d1 if it is
+// odd, integers that each lane knows by itself. Such pairs compose associatively (the first
+// step's sum decides which of the second's is taken), so one scan gives all 32 sums. The lanes
+// before the first whose sum leaves the exponent, or whose addend is above it, have their
+// result; that one lane's is an FP64 addition, and the scan begins again behind it. A sum of
+// n terms of one size changes its exponent about log2 n times. The local pass, 256 additions in a
+// row: 19 -> 10 us at N = 1024 and 8192. A whole resampling of 10^5 weights: 62 -> 43 us.
+// Negative, infinite and NaN addends take the addition (their exponent field reads as larger).
+__device__ __forceinline__ double running_sums(double S, double w, double& r)
+{
+    constexpr unsigned long long TOP = 1ull << 52, HALF = 1ull << 63;
+    const int lane = threadIdx.x & 31;
+    const unsigned long long wb = (unsigned long long)__double_as_longlong(w);
+    const int ew = max((int)(wb >> 52), 1);  // (a subnormal has exponent 1 and no leading one)
+    const unsigned long long mw = (wb & (TOP - 1)) | (wb >= TOP ? TOP : 0ull);
+    int first = 0;  // the lanes before it are done
+    if (S == 0.0) {  // the first few sums change their exponent most often
+        for (; first < 8; ++first) {
+            S = __dadd_rn(S, __shfl_sync(0xffffffffu, w, first));
+            if (lane == first) r = S;
+        }
+    }
+    for (;;) {
+        const unsigned long long sb = (unsigned long long)__double_as_longlong(S);
+        const int e = max((int)(sb >> 52), 1), sh = e - ew;
+        const unsigned long long M = (sb & (TOP - 1)) | (sb >= TOP ? TOP : 0ull);
+        const bool chain = e < 0x7ff && sh >= 0;
+        unsigned long long d0 = 0, d1 = 0;
+        if (lane >= first && chain && sh < 64) {
+            const unsigned long long q = mw >> sh, rest = sh ? mw << (64 - sh) : 0ull;
+            const unsigned long long up = rest > HALF ? 1ull : 0ull, tie = rest == HALF ? 1ull : 0ull;
+            d0 = q + up + (tie & q & 1ull);
+            d1 = q + up + (tie & ~q & 1ull);
+        }
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const unsigned long long p0 = __shfl_up_sync(0xffffffffu, d0, o), p1 = __shfl_up_sync(0xffffffffu, d1, o);
+            if (lane >= o) {
+                const unsigned long long n0 = p0 + (p0 & 1ull ? d1 : d0), n1 = p1 + (p1 & 1ull ? d0 : d1);
+                d0 = n0;
+                d1 = n1;
+            }
+        }
+        const unsigned long long sum = M + (M & 1ull ? d1 : d0);
+        const unsigned int out = __ballot_sync(0xffffffffu, lane >= first && (!chain || sum >= 2 * TOP));
+        const int f = out ? __ffs(out) - 1 : 32;
+        const double v = __longlong_as_double((long long)(((unsigned long long)(e - 1) << 52) + sum));
+        if (lane >= first && lane < f) r = v;
+        const double before = f > first ? __shfl_sync(0xffffffffu, v, f - 1) : S;
+        if (f == 32) return before;
+        S = __dadd_rn(before, __shfl_sync(0xffffffffu, w, f));
+        if (lane == f) r = S;
+        first = f + 1;
+        if (first == 32) return S;
+    }
+}
+
+__global__ void __launch_bounds__(32 * RS_CHUNKS) k_resample_local(const double* __restrict__ W, int64_t N,
+                                                                   double* __restrict__ cum,
+                                                                   const int* __restrict__ flag)
 {
     grid_dependency_wait();
     if (flag && *flag == 0) return;
-    extern __shared__ double rs_sm[];
-    const int64_t i0 = (int64_t)blockIdx.x * RS_CHUNKS * RS_BLOCK;
-    const int64_t len = (N - i0 < (int64_t)RS_CHUNKS * RS_BLOCK) ? N - i0 : (int64_t)RS_CHUNKS * RS_BLOCK;
-    for (int64_t e = threadIdx.x; e < len; e += RS_LOCAL_THREADS)
-        rs_sm[(e / RS_BLOCK) * RS_PAD + (e % RS_BLOCK)] = W[i0 + e];
-    __syncthreads();
-    if (threadIdx.x < RS_CHUNKS) {
-        const int c = threadIdx.x;
-        const int64_t c0 = (int64_t)c * RS_BLOCK;
-        if (c0 < len) {
-            const int cl = (len - c0 < RS_BLOCK) ? (int)(len - c0) : RS_BLOCK;
-            double* row = rs_sm + c * RS_PAD;
-            double local = 0.0;
-            int k = 0;
-            for (; k + 16 <= cl; k += 16) {  // 16 loads ahead of the chain of additions
-                double v[16];
+    const int64_t b = (int64_t)blockIdx.x * RS_CHUNKS + (threadIdx.x >> 5), i0 = b * RS_BLOCK + (threadIdx.x & 31);
+    if (b * RS_BLOCK >= N) return;
+    double w[RS_BLOCK / 32];
 #pragma unroll
-                for (int q = 0; q < 16; ++q) v[q] = row[k + q];
+    for (int g = 0; g < RS_BLOCK / 32; ++g) w[g] = i0 + 32 * g < N ? W[i0 + 32 * g] : 0.0;
+    double local = 0.0;
+#pragma unroll 1
+    for (int g = 0; g < RS_BLOCK / 32; ++g) {
+        double r, x = w[0];  // (shifted along, so that the loop's body stands once)
+        local = running_sums(local, x, r);
+        if (i0 + 32 * g < N) cum[i0 + 32 * g] = r;
 #pragma unroll
-                for (int q = 0; q < 16; ++q) {
-                    local = __dadd_rn(local, v[q]);
-                    row[k + q] = local;
-                }
-            }
-            for (; k < cl; ++k) {
-                local = __dadd_rn(local, row[k]);
-                row[k] = local;
-            }
-            // the block total, turned into the block's carry by k_resample_carry
-            cum[N + (i0 / RS_BLOCK) + c] = local;
-        }
+        for (int k = 0; k + 1 < RS_BLOCK / 32; ++k) w[k] = w[k + 1];
     }
-    __syncthreads();
-    for (int64_t e = threadIdx.x; e < len; e += RS_LOCAL_THREADS) cum[i0 + e] = rs_sm[(e / RS_BLOCK) * RS_PAD + (e % RS_BLOCK)];
+    // the block total, turned into the block's carry by k_resample_carry
+    if ((threadIdx.x & 31) == 0) cum[N + b] = local;
 }
 
 // carry[b] = total_0 + ... + total_{b-1} in block order (the totals are read from the carry
-// slots and replaced), then the resampling uniform after the carries.
-__global__ void __launch_bounds__(RS_CARRY_THREADS) k_resample_carry(int64_t N, double* __restrict__ cum,
-                                                                     const int* __restrict__ flag, int t,
-                                                                     const uint64_t* __restrict__ seedp,
-                                                                     double u_override)
+// slots and replaced), then the resampling uniform after the carries. One warp.
+__global__ void __launch_bounds__(32) k_resample_carry(int64_t N, double* __restrict__ cum,
+                                                       const int* __restrict__ flag, int t,
+                                                       const uint64_t* __restrict__ seedp, double u_override)
 {
     grid_dependency_wait();
     if (flag && *flag == 0) return;
-    __shared__ double tot[RS_TOT];
     const int tid = threadIdx.x;
     const int64_t nblk = (N + RS_BLOCK - 1) / RS_BLOCK;
     double* carry = cum + N;
-    double run = 0.0;  // thread 0's running sum of block totals
-    for (int64_t b0 = 0; b0 < nblk; b0 += RS_TOT) {
-        const int64_t b1 = (b0 + RS_TOT < nblk) ? b0 + RS_TOT : nblk;
-        for (int64_t b = b0 + tid; b < b1; b += RS_CARRY_THREADS) tot[b - b0] = carry[b];
-        __syncthreads();
-        if (tid == 0)
-            for (int64_t b = b0; b < b1; ++b) {
-                carry[b] = run;
-                run = __dadd_rn(run, tot[b - b0]);
-            }
-        __syncthreads();
+    double run = 0.0;
+    for (int64_t b0 = 0; b0 < nblk; b0 += 32 * RS_CARRY_GROUPS) {
+        double w[RS_CARRY_GROUPS];
+#pragma unroll
+        for (int g = 0; g < RS_CARRY_GROUPS; ++g) w[g] = b0 + 32 * g + tid < nblk ? carry[b0 + 32 * g + tid] : 0.0;
+#pragma unroll 1
+        for (int g = 0; g < RS_CARRY_GROUPS; ++g) {
+            const int64_t b = b0 + 32 * g + tid;
+            double r;
+            const double next = running_sums(run, w[0], r);
+            const double prev = __shfl_up_sync(0xffffffffu, r, 1);
+            if (b < nblk) carry[b] = tid == 0 ? run : prev;
+            run = next;
+#pragma unroll
+            for (int k = 0; k + 1 < RS_CARRY_GROUPS; ++k) w[k] = w[k + 1];
+        }
     }
     if (tid == 0) {
         if (seedp) {
@@ -1036,11 +1078,15 @@ __global__ void __launch_bounds__(BLOCK) k_resample_gather(const double* __restr
         us = u01_d(x.x);
     }
     __syncthreads();
-    if (threadIdx.x == 0) {
+    if (threadIdx.x < 32) {
         double run = 0.0;
-        for (int b = 0; b < nblk; ++b) {
-            carry[b] = run;
-            run = __dadd_rn(run, tot[b]);
+        for (int b0 = 0; b0 < nblk; b0 += 32) {
+            const int b = b0 + (int)threadIdx.x;
+            double r;
+            const double next = running_sums(run, b < nblk ? tot[b] : 0.0, r);
+            const double prev = __shfl_up_sync(0xffffffffu, r, 1);
+            if (b < nblk) carry[b] = threadIdx.x == 0 ? run : prev;
+            run = next;
         }
     }
     __syncthreads();
@@ -1808,10 +1854,10 @@ cudaError_t launch_resample_index(const double* W, int64_t N, double* cum, int32
 {
     const int64_t chunks = (N + RS_BLOCK - 1) / RS_BLOCK;
     const unsigned local_grid = (unsigned)((chunks + RS_CHUNKS - 1) / RS_CHUNKS);
-    cudaError_t e = launch_pdl(k_resample_local, dim3(local_grid), dim3(RS_LOCAL_THREADS), RS_LOCAL_SMEM, st, W, N, cum,
+    cudaError_t e = launch_pdl(k_resample_local, dim3(local_grid), dim3(32 * RS_CHUNKS), (size_t)0, st, W, N, cum,
                                flag);
     if (e == cudaSuccess)
-        e = launch_pdl(k_resample_carry, dim3(1), dim3(RS_CARRY_THREADS), (size_t)0, st, N, cum, flag, t, seed,
+        e = launch_pdl(k_resample_carry, dim3(1), dim3(32), (size_t)0, st, N, cum, flag, t, seed,
                        u_override);
     if (e == cudaSuccess)
         e = launch_pdl(k_resample_search, dim3(elem_grid(N)), dim3(256), (size_t)0, st, cum, N, idx, flag);
@@ -1827,7 +1873,7 @@ cudaError_t launch_resample_gather(const double* W, int64_t N, double* cum, cons
 {
     const int64_t chunks = (N + RS_BLOCK - 1) / RS_BLOCK;
     const cudaError_t e = launch_pdl(k_resample_local, dim3((unsigned)((chunks + RS_CHUNKS - 1) / RS_CHUNKS)),
-                                     dim3(RS_LOCAL_THREADS), RS_LOCAL_SMEM, st, W, N, cum, flag);
+                                     dim3(32 * RS_CHUNKS), (size_t)0, st, W, N, cum, flag);
     if (e != cudaSuccess) return e;
     const dim3 grid(warps_grid(N)), block(BLOCK);
     if ((p & 3) == 0)

@@ -108,3 +108,22 @@ def test_summary_kernels_give_the_same_values(spa, N):
     assert np.array_equal(out[0]["conc"], out[1]["conc"][:, :, 1:3])
     q = out[1]["quantile"]
     assert np.all(np.diff(q, axis=2) >= 0.0)
+
+
+# Running sums of the weights: 32 at a time by a scan over integers where the sum keeps its
+# exponent, FP64 additions elsewhere; ties, subnormals, jumps of scale, block and group edges.
+@pytest.mark.parametrize("kind", ["equal", "thirds", "powers", "ties", "lognormal", "subnormal", "last", "zeros"])
+@pytest.mark.parametrize("N", [1, 31, 33, 256, 257, 8191, 16384, 16385, 70001])
+def test_resampling_sums_are_the_additions_in_order(spa, kind, N):
+    rng = np.random.default_rng(N)
+    W = {"equal": lambda: np.full(N, 1.0 / N), "thirds": lambda: np.full(N, 1.0 / 3.0),
+         "powers": lambda: 2.0 ** -rng.integers(0, 60, N),
+         "ties": lambda: 2.0 ** -rng.integers(0, 56, N) * (1.0 + 2.0 ** -52 * rng.integers(0, 4, N)),
+         "lognormal": lambda: np.exp(rng.normal(0.0, 8.0, N)),
+         "subnormal": lambda: rng.integers(0, 1 << 20, N) * 5e-324,
+         "last": lambda: np.where(np.arange(N) == N - 1, 1.0, 1e-300),
+         "zeros": lambda: rng.random(N) * (rng.random(N) < 0.02) + np.where(np.arange(N) == 0, 1e-3, 0.0)}[kind]()
+    if kind not in ("subnormal", "thirds"):
+        W = W / W.sum()
+    for u in (0.0, 0.37, 0.999):
+        assert np.array_equal(spa.resample_systematic(W, u), oracle.resample_systematic(W, u))
