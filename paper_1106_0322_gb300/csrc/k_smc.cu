@@ -116,6 +116,85 @@ __device__ __forceinline__ void gather_partials(const MhState& s, int64_t N, Par
     sh.v[slice][k] = make_float2(L.s, L.c);
 }
 
+// The same for the residuals' chunk sums of a gradient evaluation, into one sum a particle: the 32
+// slices in order, by the first threads of the block. Two barriers after the caller's gather.
+struct RsumSlices {
+    float2 v[32][WARPS];
+    float sum[WARPS];
+};
+__device__ __forceinline__ void gather_rsum(const MhState& s, const GradParts& gp, int64_t N, RsumSlices& sh)
+{
+    const int k = threadIdx.x % WARPS, slice = threadIdx.x / WARPS;
+    const int64_t i = (int64_t)blockIdx.x * WARPS + k;
+    FSum r;
+    if (i < N)
+        for (int q = slice; q < s.n_parts; q += 32) r.add(gp.rsum[(int64_t)q * s.ld_part + i]);
+    sh.v[slice][k] = make_float2(r.s, r.c);
+}
+__device__ __forceinline__ void sum_rsum(RsumSlices& sh)
+{
+    if (threadIdx.x < WARPS) {
+        FSum r;
+#pragma unroll
+        for (int k = 0; k < 32; ++k) {
+            const float2 v = sh.v[k][threadIdx.x];
+            r.add(v.x);
+            r.c += v.y;
+        }
+        sh.sum[threadIdx.x] = (float)r.value();
+    }
+    __syncthreads();
+}
+
+// grad l of four coordinates of particle i, `stride` apart from j0 (those beyond p are 0), as
+// k_grad_finish forms it (rs: the sum of its residuals). The products are rounded by themselves:
+// what is added to them does not join in. Two K-split partials of each at a time are in flight.
+template <int STRIDE>
+__device__ __forceinline__ void finish_gradient4(const MoveArgs& a, int64_t i, int p, int j0, float rs, float (&out)[4])
+{
+    const GradParts& gp = a.gp;
+    const int64_t step = a.mh.ld_part * p;
+    const float* c = gp.gpart + i * p + j0;
+    FSum g[4];
+    for (int q = 0; q < gp.ksplit; q += 2, c += 2 * step) {
+        float x[2][4];
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+            const bool in = q + u < gp.ksplit;
+            if (STRIDE == 1) {
+                const float4 v = in ? ld4(c + u * step) : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+                for (int k = 0; k < 4; ++k) x[u][k] = comp(v, k);
+            } else {
+#pragma unroll
+                for (int k = 0; k < 4; ++k) x[u][k] = in && j0 + STRIDE * k < p ? c[u * step + STRIDE * k] : 0.0f;
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < 2; ++u)
+#pragma unroll
+            for (int k = 0; k < 4; ++k) g[k].add(x[u][k]);
+    }
+    float m[4], d[4];
+    if (STRIDE == 1) {
+        const float4 m4 = ldg4(a.mean_f + j0), d4 = ldg4(gp.inv_sd + j0);
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            m[k] = comp(m4, k);
+            d[k] = comp(d4, k);
+        }
+    } else {
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const bool in = j0 + STRIDE * k < p;
+            m[k] = in ? a.mean_f[j0 + STRIDE * k] : 0.0f;
+            d[k] = in ? gp.inv_sd[j0 + STRIDE * k] : 0.0f;
+        }
+    }
+#pragma unroll
+    for (int k = 0; k < 4; ++k) out[k] = __fmul_rn(fmaf(-m[k], rs, (float)g[k].value()), d[k]);
+}
+
 // The proposal's log-likelihood pair: the warp sums the slices, then adds y . eta.
 __device__ __forceinline__ FSum proposal_loglik(const MhState& s, const PartSlices& sh, int64_t i, int lane)
 {
@@ -350,15 +429,25 @@ __global__ void __launch_bounds__(BLOCK, 5) k_move_rw(MoveArgs a, int64_t N, int
 // with float4 loads; else coordinates l, l + 32, ...
 template <bool VEC>
 __device__ __forceinline__ FSum mala_reverse(const MoveArgs& a, int64_t i, int p, int lane, float h2, float a1, float ac,
-                                             float inv_c, int de)
+                                             float inv_c, int de, float rs)
 {
     FSum bwd;
+    const bool parts = a.gp.gpart != nullptr;
     const float* b0 = a.beta + i * p;
     const float* b1 = a.beta_p + i * p;
-    const float* g1 = a.gl_p + i * p;
+    float* g1 = a.gl_p + i * p;
     if (VEC) {
         for (int j0 = 4 * lane; j0 < p; j0 += 128) {
-            const float4 x0 = ld4(b0 + j0), x1 = ld4(b1 + j0), gg = ld4(g1 + j0);
+            const float4 x0 = ld4(b0 + j0), x1 = ld4(b1 + j0);
+            float4 gg;
+            if (parts) {
+                float o[4];
+                finish_gradient4<1>(a, i, p, j0, rs, o);
+                gg = make_float4(o[0], o[1], o[2], o[3]);
+                st4(g1 + j0, gg);
+            } else {
+                gg = ld4(g1 + j0);
+            }
             const float4 Dv = ldg4(a.sigma + j0), iD = ldg4(a.inv_D + j0);
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
@@ -368,10 +457,25 @@ __device__ __forceinline__ FSum mala_reverse(const MoveArgs& a, int64_t i, int p
             }
         }
     } else {
-        for (int j = lane; j < p; j += 32) {
-            const float drift = h2 * a.sigma[j] * (g1[j] + dlogprior(b1[j], a1, ac, inv_c, de));
+        auto term = [&](int j, float gg) {
+            const float drift = h2 * a.sigma[j] * (gg + dlogprior(b1[j], a1, ac, inv_c, de));
             const float d = (b0[j] - b1[j]) - drift;
             bwd.add(d * d * a.inv_D[j]);
+        };
+        if (parts) {
+            for (int j0 = lane; j0 < p; j0 += 128) {
+                float g4[4];
+                finish_gradient4<32>(a, i, p, j0, rs, g4);
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    const int j = j0 + 32 * k;
+                    if (j >= p) break;
+                    g1[j] = g4[k];
+                    term(j, g4[k]);
+                }
+            }
+        } else {
+            for (int j = lane; j < p; j += 32) term(j, g1[j]);
         }
     }
     return bwd;
@@ -395,6 +499,7 @@ __global__ void __launch_bounds__(BLOCK, 4) k_move_mala(MoveArgs a, int64_t N, i
 {
     __shared__ int accw[BLOCK / 32];
     __shared__ PartSlices parts;
+    __shared__ RsumSlices rsum;
     const int64_t i = warp_global_id();
     const int lane = threadIdx.x & 31, groups = (p + 3) >> 2;
     float4 z4 = make_float4(0.f, 0.f, 0.f, 0.f);  // (as in k_move_rw)
@@ -403,7 +508,9 @@ __global__ void __launch_bounds__(BLOCK, 4) k_move_mala(MoveArgs a, int64_t N, i
     grid_launch_dependents();
     if (DECIDE) {
         gather_partials(a.mh, N, parts);
+        if (a.gp.gpart) gather_rsum(a.mh, a.gp, N, rsum);
         __syncthreads();
+        if (a.gp.gpart) sum_rsum(rsum);
     }
     const float4 sk = stepk[t];
     bool acc = false;
@@ -413,7 +520,7 @@ __global__ void __launch_bounds__(BLOCK, 4) k_move_mala(MoveArgs a, int64_t N, i
         const float h = *a.h, h2 = 0.5f * h * h;
         const float* D = a.sigma;
         if (DECIDE) {
-            const FSum bwd = warp_sum(mala_reverse<VEC>(a, i, p, lane, h2, a1, ac, inv_c, pr.de));
+            const FSum bwd = warp_sum(mala_reverse<VEC>(a, i, p, lane, h2, a1, ac, inv_c, pr.de, rsum.sum[threadIdx.x >> 5]));
             const float2 fw = a.fwd[i];
             const float extra = -((bwd.s - fw.x) + (bwd.c - fw.y)) / (2.0f * h * h);
             acc = mh_decide(a.mh, parts, i, lane, sk.y, extra, m_prev, err);
@@ -513,14 +620,14 @@ __global__ void __launch_bounds__(BLOCK, 4) k_move_mala(MoveArgs a, int64_t N, i
 // proposals (and their gradients) are copied into the state rows, so that between steps
 // beta and gl hold the particles.
 template <bool MALA, bool VEC>
-__device__ __forceinline__ bool commit_test(const MoveArgs& a, const PartSlices& parts, int64_t i, int p, int lane, PriorArgs pr,
+__device__ __forceinline__ bool commit_test(const MoveArgs& a, const PartSlices& parts, const RsumSlices& rsum, int64_t i, int p, int lane, PriorArgs pr,
                                             float4 sk, uint32_t m_prev, uint32_t* err)
 {
     float extra = 0.0f;
     if (MALA) {
         const float ac = sk.x, a1 = pr.a + 1.0f, inv_c = sk.z;
         const float h = *a.h, h2 = 0.5f * h * h;
-        const FSum bwd = warp_sum(mala_reverse<VEC>(a, i, p, lane, h2, a1, ac, inv_c, pr.de));
+        const FSum bwd = warp_sum(mala_reverse<VEC>(a, i, p, lane, h2, a1, ac, inv_c, pr.de, rsum.sum[threadIdx.x >> 5]));
         const float2 fw = a.fwd[i];
         extra = -((bwd.s - fw.x) + (bwd.c - fw.y)) / (2.0f * h * h);
     }
@@ -550,15 +657,18 @@ __global__ void __launch_bounds__(BLOCK) k_move_commit(MoveArgs a, int64_t N, in
 {
     __shared__ int accw[BLOCK / 32];
     __shared__ PartSlices parts;
+    __shared__ RsumSlices rsum;
     grid_dependency_wait();
     gather_partials(a.mh, N, parts);
+    if (MALA && a.gp.gpart) gather_rsum(a.mh, a.gp, N, rsum);
     __syncthreads();
+    if (MALA && a.gp.gpart) sum_rsum(rsum);
     const float4 sk = stepk[t];
     const int64_t i = warp_global_id();
     const int lane = threadIdx.x & 31;
     bool acc = false;
     if (i < N) {
-        acc = commit_test<MALA, VEC>(a, parts, i, p, lane, pr, sk, m_prev, err);
+        acc = commit_test<MALA, VEC>(a, parts, rsum, i, p, lane, pr, sk, m_prev, err);
         if (acc) commit_row<MALA, VEC>(a, i, p, lane);
     }
     if (lane == 0) accw[threadIdx.x >> 5] = acc ? 1 : 0;
@@ -657,10 +767,13 @@ __global__ void __launch_bounds__(BLOCK) k_commit_reweight(MoveArgs a, int64_t N
     static_assert(RW_PER_BLOCK == WARPS, "one warp per particle in both halves");
     __shared__ int accw[BLOCK / 32];
     __shared__ PartSlices parts;
+    __shared__ RsumSlices rsum;
     __shared__ float4 sums[RW_PER_BLOCK];
     grid_dependency_wait();
     gather_partials(a.mh, N, parts);
+    if (MALA && a.gp.gpart) gather_rsum(a.mh, a.gp, N, rsum);
     __syncthreads();
+    if (MALA && a.gp.gpart) sum_rsum(rsum);
     const float4 sk = stepk[t];
     const ReweightK rk = rkp[t + 1];
     const int64_t i = warp_global_id();
@@ -668,7 +781,7 @@ __global__ void __launch_bounds__(BLOCK) k_commit_reweight(MoveArgs a, int64_t N
     bool acc = false;
     FSum sdiff, snew;
     if (i < N) {
-        acc = commit_test<MALA, VEC>(a, parts, i, p, lane, pr, sk, m_prev, err);
+        acc = commit_test<MALA, VEC>(a, parts, rsum, i, p, lane, pr, sk, m_prev, err);
         if (acc) commit_row<MALA, VEC>(a, i, p, lane);
         reweight_row((acc ? a.beta_p : a.beta) + i * p, p, pr, rk, lane, sdiff, snew);
     }

@@ -690,8 +690,17 @@ TcMaps maps_of(const spa_ctx* c)
     return m;
 }
 
+// Whether the kernel that tests a sweep's MALA proposals also forms their gradient from the
+// contraction's partials (GradParts), one kernel and one pass over the rows less, instead of
+// launch_grad_finish before it. Step of 5 moves, before and after: n = 2000, p = 200, N = 8192 352 ->
+// 344 us; n = 1234, p = 77, N = 4096 176 -> 172. Without 16-byte groups a lane's reads of the
+// partials come one coordinate at a time, and from a second batch of 128 on that costs more than the
+// kernel (5 moves at n = 1200, p = 207, N = 2048: 200 -> 213 us; p = 239: 213 -> 226).
+bool test_forms_gradient(int p) { return p % 4 == 0 || p <= 128; }
+
 // The adjoint's second half after a residual likelihood pass: C = R G, then the gradient.
-void enq_grad_tail(Enq& q, float* out, const float* Bsrc, double cs, int64_t N)
+// (finish: into `out`; else the kernel that tests the proposals forms it, grad_parts)
+void enq_grad_tail(Enq& q, float* out, const float* Bsrc, double cs, int64_t N, bool finish = true)
 {
     spa_ctx* c = q.c;
     Workspace& w = c->ws;
@@ -701,11 +710,12 @@ void enq_grad_tail(Enq& q, float* out, const float* Bsrc, double cs, int64_t N)
     const AdjPlan a = adj_plan((int)c->p, c->n, w.N_pad, c->num_sms);
     q.ck(launch_adjoint_tc(w.mapR, c->mapGT, a, (int)c->p, w.gpart, w.N_pad, c->d_err, q.st, c->wait_ns,
                            c->plan_sms > 0 ? c->plan_sms : 0, /*r_last_use_hint=*/c->plan_sms == 0));
-    q.ck(launch_grad_finish(w.gpart, a.ksplit, w.rsum, plan.n_parts, w.N_pad, N, (int)c->p, c->mean_f, c->colf, Bsrc,
+    if (finish)
+        q.ck(launch_grad_finish(w.gpart, a.ksplit, w.rsum, plan.n_parts, w.N_pad, N, (int)c->p, c->mean_f, c->colf, Bsrc,
                             c->pr, cs, out, q.st));
 }
 
-void enq_grad_tc(Enq& q, float* out, const float* Bsrc, double cs, int64_t N)
+void enq_grad_tc(Enq& q, float* out, const float* Bsrc, double cs, int64_t N, bool finish = true)
 {
     spa_ctx* c = q.c;
     Workspace& w = c->ws;
@@ -733,14 +743,15 @@ void enq_grad_tc(Enq& q, float* out, const float* Bsrc, double cs, int64_t N)
         g.wait_ns = c->wait_ns;
         g.stall = c->fault & FAULT_STALL;
         q.ck(launch_grad_tc(w.mapA, w.mapAt, m, gp, a, g, q.st));
-        q.ck(launch_grad_finish(w.gpart, a.ksplit, w.rsum, (int)((c->n + 31) / 32), w.N_pad, N, (int)c->p, c->mean_f, c->colf,
+        if (finish)
+            q.ck(launch_grad_finish(w.gpart, a.ksplit, w.rsum, (int)((c->n + 31) / 32), w.N_pad, N, (int)c->p, c->mean_f, c->colf,
                                 Bsrc, c->pr, cs, out, q.st));
         return;
     }
     ResidArgs ra{w.R, a.n_r, w.rsum};
     q.ck(launch_loglik_tc(maps_of(c), plan_of(c), c->n, c->Kp, c->ybits, w.partial, w.N_pad, c->d_err, q.st, &ra,
                           c->wait_ns, c->fault & FAULT_STALL));
-    enq_grad_tail(q, out, Bsrc, cs, N);
+    enq_grad_tail(q, out, Bsrc, cs, N, finish);
 }
 
 // log-likelihood of the current proposals (beta_p) into the partial sums
@@ -799,6 +810,10 @@ MoveArgs move_args(spa_ctx* c, unsigned long long* acc)
     a.mh = mh_state(c, acc);
     a.gl = w.gl;
     a.gl_p = w.gl_p;
+    if (tc && w.gpart && test_forms_gradient((int)c->p)) {
+        const AdjPlan ap = adj_plan((int)c->p, c->n, w.N_pad, c->num_sms);
+        a.gp = GradParts{w.gpart, w.rsum, c->colf, ap.ksplit};
+    }
     a.fwd = w.fwd;
     a.h = w.h;
     return a;
@@ -869,7 +884,7 @@ void enq_likelihood(Enq& q, const LikPoint& lp)
     float* out = lp.init ? w.gl : w.gl_p;
     const float* src = lp.init ? w.beta : w.beta_p;
     if (mala && c->cfg.precision == SPA_PREC_SPLIT_BF16) {
-        enq_grad_tc(q, out, src, 0.0, w.N);  // also leaves the softplus partials
+        enq_grad_tc(q, out, src, 0.0, w.N, lp.init || !test_forms_gradient((int)c->p));  // also leaves the softplus partials
         return;
     }
     enq_loglik(q);
@@ -1387,7 +1402,8 @@ cudaError_t batch_capture_lockstep(spa_batch* b, const spa_batch_args* args)
             e = cudaStreamWaitEvent(qs[(size_t)r].st, b->ev_grouped, 0);
             if (e == cudaSuccess && mala) {
                 Workspace& w = b->ctxs[r]->ws;
-                enq_grad_tail(qs[(size_t)r], lp.init ? w.gl : w.gl_p, lp.init ? w.beta : w.beta_p, 0.0, w.N);
+                enq_grad_tail(qs[(size_t)r], lp.init ? w.gl : w.gl_p, lp.init ? w.beta : w.beta_p, 0.0, w.N,
+                              lp.init || !test_forms_gradient((int)b->ctxs[r]->p));
                 e = qs[(size_t)r].e;
             }
         }

@@ -103,6 +103,16 @@ struct ResampledState {
     uint32_t wf = 0;
 };
 
+// A gradient evaluation of the proposals as its contraction leaves it: the K-split partials of
+// C = R G and the residuals' chunk sums, from which the kernel that tests the proposals forms
+// grad l (finish_gradient4) on the way.
+struct GradParts {
+    const float* gpart = nullptr;   // [ksplit][N_pad][p]; NULL: the gradient's rows are in gl_p
+    const float* rsum = nullptr;    // [n_parts][N_pad], as the softplus partials
+    const float* inv_sd = nullptr;
+    int ksplit = 0;
+};
+
 struct MoveArgs {
     float* beta;                 // particle states
     float* beta_p;               // proposals
@@ -119,7 +129,8 @@ struct MoveArgs {
     MhState mh;
     // MALA only
     float* gl;                   // grad l of the states
-    const float* gl_p;           // grad l of the proposals
+    float* gl_p;                 // grad l of the proposals
+    GradParts gp;                // where the test of the proposals finds it, if not there
     float2* fwd;                 // forward-move residual sum of the proposals
     const float* h;              // step size
     ResampledState rs;           // a step's first move only

@@ -127,3 +127,21 @@ def test_resampling_sums_are_the_additions_in_order(spa, kind, N):
         W = W / W.sum()
     for u in (0.0, 0.37, 0.999):
         assert np.array_equal(spa.resample_systematic(W, u), oracle.resample_systematic(W, u))
+
+
+# The kernel that tests a MALA proposal forms its gradient from the contraction's K-split partials
+# for p % 4 == 0 (groups of 4) and p <= 128 (4 coordinates 32 apart); other p take the finish kernel.
+@pytest.mark.parametrize("n,p", [(40, 1), (100, 3), (129, 4), (300, 31), (400, 33), (800, 97), (1500, 127), (2100, 128),
+                                 (700, 129), (600, 132), (900, 252), (500, 256), (500, 260)])
+def test_mala_gradient_formed_where_it_is_tested(spa, n, p):
+    """One seed, so the same proposals on both sides: the first step's decisions differ where a log
+    ratio lies within the split product's rounding of log U (a few 1e-3 at most): about 0.3 of 256
+    proposals are expected to, 4 are allowed, each moving a particle's coordinates by less than 1."""
+    N, M = 128, 2
+    reg = synth.make_region(n, p, 0.9, (0.5,), seed=1700 + n)
+    sched = synth.geometric_schedule(2, -3.0, -2.0)
+    with spa.Region(reg.G, reg.y, 2.0, config=spa.make_config(move="mala", init="resample_move")) as r:
+        g = r.run(sched, N, M, 9)
+    o = oracle.run(reg.G, reg.y, 2.0, sched, N, M, seed=9, cfg=oracle.make_config(move="mala", init="mcmc"))
+    assert abs(g["accept_rate"][0] - o["accept_rate"][0]) <= 4.0 / (N * M) + 1e-12
+    assert np.max(np.abs(g["mean"][0] - o["mean"][0])) <= 4.0 / N + 1e-4
