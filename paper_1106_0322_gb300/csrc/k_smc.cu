@@ -68,17 +68,26 @@ __device__ __forceinline__ float pack_coord(__nv_bfloat16* __restrict__ Arow, in
     return mean_f[j] * bt;
 }
 
+__device__ __forceinline__ uint32_t bf16x2_bits(float lo, float hi)
+{
+    const __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);
+    return *reinterpret_cast<const uint32_t*>(&v);
+}
+
 // Four consecutive coordinates j..j+3 (j a multiple of 4): two 8-byte stores per half.
 __device__ __forceinline__ float pack_coord4(__nv_bfloat16* __restrict__ Arow, int Kp, int j, float4 b, float4 l2e,
                                              float4 mf)
 {
     const float bt[4] = {b.x * l2e.x, b.y * l2e.y, b.z * l2e.z, b.w * l2e.w};
-    __align__(8) __nv_bfloat16 hi[4];
-    __align__(8) __nv_bfloat16 lo[4];
+    // split_bf16, two at a time: a pair's BF16 values as FP32 are the word's halves shifted up
+    uint32_t hi[2], lo[2];
 #pragma unroll
-    for (int k = 0; k < 4; ++k) split_bf16(bt[k], hi[k], lo[k]);
-    *reinterpret_cast<uint2*>(Arow + j) = *reinterpret_cast<const uint2*>(hi);
-    *reinterpret_cast<uint2*>(Arow + Kp + j) = *reinterpret_cast<const uint2*>(lo);
+    for (int k = 0; k < 2; ++k) {
+        hi[k] = bf16x2_bits(bt[2 * k], bt[2 * k + 1]);
+        lo[k] = bf16x2_bits(bt[2 * k] - __uint_as_float(hi[k] << 16), bt[2 * k + 1] - __uint_as_float(hi[k] & 0xFFFF0000u));
+    }
+    *reinterpret_cast<uint2*>(Arow + j) = make_uint2(hi[0], hi[1]);
+    *reinterpret_cast<uint2*>(Arow + Kp + j) = make_uint2(lo[0], lo[1]);
     return mf.x * bt[0] + mf.y * bt[1] + mf.z * bt[2] + mf.w * bt[3];
 }
 

@@ -52,8 +52,14 @@ __device__ __forceinline__ uint2 seed_key(uint64_t seed)
     return make_uint2((uint32_t)seed, (uint32_t)(seed >> 32));
 }
 
-// (k + 1/2) 2^-23, k = top 23 bits: exact in single precision, in (0,1).
-__device__ __forceinline__ float u01_open_f(uint32_t u) { return ((float)(u >> 9) + 0.5f) * 1.1920928955078125e-7f; }
+// (k + 1/2) 2^-23, k = top 23 bits: exact in single precision, in (0,1). As 1 + k 2^-23, whose bits are
+// those of 1 with k in the mantissa, less 1 - 2^-24 (exact: the difference has 24 bits); no
+// conversion, which the units for logarithms and roots would have to make. With the packed split of
+// pack_coord4, the RW move kernel at p = 200, N = 8192: 1233 -> 1148 instructions a warp, 16.6 -> 15.7 us
+// alone.
+__device__ __forceinline__ float u01_open_f(uint32_t u) { return __uint_as_float((u >> 9) + 0x3F800000u) - 0.999999940395355224609375f; }
+// twice that, in (0,2)
+__device__ __forceinline__ float u02_open_f(uint32_t u) { return __uint_as_float((u >> 9) + 0x40000000u) - 1.99999988079071044921875f; }
 __device__ __forceinline__ double u01_open_d(uint32_t u) { return ((double)(u >> 9) + 0.5) * 1.1920928955078125e-7; }
 // top 24 bits / 2^24 in [0,1)
 __device__ __forceinline__ double u01_d(uint32_t u) { return (double)(u >> 8) * 5.9604644775390625e-8; }
@@ -65,8 +71,8 @@ __device__ __forceinline__ float4 normals4(uint64_t seed, uint32_t blk, uint32_t
     float s0, c0, s1, c1;
     const float r0 = sqrtf(-2.0f * logf(u01_open_f(u.x)));
     const float r1 = sqrtf(-2.0f * logf(u01_open_f(u.z)));
-    sincospif(2.0f * u01_open_f(u.y), &s0, &c0);
-    sincospif(2.0f * u01_open_f(u.w), &s1, &c1);
+    sincospif(u02_open_f(u.y), &s0, &c0);
+    sincospif(u02_open_f(u.w), &s1, &c1);
     return make_float4(r0 * c0, r0 * s0, r1 * c1, r1 * s1);
 }
 
