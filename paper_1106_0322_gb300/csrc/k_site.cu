@@ -101,9 +101,9 @@ __global__ void __launch_bounds__(32 * SITE_WARPS, site_min_blocks(KC))
                 const uint4 u = philox4x32_10(make_uint4((uint32_t)jl, (uint32_t)i, (uint32_t)t, (TAG_SITE << 16) | m),
                                               seed_key(seed));
                 float sn, cs;
-                sincospif(2.0f * u01_open_f(u.y), &sn, &cs);
-                const float delta_l = __fmul_rn(a.sd, __fmul_rn(sqrtf(-2.0f * logf(u01_open_f(u.x))), cs));
-                const float lu_l = logf(u01_open_f(u.z));
+                sincospif(2.0f * u01_open_cvt_f(u.y), &sn, &cs);
+                const float delta_l = __fmul_rn(a.sd, __fmul_rn(sqrtf(-2.0f * logf(u01_open_cvt_f(u.x))), cs));
+                const float lu_l = logf(u01_open_cvt_f(u.z));
                 const float b0 = in ? bg[jl] : 0.0f, v_l = in ? a.vy[jl] : 0.0f;
                 const float b1 = __fadd_rn(b0, delta_l);
                 const float dq_l = prior_term(b1, inv_ac, pr.de) - prior_term(b0, inv_ac, pr.de);
@@ -264,15 +264,15 @@ __global__ void k_move_site(SiteArgs a, int64_t N, int p, int n, PriorArgs pr, c
                 const uint4 u = philox4x32_10(make_uint4((uint32_t)j, (uint32_t)i, (uint32_t)t, (TAG_SITE << 16) | m),
                                               seed_key(seed));
                 float sn, cs;
-                sincospif(2.0f * u01_open_f(u.y), &sn, &cs);
-                const float delta = a.sd * (sqrtf(-2.0f * logf(u01_open_f(u.x))) * cs);
+                sincospif(2.0f * u01_open_cvt_f(u.y), &sn, &cs);
+                const float delta = a.sd * (sqrtf(-2.0f * logf(u01_open_cvt_f(u.x))) * cs);
                 const float* xr = a.XT2 + (size_t)j * n;
                 const float lq1 = site_trial(eta, xr, n, lane, delta, dm);
                 const float dsp = warp_sum(dm + (lq1 - lq));
                 const float b0 = brow[j], b1 = b0 + delta;
                 const float dlp = coef * (prior_term(b1, inv_ac, pr.de) - prior_term(b0, inv_ac, pr.de));
                 const float dl = fmaf(delta, a.vy[j], -0.69314718f * dsp);
-                int acc = logf(u01_open_f(u.z)) < dl + dlp;
+                int acc = logf(u01_open_cvt_f(u.z)) < dl + dlp;
                 acc = __shfl_sync(0xffffffffu, acc, 0);
                 if (acc) {
                     for (int r = lane; r < n; r += 32) eta[r] = fmaf(xr[r], delta, eta[r]);
