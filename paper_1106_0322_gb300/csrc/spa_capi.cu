@@ -721,8 +721,9 @@ void enq_grad_tc(Enq& q, float* out, const float* Bsrc, double cs, int64_t N, bo
     Workspace& w = c->ws;
     const AdjPlan a = adj_plan((int)c->p, c->n, w.N_pad, c->num_sms);
     GradPlan gp;
-    // (a batch's regions, on a share of the SMs each, keep the two kernels: CTAs that loop over many
-    // units wait for each unit's C to leave, 76 against 67 ms for a batch of 8 regions)
+    // (a batch's regions, on a share of the SMs each, keep the two kernels: a fused CTA holds its SM for
+    // all its units, and with uneven regions the small ones' keep the largest, which the batch waits
+    // for, off the SMs: 52 against 49 ms for 8 regions of n = 1000..5000, p = 20..500)
     if (c->plan_sms == 0 && grad_tc_plan(gp, c->n, (int)c->p, a, c->num_sms)) {
         GradMaps m;
         if (!grad_tc_make_maps(m, c->Gbf, c->GT, c->n, (int)c->p, c->Kp, a.n_r, gp)) {
@@ -1250,15 +1251,32 @@ void batch_free(spa_batch* b)
 // the 64-region batched workload that measures 1.84 s per batch against 2.26 s in lock step,
 // whose joins at every evaluation stop the regions' other kernels from overlapping.
 // The SMs each region's likelihood launches are sized for when a batch runs its regions as
-// graph branches side by side: an eighth of the GPU once 8 or more regions share it, else
-// an equal share. Smaller grids give each CTA more units (the per-CTA set-up and last
-// epilogue are paid fewer times over the batch's work), while the other regions' branches
-// keep the SMs busy. The likelihood partials are per 32 individuals whatever the grid, so
-// the batch's results stay bit-identical to single runs.
-int batch_plan_sms(int num_sms, int32_t R)
+// graph branches side by side: shares in proportion to the regions' work, twice the GPU in all
+// (an eighth of it a region on average from 16 regions on). Smaller grids give each CTA more units
+// (the per-CTA set-up and last epilogue are paid fewer times over the batch's work), while the
+// other branches keep the SMs busy; but a batch ends with its slowest region, and with equal
+// shares the largest of uneven ones went on alone on its few SMs. Work: evaluations x N n (p + 256),
+// the constant for the epilogue's share of a unit. Against equal shares of the GPU (MALA, N = 4096,
+// 20 steps of 5, n = 1000..5000, p = 20..500): 8 regions 62.6 -> 48.5 ms (once the GPU in all: 58; four
+// times: 51), 24 regions and 5 steps 37.4 -> 37.2, 8 equal ones 17.0 -> 16.4. The likelihood partials
+// are per 32 individuals whatever the grid, so the batch's results stay bit-identical to single runs.
+std::vector<int> batch_plan_sms(const spa_batch* b, const spa_batch_args* args)
 {
-    const int share = R > 0 ? num_sms / (R < 8 ? R : 8) : num_sms;
-    return share > 0 ? share : 1;
+    const size_t R = b->ctxs.size();
+    std::vector<double> work(R);
+    double total = 0.0;
+    for (size_t r = 0; r < R; ++r) {
+        const spa_ctx* c = b->ctxs[r];
+        work[r] = (double)b->T[r] * (1.0 + args->moves_per_step[r]) * (double)c->ws.N * (double)c->n * ((double)c->p + 256.0);
+        total += work[r];
+    }
+    std::vector<int> sms(R);
+    for (size_t r = 0; r < R; ++r) {
+        const int num = b->ctxs[r]->num_sms;
+        const double share = num * std::max(2.0, (double)R / 8.0) * work[r] / std::max(total, 1.0);
+        sms[r] = (int)std::min((double)num, std::max(1.0, std::round(share)));
+    }
+    return sms;
 }
 
 bool batch_lockstep(spa_ctx* const* ctxs, int32_t R, const spa_batch_args* args)
@@ -1486,11 +1504,12 @@ int batch_build(spa_batch* b, spa_ctx* const* ctxs, int32_t R, const spa_batch_a
         for (int32_t r = 0; r < R && ee == cudaSuccess; ++r) ee = cudaStreamWaitEvent(b->ctxs[r]->stream(), b->fork, 0);
         if (ee == cudaSuccess) ee = batch_capture_lockstep(b, args);
     } else {
+        const std::vector<int> sms = batch_plan_sms(b, args);
         for (int32_t r = 0; r < R && ee == cudaSuccess; ++r) {
             spa_ctx* c = b->ctxs[r];
             ee = cudaStreamWaitEvent(c->stream(), b->fork, 0);
             if (ee != cudaSuccess) break;
-            c->plan_sms = batch_plan_sms(c->num_sms, R);  // only while this batch's graph is captured
+            c->plan_sms = sms[(size_t)r];  // only while this batch's graph is captured
             const int64_t n = enqueue_sweep(c, b->T[r], args->moves_per_step[r], &ee);
             c->plan_sms = 0;
             b->per_ctx_launches.push_back(n);

@@ -145,3 +145,22 @@ def test_mala_gradient_formed_where_it_is_tested(spa, n, p):
     o = oracle.run(reg.G, reg.y, 2.0, sched, N, M, seed=9, cfg=oracle.make_config(move="mala", init="mcmc"))
     assert abs(g["accept_rate"][0] - o["accept_rate"][0]) <= 4.0 / (N * M) + 1e-12
     assert np.max(np.abs(g["mean"][0] - o["mean"][0])) <= 4.0 / N + 1e-4
+
+
+# A batch's likelihood launches are sized by the regions' shares of the work (down to one CTA for a
+# small region beside large ones, all SMs for a large one); alone each takes all SMs.
+@pytest.mark.parametrize("move", ["rw", "mala"])
+def test_uneven_batch_shares_give_the_single_runs(spa, move):
+    shapes = [(31, 1, 5, 2), (4000, 200, 9000, 2), (513, 255, 770, 0), (900, 300, 2000, 3), (129, 64, 2600, 1)]
+    sched = synth.geometric_schedule(3, -4.0, -1.0)
+    regs = [synth.make_region(n, p, 0.9, (0.4, -0.3), seed=1800 + n) for n, p, _, _ in shapes]
+    rs = [spa.Region(g.G, g.y, 2.0, config=spa.make_config(move=move)) for g in regs]
+    alone = [r.run(sched, s[2], s[3], 5 + k) for k, (r, s) in enumerate(zip(rs, shapes))]
+    b = spa.Batch(rs, [sched] * 5, [s[2] for s in shapes], [s[3] for s in shapes], [5 + k for k in range(5)])
+    together = b.run()
+    b.close()
+    for one, two in zip(alone, together):
+        for k in one:
+            assert np.array_equal(one[k], two[k]), k
+    for r in rs:
+        r.close()
