@@ -218,6 +218,62 @@ __device__ __forceinline__ FSum proposal_loglik(const MhState& s, const PartSlic
     return L;
 }
 
+// ---- the block's sums at once
+// A block's warps each hold one particle's 32 lane partials of several sums. Reduced by the
+// warp that holds them, a compensated sum is 5 shuffled additions, made by 8 warps for 8
+// sums; here one warp reduces all 8: lane 4 k + s first adds the partials s, s + 4, ... of
+// particle k in the order in which lane s of the warp tree would, then two shuffles end the
+// tree. The lanes 4 k have the results: the bits that lane 0 of warp_sum has.
+constexpr int LANES_LD = WARPS + 1;  // (an odd stride keeps a warp's column off one bank)
+struct LaneSums {
+    float2 v[32][LANES_LD];
+};
+template <int LD>
+__device__ __forceinline__ FSum block_fsum(const float2 (&v)[32][LD])
+{
+    const int lane = threadIdx.x & 31, k = lane >> 2, s = lane & 3;
+    FSum a[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        const float2 x = v[s + 4 * j][k], y = v[s + 4 * j + 16][k];
+        FSum o;
+        a[j].s = x.x;
+        a[j].c = x.y;
+        o.s = y.x;
+        o.c = y.y;
+        a[j].add(o);
+    }
+    a[0].add(a[2]);
+    a[1].add(a[3]);
+    a[0].add(a[1]);
+#pragma unroll
+    for (int o = 2; o > 0; o >>= 1) {
+        FSum w;
+        w.s = __shfl_xor_sync(0xffffffffu, a[0].s, o);
+        w.c = __shfl_xor_sync(0xffffffffu, a[0].c, o);
+        a[0].add(w);
+    }
+    return a[0];
+}
+// The same of two plain sums.
+__device__ __forceinline__ float2 block_sum2(const float2 (&v)[32][LANES_LD])
+{
+    const int lane = threadIdx.x & 31, k = lane >> 2, s = lane & 3;
+    float2 a[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        const float2 x = v[s + 4 * j][k], y = v[s + 4 * j + 16][k];
+        a[j] = make_float2(x.x + y.x, x.y + y.y);
+    }
+    float2 r = make_float2((a[0].x + a[2].x) + (a[1].x + a[3].x), (a[0].y + a[2].y) + (a[1].y + a[3].y));
+#pragma unroll
+    for (int o = 2; o > 0; o >>= 1) {
+        r.x += __shfl_xor_sync(0xffffffffu, r.x, o);
+        r.y += __shfl_xor_sync(0xffffffffu, r.y, o);
+    }
+    return r;
+}
+
 // log U of the MH test of move m for the block's particles (one warp per particle, so
 // blockDim.x / 32 of them), by the kernel that proposes move m: lanes 0.. of warp 0 draw
 // them side by side instead of lane 0 of every warp one at a time in the test.
@@ -235,29 +291,50 @@ __device__ __forceinline__ void draw_accept_logu(const MhState& s, int64_t N, in
 // q-correction. Lane 0 decides with the accept uniform of move m_prev (drawn by the kernel
 // that proposed it) and, on acceptance, moves the proposal's log-likelihood and log-prior
 // into the current state. Returns the decision on every lane.
+__device__ __forceinline__ bool mh_test(const MhState& s, const FSum& L, int64_t i, float coef, float extra, uint32_t m_prev,
+                                        uint32_t* err)
+{
+    const float2 L0 = s.llq[i];
+    const float2 Q1 = s.lpt_p[i], Q0 = s.lpq[i];
+    // written two launches back, by the kernel that proposed (read from L2)
+    const float lu = __ldcg(s.lu + (int64_t)(m_prev & 1u) * s.ld_lu + i);
+    const float dL = (L.s - L0.x) + (L.c - L0.y);
+    const float dQ = (Q1.x - Q0.x) + (Q1.y - Q0.y);
+    // rounded as written (no contraction), so that the decision does not depend on
+    // how the compiler schedules the surrounding code
+    const float log_alpha = __fadd_rn(__fadd_rn(__fmul_rn(s.sp_scale, dL), __fmul_rn(coef, dQ)), extra);
+    if (!isfinite(L.s)) atomicOr(err, DERR_NONFINITE);
+    const bool accept = lu < log_alpha;
+    if (accept) {
+        s.llq[i] = make_float2(L.s, L.c);
+        s.lpq[i] = Q1;
+    }
+    return accept;
+}
 __device__ __forceinline__ bool mh_decide(const MhState& s, const PartSlices& sh, int64_t i, int lane, float coef,
                                           float extra, uint32_t m_prev, uint32_t* err)
 {
     const FSum L = proposal_loglik(s, sh, i, lane);
     int accept = 0;
-    if (lane == 0) {
-        const float2 L0 = s.llq[i];
-        const float2 Q1 = s.lpt_p[i], Q0 = s.lpq[i];
-        // written two launches back, by the kernel that proposed (read from L2)
-        const float lu = __ldcg(s.lu + (int64_t)(m_prev & 1u) * s.ld_lu + i);
-        const float dL = (L.s - L0.x) + (L.c - L0.y);
-        const float dQ = (Q1.x - Q0.x) + (Q1.y - Q0.y);
-        // rounded as written (no contraction), so that the decision does not depend on
-        // how the compiler schedules the surrounding code
-        const float log_alpha = __fadd_rn(__fadd_rn(__fmul_rn(s.sp_scale, dL), __fmul_rn(coef, dQ)), extra);
-        if (!isfinite(L.s)) atomicOr(err, DERR_NONFINITE);
-        accept = lu < log_alpha;
-        if (accept) {
-            s.llq[i] = make_float2(L.s, L.c);
-            s.lpq[i] = Q1;
-        }
-    }
+    if (lane == 0) accept = mh_test(s, L, i, coef, extra, m_prev, err);
     return __shfl_sync(0xffffffffu, accept, 0) != 0;
+}
+// The tests of all the block's particles, by one warp: lane 4 k decides for particle k, into acc[k].
+__device__ __forceinline__ void mh_decide_block(const MhState& s, const PartSlices& sh, int64_t N, float coef, uint32_t m_prev,
+                                                int* acc, uint32_t* err)
+{
+    const int lane = threadIdx.x & 31;
+    const int64_t i = (int64_t)blockIdx.x * WARPS + (lane >> 2);
+    FSum L = block_fsum(sh.v);
+    if (lane & 3) return;
+    int accept = 0;
+    if (i < N) {
+        const float2 yd = s.ydq[i];
+        L.add(yd.x);
+        L.add(yd.y);
+        accept = mh_test(s, L, i, coef, 0.0f, m_prev, err);
+    }
+    acc[lane >> 2] = accept;
 }
 
 
@@ -384,6 +461,8 @@ __global__ void __launch_bounds__(BLOCK, 5) k_move_rw(MoveArgs a, int64_t N, int
 {
     __shared__ int accw[BLOCK / 32];
     __shared__ PartSlices parts;
+    __shared__ LaneSums lts, yos;
+    const int w = threadIdx.x >> 5;
     const int64_t i = warp_global_id();
     const int lane = threadIdx.x & 31, groups = (p + 3) >> 2;
     // The first group's normals depend on nothing that the previous kernel writes: drawn by blocks that
@@ -398,36 +477,47 @@ __global__ void __launch_bounds__(BLOCK, 5) k_move_rw(MoveArgs a, int64_t N, int
         __syncthreads();
     }
     const float4 sk = stepk[t];
+    if (DECIDE) {
+        if (w == 0) mh_decide_block(a.mh, parts, N, sk.y, m_prev, accw, err);
+        __syncthreads();
+    }
+    FSum lt;
+    float yd = 0.0f, off = 0.0f;
     bool acc = false;  // the state is the row in beta_p: an accepted proposal, or a resampled particle
     if (i < N) {
         const uint64_t seed = (noise || DECIDE) ? *seedp : 0ull;
         if (DECIDE)
-            acc = mh_decide(a.mh, parts, i, lane, sk.y, 0.0f, m_prev, err);
+            acc = accw[w] != 0;
         else
             acc = take_resampled(a, i, lane);
         const float* src = (acc ? a.beta_p : a.beta) + i * p;
         float* dst = a.beta_p + i * p;
         float* cur = a.beta + i * p;
         __nv_bfloat16* Arow = a.A ? a.A + i * (int64_t)a.ldA : nullptr;
-        FSum lt;
-        float yd = 0.0f, off = 0.0f;
         for (int g = lane; g < groups; g += 32) {
             if (noise && g >= 32) z = normals4(seed, (uint32_t)g, (uint32_t)i, (uint32_t)t, m);
             rw_group<VEC>(a, p, g, true, acc, noise, z, sk.w, pr.de, src, dst, cur, Arow, lt, yd, off);
         }
-        lt = warp_sum(lt);
-        yd = warp_sum(yd);
-        off = warp_sum(off);
-        if (lane == 0) {
-            a.lpt_p[i] = make_float2(lt.s, lt.c);
-            a.ydq[i] = make_float2(yd, 0.0f);
-            if (Arow) pack_offset(Arow, a.Kp, p, off);
+    }
+    lts.v[lane][w] = make_float2(lt.s, lt.c);
+    yos.v[lane][w] = make_float2(yd, off);
+    __syncthreads();
+    const int64_t ib = (int64_t)blockIdx.x * WARPS + (lane >> 2);
+    const bool mine = (lane & 3) == 0 && ib < N;
+    if (w == 0) {
+        const FSum q = block_fsum(lts.v);
+        if (mine) a.lpt_p[ib] = make_float2(q.s, q.c);
+    } else if (w == 1) {
+        const float2 q = block_sum2(yos.v);
+        if (mine) {
+            a.ydq[ib] = make_float2(q.x, 0.0f);
+            if (a.A) pack_offset(a.A + ib * (int64_t)a.ldA, a.Kp, p, q.y);
         }
     }
     if (noise) draw_accept_logu(a.mh, N, t, m, *seedp);
-    if (DECIDE) {
-        if (lane == 0) accw[threadIdx.x >> 5] = acc ? 1 : 0;
-        count_warps(a.mh.acc_count, accw);
+    if (DECIDE && w == 2) {
+        const int n_acc = __popc(__ballot_sync(0xffffffffu, lane < WARPS && accw[lane % WARPS] != 0));
+        if (lane == 0 && a.mh.acc_count && n_acc) atomicAdd(a.mh.acc_count, (unsigned long long)n_acc);
     }
 }
 
