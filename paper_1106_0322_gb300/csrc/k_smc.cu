@@ -311,28 +311,30 @@ __device__ __forceinline__ bool mh_test(const MhState& s, const FSum& L, int64_t
     }
     return accept;
 }
-__device__ __forceinline__ bool mh_decide(const MhState& s, const PartSlices& sh, int64_t i, int lane, float coef,
-                                          float extra, uint32_t m_prev, uint32_t* err)
-{
-    const FSum L = proposal_loglik(s, sh, i, lane);
-    int accept = 0;
-    if (lane == 0) accept = mh_test(s, L, i, coef, extra, m_prev, err);
-    return __shfl_sync(0xffffffffu, accept, 0) != 0;
-}
 // The tests of all the block's particles, by one warp: lane 4 k decides for particle k, into acc[k].
-__device__ __forceinline__ void mh_decide_block(const MhState& s, const PartSlices& sh, int64_t N, float coef, uint32_t m_prev,
-                                                int* acc, uint32_t* err)
+// MALA: with the lane partials of the reverse moves' residual sums (mala_reverse) in bwd.
+template <bool MALA>
+__device__ __forceinline__ void mh_decide_block(const MoveArgs& a, const PartSlices& sh, const LaneSums& bwd, int64_t N,
+                                                float coef, uint32_t m_prev, int* acc, uint32_t* err)
 {
+    const MhState& s = a.mh;
     const int lane = threadIdx.x & 31;
     const int64_t i = (int64_t)blockIdx.x * WARPS + (lane >> 2);
-    FSum L = block_fsum(sh.v);
+    FSum L = block_fsum(sh.v), B;
+    if (MALA) B = block_fsum(bwd.v);
     if (lane & 3) return;
     int accept = 0;
     if (i < N) {
         const float2 yd = s.ydq[i];
         L.add(yd.x);
         L.add(yd.y);
-        accept = mh_test(s, L, i, coef, 0.0f, m_prev, err);
+        float extra = 0.0f;
+        if (MALA) {
+            const float2 fw = a.fwd[i];
+            const float h = *a.h;
+            extra = -((B.s - fw.x) + (B.c - fw.y)) / (2.0f * h * h);
+        }
+        accept = mh_test(s, L, i, coef, extra, m_prev, err);
     }
     acc[lane >> 2] = accept;
 }
@@ -442,16 +444,13 @@ __global__ void k_step_constants(PriorArgs pr, const double* __restrict__ sched,
     }
 }
 
-// Accepted-proposal count of a block: one slot per warp, written by its lane 0 whatever the
-// outcome; thread 0 sums them and makes one global atomic.
-__device__ __forceinline__ void count_warps(unsigned long long* acc_count, const int* accw)
+// Accepted proposals of a block, from its particles' decisions (one warp, after the barrier that
+// follows them): one global atomic.
+__device__ __forceinline__ void count_accepts(unsigned long long* acc_count, const int* accw)
 {
-    __syncthreads();
-    if (threadIdx.x == 0 && acc_count) {
-        int s = 0;
-        for (int k = 0; k < (int)(blockDim.x >> 5); ++k) s += accw[k];
-        if (s) atomicAdd(acc_count, (unsigned long long)s);
-    }
+    const int lane = threadIdx.x & 31;
+    const int n = __popc(__ballot_sync(0xffffffffu, lane < WARPS && accw[lane % WARPS] != 0));
+    if (lane == 0 && acc_count && n) atomicAdd(acc_count, (unsigned long long)n);
 }
 
 template <bool DECIDE, bool VEC>
@@ -478,7 +477,7 @@ __global__ void __launch_bounds__(BLOCK, 5) k_move_rw(MoveArgs a, int64_t N, int
     }
     const float4 sk = stepk[t];
     if (DECIDE) {
-        if (w == 0) mh_decide_block(a.mh, parts, N, sk.y, m_prev, accw, err);
+        if (w == 0) mh_decide_block<false>(a, parts, lts, N, sk.y, m_prev, accw, err);
         __syncthreads();
     }
     FSum lt;
@@ -515,10 +514,7 @@ __global__ void __launch_bounds__(BLOCK, 5) k_move_rw(MoveArgs a, int64_t N, int
         }
     }
     if (noise) draw_accept_logu(a.mh, N, t, m, *seedp);
-    if (DECIDE && w == 2) {
-        const int n_acc = __popc(__ballot_sync(0xffffffffu, lane < WARPS && accw[lane % WARPS] != 0));
-        if (lane == 0 && a.mh.acc_count && n_acc) atomicAdd(a.mh.acc_count, (unsigned long long)n_acc);
-    }
+    if (DECIDE && w == 2) count_accepts(a.mh.acc_count, accw);
 }
 
 // ------------------------------------------------------------ MALA move kernel
@@ -599,6 +595,8 @@ __global__ void __launch_bounds__(BLOCK, 4) k_move_mala(MoveArgs a, int64_t N, i
     __shared__ int accw[BLOCK / 32];
     __shared__ PartSlices parts;
     __shared__ RsumSlices rsum;
+    __shared__ LaneSums lts, fws, yos;  // (lts: the reverse sums first)
+    const int w = threadIdx.x >> 5;
     const int64_t i = warp_global_id();
     const int lane = threadIdx.x & 31, groups = (p + 3) >> 2;
     float4 z4 = make_float4(0.f, 0.f, 0.f, 0.f);  // (as in k_move_rw)
@@ -613,27 +611,35 @@ __global__ void __launch_bounds__(BLOCK, 4) k_move_mala(MoveArgs a, int64_t N, i
     }
     const float4 sk = stepk[t];
     bool acc = false;
-    if (i < N) {
-        const uint64_t seed = *seedp;
-        const float ac = sk.x, a1 = pr.a + 1.0f, inv_c = sk.z;
-        const float h = *a.h, h2 = 0.5f * h * h;
-        const float* D = a.sigma;
-        if (DECIDE) {
-            const FSum bwd = warp_sum(mala_reverse<VEC>(a, i, p, lane, h2, a1, ac, inv_c, pr.de, rsum.sum[threadIdx.x >> 5]));
-            const float2 fw = a.fwd[i];
-            const float extra = -((bwd.s - fw.x) + (bwd.c - fw.y)) / (2.0f * h * h);
-            acc = mh_decide(a.mh, parts, i, lane, sk.y, extra, m_prev, err);
-        } else {
-            acc = take_resampled(a, i, lane);
+    const uint64_t seed = *seedp;
+    const float ac = sk.x, a1 = pr.a + 1.0f, inv_c = sk.z;
+    const float h = *a.h, h2 = 0.5f * h * h;
+    const float* D = a.sigma;
+    if (DECIDE) {
+        // (each warp by itself: two more barriers here cost as much as the block's way saves)
+        int accept = 0;
+        if (i < N) {
+            const FSum bwd = warp_sum(mala_reverse<VEC>(a, i, p, lane, h2, a1, ac, inv_c, pr.de, rsum.sum[w]));
+            const FSum L = proposal_loglik(a.mh, parts, i, lane);
+            if (lane == 0) {
+                const float2 fq = a.fwd[i];
+                accept = mh_test(a.mh, L, i, sk.y, -((bwd.s - fq.x) + (bwd.c - fq.y)) / (2.0f * h * h), m_prev, err);
+            }
         }
+        if (lane == 0) accw[w] = accept;
+        acc = __shfl_sync(0xffffffffu, accept, 0) != 0;
+    } else if (i < N) {
+        acc = take_resampled(a, i, lane);
+    }
+    FSum lt, fw;
+    float yd = 0.0f, off = 0.0f;
+    if (i < N) {
         const float* src = (acc ? a.beta_p : a.beta) + i * p;
         const float* gsrc = (acc ? a.gl_p : a.gl) + i * p;
         float* cur = a.beta + i * p;
         float* gcur = a.gl + i * p;
         float* dst = a.beta_p + i * p;
         __nv_bfloat16* Arow = a.A ? a.A + i * (int64_t)a.ldA : nullptr;
-        FSum lt, fw;
-        float yd = 0.0f, off = 0.0f;
         const bool grouped = (p & 3) == 0 && !pr.de;  // the four-coordinate prior term
         if (VEC) {
             // p % 4 == 0: the same per-coordinate arithmetic on float4 groups, the state's and
@@ -696,41 +702,52 @@ __global__ void __launch_bounds__(BLOCK, 4) k_move_mala(MoveArgs a, int64_t N, i
             }
             if (grouped) lt.add(prior_terms4(make_float4(bq[0], bq[1], bq[2], bq[3]), sk.w));
         }
-        lt = warp_sum(lt);
-        fw = warp_sum(fw);
-        yd = warp_sum(yd);
-        off = warp_sum(off);
-        if (lane == 0) {
-            a.lpt_p[i] = make_float2(lt.s, lt.c);
-            a.fwd[i] = make_float2(fw.s, fw.c);
-            a.ydq[i] = make_float2(yd, 0.0f);
-            if (Arow) pack_offset(Arow, a.Kp, p, off);
+    }
+    lts.v[lane][w] = make_float2(lt.s, lt.c);
+    fws.v[lane][w] = make_float2(fw.s, fw.c);
+    yos.v[lane][w] = make_float2(yd, off);
+    __syncthreads();
+    const int64_t ib = (int64_t)blockIdx.x * WARPS + (lane >> 2);
+    const bool mine = (lane & 3) == 0 && ib < N;
+    if (w == 0) {
+        const FSum q = block_fsum(lts.v);
+        if (mine) a.lpt_p[ib] = make_float2(q.s, q.c);
+    } else if (w == 1) {
+        const float2 q = block_sum2(yos.v);
+        if (mine) {
+            a.ydq[ib] = make_float2(q.x, 0.0f);
+            if (a.A) pack_offset(a.A + ib * (int64_t)a.ldA, a.Kp, p, q.y);
         }
+    } else if (w == 2) {
+        const FSum q = block_fsum(fws.v);
+        if (mine) a.fwd[ib] = make_float2(q.s, q.c);
     }
     draw_accept_logu(a.mh, N, t, m, *seedp);
-    if (DECIDE) {
-        if (lane == 0) accw[threadIdx.x >> 5] = acc ? 1 : 0;
-        count_warps(a.mh.acc_count, accw);
-    }
+    if (DECIDE && w == 3) count_accepts(a.mh.acc_count, accw);
 }
 
 // ------------------------------------------------------------ last move of a step
 // MH test of the pending proposals (RW, or MALA with the reverse term), then accepted
 // proposals (and their gradients) are copied into the state rows, so that between steps
 // beta and gl hold the particles.
+// The block's tests: accw[k] = the decision on its particle k, for all threads on return.
 template <bool MALA, bool VEC>
-__device__ __forceinline__ bool commit_test(const MoveArgs& a, const PartSlices& parts, const RsumSlices& rsum, int64_t i, int p, int lane, PriorArgs pr,
-                                            float4 sk, uint32_t m_prev, uint32_t* err)
+__device__ __forceinline__ void commit_tests(const MoveArgs& a, const PartSlices& parts, const RsumSlices& rsum, LaneSums& bwds,
+                                             int64_t N, int p, PriorArgs pr, float4 sk, uint32_t m_prev, int* accw,
+                                             uint32_t* err)
 {
-    float extra = 0.0f;
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (MALA) {
+        const int64_t i = warp_global_id();
         const float ac = sk.x, a1 = pr.a + 1.0f, inv_c = sk.z;
         const float h = *a.h, h2 = 0.5f * h * h;
-        const FSum bwd = warp_sum(mala_reverse<VEC>(a, i, p, lane, h2, a1, ac, inv_c, pr.de, rsum.sum[threadIdx.x >> 5]));
-        const float2 fw = a.fwd[i];
-        extra = -((bwd.s - fw.x) + (bwd.c - fw.y)) / (2.0f * h * h);
+        FSum bwd;
+        if (i < N) bwd = mala_reverse<VEC>(a, i, p, lane, h2, a1, ac, inv_c, pr.de, rsum.sum[w]);
+        bwds.v[lane][w] = make_float2(bwd.s, bwd.c);
+        __syncthreads();
     }
-    return mh_decide(a.mh, parts, i, lane, sk.y, extra, m_prev, err);
+    if (w == 0) mh_decide_block<MALA>(a, parts, bwds, N, sk.y, m_prev, accw, err);
+    __syncthreads();
 }
 
 template <bool MALA, bool VEC>
@@ -757,6 +774,7 @@ __global__ void __launch_bounds__(BLOCK) k_move_commit(MoveArgs a, int64_t N, in
     __shared__ int accw[BLOCK / 32];
     __shared__ PartSlices parts;
     __shared__ RsumSlices rsum;
+    __shared__ LaneSums bwds;
     grid_dependency_wait();
     gather_partials(a.mh, N, parts);
     if (MALA && a.gp.gpart) gather_rsum(a.mh, a.gp, N, rsum);
@@ -765,13 +783,9 @@ __global__ void __launch_bounds__(BLOCK) k_move_commit(MoveArgs a, int64_t N, in
     const float4 sk = stepk[t];
     const int64_t i = warp_global_id();
     const int lane = threadIdx.x & 31;
-    bool acc = false;
-    if (i < N) {
-        acc = commit_test<MALA, VEC>(a, parts, rsum, i, p, lane, pr, sk, m_prev, err);
-        if (acc) commit_row<MALA, VEC>(a, i, p, lane);
-    }
-    if (lane == 0) accw[threadIdx.x >> 5] = acc ? 1 : 0;
-    count_warps(a.mh.acc_count, accw);
+    commit_tests<MALA, VEC>(a, parts, rsum, bwds, N, p, pr, sk, m_prev, accw, err);
+    if (accw[threadIdx.x >> 5]) commit_row<MALA, VEC>(a, i, p, lane);
+    if (threadIdx.x < 32) count_accepts(a.mh.acc_count, accw);
 }
 
 // ------------------------------------------------------------ log-likelihood finish
@@ -800,8 +814,7 @@ __global__ void __launch_bounds__(BLOCK) k_finish_loglik(MhState s, int64_t N, d
 // log w_i = sum_j log p(beta_ij | c_t) - log p(beta_ij | c_{t-1}) in the form without
 // cancellation: -log(c_t/c_{t-1}) - (a+1) log1p(x (c_{t-1} - c_t) / (c_t (a c_{t-1} + x))),
 // x = |beta_ij| (double exponential: -log(c_t/c_{t-1}) - x (1/c_t - 1/c_{t-1})).
-// A block handles 32 particles: its warps form the FP32 row sums, then warp 0 finishes one
-// particle per lane in FP64. The step's constants come from the per-sweep table.
+// A block handles 8 particles: its warps form the FP32 row sums, then warp 0 finishes them in FP64. The step's constants come from the per-sweep table.
 constexpr int RW_PER_BLOCK = 8;
 constexpr int RW_THREADS = 32 * RW_PER_BLOCK;
 
@@ -820,20 +833,23 @@ __device__ __forceinline__ void reweight_row(const float* b, int p, PriorArgs pr
         for (int g = lane; 4 * g < p; g += 32) snew.add(prior_terms4(ld4(b + 4 * g), inv_ac));
 }
 
-// The block's particles' log-weights from the row sums (warp 0, one particle per lane, FP64).
-__device__ __forceinline__ void reweight_finish(const float4* sums, int64_t base, int64_t N, PriorArgs pr, const ReweightK& rk,
-                                                double* __restrict__ logw, float2* __restrict__ lpq, uint32_t* err)
+// The block's particles' log-weights from the lane partials of their row sums (one warp; lane 4 k
+// finishes particle k in FP64).
+__device__ __forceinline__ void reweight_block(const LaneSums& diffs, const LaneSums& news, int64_t N, PriorArgs pr,
+                                               const ReweightK& rk, double* __restrict__ logw, float2* __restrict__ lpq,
+                                               uint32_t* err)
 {
-    const int lane = threadIdx.x;
-    if (lane >= RW_PER_BLOCK || base + lane >= N) return;
-    const int64_t i = base + lane;
-    const float4 s = sums[lane];
-    const double sd = (double)s.x + (double)s.y;
+    static_assert(RW_PER_BLOCK == WARPS, "one warp per particle");
+    const int lane = threadIdx.x & 31;
+    const int64_t i = (int64_t)blockIdx.x * WARPS + (lane >> 2);
+    const FSum ds = block_fsum(diffs.v), q = block_fsum(news.v);
+    if ((lane & 3) || i >= N) return;
+    const double sd = (double)ds.s + (double)ds.c;
     const double d = pr.de ? rk.lbase - sd * rk.dinv : rk.lbase - ((double)pr.a + 1.0) * sd;
     const double nl = logw[i] + d;
     if (!isfinite(nl)) atomicOr(err, DERR_NONFINITE);
     logw[i] = nl;
-    lpq[i] = make_float2(s.z, s.w);
+    lpq[i] = make_float2(q.s, q.c);
 }
 
 __global__ void __launch_bounds__(RW_THREADS) k_reweight(const float* __restrict__ beta, double* __restrict__ logw,
@@ -841,17 +857,16 @@ __global__ void __launch_bounds__(RW_THREADS) k_reweight(const float* __restrict
                                                    const ReweightK* __restrict__ rkp, int t, uint32_t* __restrict__ err)
 {
     grid_dependency_wait();
-    __shared__ float4 sums[RW_PER_BLOCK];
+    __shared__ LaneSums diffs, news;
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int64_t base = (int64_t)blockIdx.x * RW_PER_BLOCK;
     const ReweightK rk = rkp[t];
     FSum sdiff, snew;
     if (base + w < N) reweight_row(beta + (base + w) * p, p, pr, rk, lane, sdiff, snew);
-    sdiff = warp_sum(sdiff);
-    snew = warp_sum(snew);
-    if (lane == 0) sums[w] = make_float4(sdiff.s, sdiff.c, snew.s, snew.c);
+    diffs.v[lane][w] = make_float2(sdiff.s, sdiff.c);
+    news.v[lane][w] = make_float2(snew.s, snew.c);
     __syncthreads();
-    reweight_finish(sums, base, N, pr, rk, logw, lpq, err);
+    if (w == 0) reweight_block(diffs, news, N, pr, rk, logw, lpq, err);
 }
 
 // The step's last MH test with its commit (k_move_commit), then the reweighting to the next
@@ -863,11 +878,10 @@ __global__ void __launch_bounds__(BLOCK) k_commit_reweight(MoveArgs a, int64_t N
                                                           double* __restrict__ logw, const ReweightK* __restrict__ rkp,
                                                           uint32_t* err)
 {
-    static_assert(RW_PER_BLOCK == WARPS, "one warp per particle in both halves");
     __shared__ int accw[BLOCK / 32];
     __shared__ PartSlices parts;
     __shared__ RsumSlices rsum;
-    __shared__ float4 sums[RW_PER_BLOCK];
+    __shared__ LaneSums diffs, news;  // (diffs: the reverse moves' sums first)
     grid_dependency_wait();
     gather_partials(a.mh, N, parts);
     if (MALA && a.gp.gpart) gather_rsum(a.mh, a.gp, N, rsum);
@@ -877,21 +891,18 @@ __global__ void __launch_bounds__(BLOCK) k_commit_reweight(MoveArgs a, int64_t N
     const ReweightK rk = rkp[t + 1];
     const int64_t i = warp_global_id();
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    bool acc = false;
+    commit_tests<MALA, VEC>(a, parts, rsum, diffs, N, p, pr, sk, m_prev, accw, err);
     FSum sdiff, snew;
     if (i < N) {
-        acc = commit_test<MALA, VEC>(a, parts, rsum, i, p, lane, pr, sk, m_prev, err);
+        const bool acc = accw[w] != 0;
         if (acc) commit_row<MALA, VEC>(a, i, p, lane);
         reweight_row((acc ? a.beta_p : a.beta) + i * p, p, pr, rk, lane, sdiff, snew);
     }
-    sdiff = warp_sum(sdiff);
-    snew = warp_sum(snew);
-    if (lane == 0) {
-        sums[w] = make_float4(sdiff.s, sdiff.c, snew.s, snew.c);
-        accw[w] = acc ? 1 : 0;
-    }
-    count_warps(a.mh.acc_count, accw);  // a block barrier first
-    reweight_finish(sums, (int64_t)blockIdx.x * RW_PER_BLOCK, N, pr, rk, logw, a.mh.lpq, err);
+    diffs.v[lane][w] = make_float2(sdiff.s, sdiff.c);
+    news.v[lane][w] = make_float2(snew.s, snew.c);
+    __syncthreads();
+    if (w == 1) count_accepts(a.mh.acc_count, accw);
+    if (w == 0) reweight_block(diffs, news, N, pr, rk, logw, a.mh.lpq, err);
 }
 
 // ---------------------------------------------------------- log-sum-exp and ESS
