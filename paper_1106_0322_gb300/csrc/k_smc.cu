@@ -42,6 +42,14 @@ __device__ __forceinline__ float dlogprior(float b, float a1, float ac, float in
     return de ? -sg * inv_c : __fdividef(-a1 * sg, ac + fabsf(b));
 }
 
+// g + dlogprior(b) as one multiply-add: what the sum of the two compiles to in the MALA kernels, written
+// out so that the reverse move's bits do not depend on the code around it.
+__device__ __forceinline__ float dlogpost(float g, float b, float a1, float ac, float inv_c, int de)
+{
+    const float sg = (b > 0.0f) ? 1.0f : ((b < 0.0f) ? -1.0f : 0.0f);
+    return de ? fmaf(-sg, inv_c, g) : fmaf(-a1 * sg, rcp_approx(ac + fabsf(b)), g);
+}
+
 // ------------------------------------------------------------------- init (t = 0)
 __global__ void k_init_prior(float* __restrict__ beta, int64_t N, int p, PriorArgs pr, const double* __restrict__ sched,
                              int t0, const uint64_t* __restrict__ seedp)
@@ -522,12 +530,11 @@ __global__ void __launch_bounds__(BLOCK, 5) k_move_rw(MoveArgs a, int64_t N, int
 // warp sum): sum_j (beta_j - beta'_j - (h^2/2) D_j g'_j)^2 / D_j, g' = grad l' + the prior
 // gradient at beta'. VEC (p % 4 == 0): lane l takes the 4-coordinate groups l, l + 32, ...
 // with float4 loads; else coordinates l, l + 32, ...
-template <bool VEC>
+template <bool VEC, bool PARTS>
 __device__ __forceinline__ FSum mala_reverse(const MoveArgs& a, int64_t i, int p, int lane, float h2, float a1, float ac,
                                              float inv_c, int de, float rs)
 {
     FSum bwd;
-    const bool parts = a.gp.gpart != nullptr;
     const float* b0 = a.beta + i * p;
     const float* b1 = a.beta_p + i * p;
     float* g1 = a.gl_p + i * p;
@@ -535,7 +542,7 @@ __device__ __forceinline__ FSum mala_reverse(const MoveArgs& a, int64_t i, int p
         for (int j0 = 4 * lane; j0 < p; j0 += 128) {
             const float4 x0 = ld4(b0 + j0), x1 = ld4(b1 + j0);
             float4 gg;
-            if (parts) {
+            if (PARTS) {
                 float o[4];
                 finish_gradient4<1>(a, i, p, j0, rs, o);
                 gg = make_float4(o[0], o[1], o[2], o[3]);
@@ -546,31 +553,31 @@ __device__ __forceinline__ FSum mala_reverse(const MoveArgs& a, int64_t i, int p
             const float4 Dv = ldg4(a.sigma + j0), iD = ldg4(a.inv_D + j0);
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
-                const float drift = h2 * comp(Dv, k) * (comp(gg, k) + dlogprior(comp(x1, k), a1, ac, inv_c, de));
+                const float drift = h2 * comp(Dv, k) * dlogpost(comp(gg, k), comp(x1, k), a1, ac, inv_c, de);
                 const float d = (comp(x0, k) - comp(x1, k)) - drift;
                 bwd.add(d * d * comp(iD, k));
             }
         }
+    } else if (PARTS) {
+        for (int j0 = lane; j0 < p; j0 += 128) {
+            float g4[4];
+            finish_gradient4<32>(a, i, p, j0, rs, g4);
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                const int j = j0 + 32 * k;
+                if (j >= p) break;
+                g1[j] = g4[k];
+                const float drift = h2 * a.sigma[j] * dlogpost(g4[k], b1[j], a1, ac, inv_c, de);
+                const float d = (b0[j] - b1[j]) - drift;
+                bwd.add(d * d * a.inv_D[j]);
+            }
+        }
     } else {
-        auto term = [&](int j, float gg) {
-            const float drift = h2 * a.sigma[j] * (gg + dlogprior(b1[j], a1, ac, inv_c, de));
+        const float* g = a.gl_p + i * p;
+        for (int j = lane; j < p; j += 32) {
+            const float drift = h2 * a.sigma[j] * dlogpost(g[j], b1[j], a1, ac, inv_c, de);
             const float d = (b0[j] - b1[j]) - drift;
             bwd.add(d * d * a.inv_D[j]);
-        };
-        if (parts) {
-            for (int j0 = lane; j0 < p; j0 += 128) {
-                float g4[4];
-                finish_gradient4<32>(a, i, p, j0, rs, g4);
-#pragma unroll
-                for (int k = 0; k < 4; ++k) {
-                    const int j = j0 + 32 * k;
-                    if (j >= p) break;
-                    g1[j] = g4[k];
-                    term(j, g4[k]);
-                }
-            }
-        } else {
-            for (int j = lane; j < p; j += 32) term(j, g1[j]);
         }
     }
     return bwd;
@@ -587,7 +594,7 @@ __device__ __forceinline__ FSum mala_reverse(const MoveArgs& a, int64_t i, int p
 // log alpha = l' + lp' - l - lp - (bwd - fwd)/(2h^2); an accepted proposal and its gradient
 // are written back as the state while being read. At most 64 registers, so that 4 blocks
 // fit an SM (1.68 waves of 8192 particle warps; the test variant would take 74 and 3 blocks).
-template <bool DECIDE, bool VEC>
+template <bool DECIDE, bool VEC, bool PARTS>
 __global__ void __launch_bounds__(BLOCK, 4) k_move_mala(MoveArgs a, int64_t N, int p, PriorArgs pr,
                                                     const float4* __restrict__ stepk, int t, uint32_t m,
                                                     uint32_t m_prev, const uint64_t* __restrict__ seedp, uint32_t* err)
@@ -605,9 +612,9 @@ __global__ void __launch_bounds__(BLOCK, 4) k_move_mala(MoveArgs a, int64_t N, i
     grid_launch_dependents();
     if (DECIDE) {
         gather_partials(a.mh, N, parts);
-        if (a.gp.gpart) gather_rsum(a.mh, a.gp, N, rsum);
+        if (PARTS) gather_rsum(a.mh, a.gp, N, rsum);
         __syncthreads();
-        if (a.gp.gpart) sum_rsum(rsum);
+        if (PARTS) sum_rsum(rsum);
     }
     const float4 sk = stepk[t];
     bool acc = false;
@@ -619,7 +626,7 @@ __global__ void __launch_bounds__(BLOCK, 4) k_move_mala(MoveArgs a, int64_t N, i
         // (each warp by itself: two more barriers here cost as much as the block's way saves)
         int accept = 0;
         if (i < N) {
-            const FSum bwd = warp_sum(mala_reverse<VEC>(a, i, p, lane, h2, a1, ac, inv_c, pr.de, rsum.sum[w]));
+            const FSum bwd = warp_sum(mala_reverse<VEC, PARTS>(a, i, p, lane, h2, a1, ac, inv_c, pr.de, PARTS ? rsum.sum[w] : 0.0f));
             const FSum L = proposal_loglik(a.mh, parts, i, lane);
             if (lane == 0) {
                 const float2 fq = a.fwd[i];
@@ -731,7 +738,7 @@ __global__ void __launch_bounds__(BLOCK, 4) k_move_mala(MoveArgs a, int64_t N, i
 // proposals (and their gradients) are copied into the state rows, so that between steps
 // beta and gl hold the particles.
 // The block's tests: accw[k] = the decision on its particle k, for all threads on return.
-template <bool MALA, bool VEC>
+template <bool MALA, bool VEC, bool PARTS>
 __device__ __forceinline__ void commit_tests(const MoveArgs& a, const PartSlices& parts, const RsumSlices& rsum, LaneSums& bwds,
                                              int64_t N, int p, PriorArgs pr, float4 sk, uint32_t m_prev, int* accw,
                                              uint32_t* err)
@@ -742,7 +749,7 @@ __device__ __forceinline__ void commit_tests(const MoveArgs& a, const PartSlices
         const float ac = sk.x, a1 = pr.a + 1.0f, inv_c = sk.z;
         const float h = *a.h, h2 = 0.5f * h * h;
         FSum bwd;
-        if (i < N) bwd = mala_reverse<VEC>(a, i, p, lane, h2, a1, ac, inv_c, pr.de, rsum.sum[w]);
+        if (i < N) bwd = mala_reverse<VEC, PARTS>(a, i, p, lane, h2, a1, ac, inv_c, pr.de, PARTS ? rsum.sum[w] : 0.0f);
         bwds.v[lane][w] = make_float2(bwd.s, bwd.c);
         __syncthreads();
     }
@@ -766,7 +773,7 @@ __device__ __forceinline__ void commit_row(const MoveArgs& a, int64_t i, int p, 
     }
 }
 
-template <bool MALA, bool VEC>
+template <bool MALA, bool VEC, bool PARTS>
 __global__ void __launch_bounds__(BLOCK) k_move_commit(MoveArgs a, int64_t N, int p, PriorArgs pr,
                                                       const float4* __restrict__ stepk, int t, uint32_t m_prev,
                                                       const uint64_t* __restrict__ seedp, uint32_t* err)
@@ -777,13 +784,13 @@ __global__ void __launch_bounds__(BLOCK) k_move_commit(MoveArgs a, int64_t N, in
     __shared__ LaneSums bwds;
     grid_dependency_wait();
     gather_partials(a.mh, N, parts);
-    if (MALA && a.gp.gpart) gather_rsum(a.mh, a.gp, N, rsum);
+    if (PARTS) gather_rsum(a.mh, a.gp, N, rsum);
     __syncthreads();
-    if (MALA && a.gp.gpart) sum_rsum(rsum);
+    if (PARTS) sum_rsum(rsum);
     const float4 sk = stepk[t];
     const int64_t i = warp_global_id();
     const int lane = threadIdx.x & 31;
-    commit_tests<MALA, VEC>(a, parts, rsum, bwds, N, p, pr, sk, m_prev, accw, err);
+    commit_tests<MALA, VEC, PARTS>(a, parts, rsum, bwds, N, p, pr, sk, m_prev, accw, err);
     if (accw[threadIdx.x >> 5]) commit_row<MALA, VEC>(a, i, p, lane);
     if (threadIdx.x < 32) count_accepts(a.mh.acc_count, accw);
 }
@@ -872,7 +879,7 @@ __global__ void __launch_bounds__(RW_THREADS) k_reweight(const float* __restrict
 // The step's last MH test with its commit (k_move_commit), then the reweighting to the next
 // scale of the row just settled, in one launch: one kernel boundary less a step, and the row is
 // read once.
-template <bool MALA, bool VEC>
+template <bool MALA, bool VEC, bool PARTS>
 __global__ void __launch_bounds__(BLOCK) k_commit_reweight(MoveArgs a, int64_t N, int p, PriorArgs pr,
                                                           const float4* __restrict__ stepk, int t, uint32_t m_prev,
                                                           double* __restrict__ logw, const ReweightK* __restrict__ rkp,
@@ -884,14 +891,14 @@ __global__ void __launch_bounds__(BLOCK) k_commit_reweight(MoveArgs a, int64_t N
     __shared__ LaneSums diffs, news;  // (diffs: the reverse moves' sums first)
     grid_dependency_wait();
     gather_partials(a.mh, N, parts);
-    if (MALA && a.gp.gpart) gather_rsum(a.mh, a.gp, N, rsum);
+    if (PARTS) gather_rsum(a.mh, a.gp, N, rsum);
     __syncthreads();
-    if (MALA && a.gp.gpart) sum_rsum(rsum);
+    if (PARTS) sum_rsum(rsum);
     const float4 sk = stepk[t];
     const ReweightK rk = rkp[t + 1];
     const int64_t i = warp_global_id();
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    commit_tests<MALA, VEC>(a, parts, rsum, diffs, N, p, pr, sk, m_prev, accw, err);
+    commit_tests<MALA, VEC, PARTS>(a, parts, rsum, diffs, N, p, pr, sk, m_prev, accw, err);
     FSum sdiff, snew;
     if (i < N) {
         const bool acc = accw[w] != 0;
@@ -1995,12 +2002,13 @@ cudaError_t launch_move_mala(const MoveArgs& a, bool decide, int64_t N, int p, P
     cudaLaunchConfig_t cfg = pdl_config(warps_grid(N), BLOCK, st);  // follows the gradient finish or the scales
     cudaLaunchAttribute attr[1];
     pdl_attr(cfg, attr);
-    if (decide) {
-        if (vec) return cudaLaunchKernelEx(&cfg, k_move_mala<true, true>, a, N, p, pr, stepk, t, m, m_prev, seed, err);
-        return cudaLaunchKernelEx(&cfg, k_move_mala<true, false>, a, N, p, pr, stepk, t, m, m_prev, seed, err);
-    }
-    if (vec) return cudaLaunchKernelEx(&cfg, k_move_mala<false, true>, a, N, p, pr, stepk, t, m, m_prev, seed, err);
-    return cudaLaunchKernelEx(&cfg, k_move_mala<false, false>, a, N, p, pr, stepk, t, m, m_prev, seed, err);
+    const bool parts = a.gp.gpart != nullptr;
+    auto* kern = vec ? k_move_mala<false, true, false> : k_move_mala<false, false, false>;
+    if (decide && parts)
+        kern = vec ? k_move_mala<true, true, true> : k_move_mala<true, false, true>;
+    else if (decide)
+        kern = vec ? k_move_mala<true, true, false> : k_move_mala<true, false, false>;
+    return cudaLaunchKernelEx(&cfg, kern, a, N, p, pr, stepk, t, m, m_prev, seed, err);
 }
 
 cudaError_t launch_move_commit(const MoveArgs& a, bool mala, int64_t N, int p, PriorArgs pr, const float4* stepk, int t,
@@ -2010,12 +2018,13 @@ cudaError_t launch_move_commit(const MoveArgs& a, bool mala, int64_t N, int p, P
     cudaLaunchConfig_t cfg = pdl_config(warps_grid(N), BLOCK, st);  // follows the likelihood GEMM
     cudaLaunchAttribute attr[1];
     pdl_attr(cfg, attr);
-    if (mala) {
-        if (vec) return cudaLaunchKernelEx(&cfg, k_move_commit<true, true>, a, N, p, pr, stepk, t, m_prev, seed, err);
-        return cudaLaunchKernelEx(&cfg, k_move_commit<true, false>, a, N, p, pr, stepk, t, m_prev, seed, err);
-    }
-    if (vec) return cudaLaunchKernelEx(&cfg, k_move_commit<false, true>, a, N, p, pr, stepk, t, m_prev, seed, err);
-    return cudaLaunchKernelEx(&cfg, k_move_commit<false, false>, a, N, p, pr, stepk, t, m_prev, seed, err);
+    const bool parts = mala && a.gp.gpart != nullptr;
+    auto* kern = vec ? k_move_commit<false, true, false> : k_move_commit<false, false, false>;
+    if (parts)
+        kern = vec ? k_move_commit<true, true, true> : k_move_commit<true, false, true>;
+    else if (mala)
+        kern = vec ? k_move_commit<true, true, false> : k_move_commit<true, false, false>;
+    return cudaLaunchKernelEx(&cfg, kern, a, N, p, pr, stepk, t, m_prev, seed, err);
 }
 
 cudaError_t launch_finish_loglik(const MhState& s, int64_t N, double* logw, double* ll_out, uint32_t* err,
@@ -2030,11 +2039,13 @@ cudaError_t launch_commit_reweight(const MoveArgs& a, bool mala, int64_t N, int 
 {
     const bool vec = (p & 3) == 0;
     const dim3 grid(warps_grid(N)), block(BLOCK);
-    if (mala)
-        return vec ? launch_pdl(k_commit_reweight<true, true>, grid, block, (size_t)0, st, a, N, p, pr, stepk, t, m_prev, logw, rk, err)
-                   : launch_pdl(k_commit_reweight<true, false>, grid, block, (size_t)0, st, a, N, p, pr, stepk, t, m_prev, logw, rk, err);
-    return vec ? launch_pdl(k_commit_reweight<false, true>, grid, block, (size_t)0, st, a, N, p, pr, stepk, t, m_prev, logw, rk, err)
-               : launch_pdl(k_commit_reweight<false, false>, grid, block, (size_t)0, st, a, N, p, pr, stepk, t, m_prev, logw, rk, err);
+    const bool parts = mala && a.gp.gpart != nullptr;
+    auto* kern = vec ? k_commit_reweight<false, true, false> : k_commit_reweight<false, false, false>;
+    if (parts)
+        kern = vec ? k_commit_reweight<true, true, true> : k_commit_reweight<true, false, true>;
+    else if (mala)
+        kern = vec ? k_commit_reweight<true, true, false> : k_commit_reweight<true, false, false>;
+    return launch_pdl(kern, grid, block, (size_t)0, st, a, N, p, pr, stepk, t, m_prev, logw, rk, err);
 }
 
 cudaError_t launch_reweight(const float* beta, double* logw, float2* lpq, int64_t N, int p, PriorArgs pr,
