@@ -535,7 +535,8 @@ def grad_roofline(reg, w, stream):
     achieved = flop / (ms / 1e3) / 1e12
     peak, src = tensor_peak_burst()
     return {"bound": "tensor", "achieved": achieved, "peak": peak, "unit": "TFLOP/s", "frac": achieved / peak,
-            "traffic": None, "kernel": "k_loglik_tc<resid> + k_adjoint_tc + k_grad_finish", "launch_ms": ms,
+            "traffic": None, "kernel": "k_grad_tc (p <= 255; else k_loglik_tc<resid> + k_adjoint_tc) + k_grad_finish",
+            "launch_ms": ms,
             "peak_source": src, "algorithmic_flop_per_launch": flop}
 
 

@@ -168,8 +168,8 @@ int spa_run_batch(spa_ctx* const* ctxs, int32_t R, const spa_batch_args* args, s
  * per context, on the context's stream) run concurrently on the GPU, and every
  * spa_batch_run is a single graph launch on the batch's own stream. Each region's
  * likelihood tile configuration comes from the tile table or the tuner. In this branch form
- * each region's likelihood and adjoint launches are sized for an eighth of the SMs (an
- * equal share when fewer than 8 regions), so that the regions share the GPU; the partials,
+ * each region's likelihood and adjoint launches are sized for a share of the SMs in
+ * proportion to the region's work, so that the regions share the GPU; the partials,
  * and so the results, do not depend on the grid.
  * With the environment variable SPA_BATCH_MODE=lockstep at creation, a batch whose regions
  * share T, N, moves_per_step, the move kind (RW or MALA), the start and the burn-in, on the
