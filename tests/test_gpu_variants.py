@@ -164,3 +164,21 @@ def test_uneven_batch_shares_give_the_single_runs(spa, move):
             assert np.array_equal(one[k], two[k]), k
     for r in rs:
         r.close()
+
+
+# The reverse move's gradient sum is one multiply-add in every form of the MALA kernels: for p <= 255
+# a region alone takes the fused gradient kernel and, beside another, the two kernels, and p decides
+# whether the gradient is formed where it is tested. A rounding more in one form shows only in
+# about one of 10^7 decisions, so the sweeps are long enough to meet one.
+@pytest.mark.parametrize("n,p", [(2714, 226), (1500, 190), (1200, 77)])
+def test_mala_decisions_do_not_depend_on_the_launches(spa, n, p):
+    reg = synth.make_region(n, p, 0.86, (0.3, 0.5, -0.4), seed=1803)
+    sched = synth.geometric_schedule(10)
+    with spa.Region(reg.G, reg.y, 16.0, config=spa.make_config(move="mala")) as r:
+        for seed in (100, 101):
+            one = r.run(sched, 16384, 12, seed)
+            b = spa.Batch([r], [sched], [16384], [12], [seed])
+            (two,) = b.run()
+            b.close()
+            for k in one:
+                assert np.array_equal(one[k], two[k]), k
