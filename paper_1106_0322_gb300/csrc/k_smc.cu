@@ -572,6 +572,8 @@ __device__ __forceinline__ FSum mala_reverse(const MoveArgs& a, int64_t i, int p
                 bwd.add(d * d * a.inv_D[j]);
             }
         }
+        // k_move_mala reads an accepted row back by fours, from other lanes than stored it here
+        __syncwarp();
     } else {
         const float* g = a.gl_p + i * p;
         for (int j = lane; j < p; j += 32) {
