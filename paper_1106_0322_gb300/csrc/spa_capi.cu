@@ -24,6 +24,7 @@
 
 #include "../../include/spa.h"
 #include "spa_device.cuh"
+#include "spa_host_rules.h"
 #include "spa_internal.h"
 
 using namespace spa;
@@ -298,13 +299,43 @@ int settle_stream(spa_ctx* c, cudaStream_t st)
     return SPA_OK;
 }
 
-// Whether the likelihood entry points can read the caller's device particles in place: rows
-// read 16 bytes at a time are aligned, and nothing the call writes overlaps them.
-bool particles_in_place(const float* B, int64_t N, int64_t p, const void* out, size_t out_bytes)
+// What the driver knows of the memory at ptr (nothing where it cannot be asked). The entry point is
+// looked up through the runtime, so the library needs no -lcuda.
+MemoryFacts memory_facts(const void* ptr)
 {
-    const uintptr_t b = reinterpret_cast<uintptr_t>(B), o = reinterpret_cast<uintptr_t>(out);
-    if ((p & 3) == 0 && (b & 15u) != 0) return false;
-    return !out || o + out_bytes <= b || b + sizeof(float) * (size_t)(N * p) <= o;
+    typedef CUresult (*GetAttributesFn)(unsigned int, CUpointer_attribute*, void**, CUdeviceptr);
+    static GetAttributesFn get = nullptr;
+    static std::once_flag once;
+    std::call_once(once, [] {
+        void* p = nullptr;
+        cudaDriverEntryPointQueryResult q;
+        if (cudaGetDriverEntryPointByVersion("cuPointerGetAttributes", &p, 12000, cudaEnableDefault, &q) == cudaSuccess &&
+            q == cudaDriverEntryPointSuccess)
+            get = reinterpret_cast<GetAttributesFn>(p);
+    });
+    MemoryFacts m;
+    unsigned int type = 0, managed = 0;
+    int ordinal = -1;
+    CUdeviceptr begin = 0;
+    size_t bytes = 0;
+    CUpointer_attribute what[5] = {CU_POINTER_ATTRIBUTE_MEMORY_TYPE, CU_POINTER_ATTRIBUTE_IS_MANAGED,
+                                   CU_POINTER_ATTRIBUTE_DEVICE_ORDINAL, CU_POINTER_ATTRIBUTE_RANGE_START_ADDR,
+                                   CU_POINTER_ATTRIBUTE_RANGE_SIZE};
+    void* out[5] = {&type, &managed, &ordinal, &begin, &bytes};
+    if (!get || get(5, what, out, (CUdeviceptr)reinterpret_cast<uintptr_t>(ptr)) != CUDA_SUCCESS) return m;
+    m.device = type == CU_MEMORYTYPE_DEVICE && managed == 0;
+    m.ordinal = ordinal;
+    m.begin = (uintptr_t)begin;
+    m.bytes = bytes;
+    return m;
+}
+
+// Whether the likelihood entry points can read the caller's device particles where they lie, given
+// an output of the call (spa_host_rules.h).
+bool reads_in_place(const spa_ctx* c, const MemoryFacts& m, const float* B, int64_t N, const void* out, size_t out_bytes)
+{
+    return particles_in_place(m, c->device, reinterpret_cast<uintptr_t>(B), N, c->p, reinterpret_cast<uintptr_t>(out),
+                              out_bytes);
 }
 
 void free_workspace(Workspace& w)
@@ -1919,7 +1950,7 @@ static int loglik_impl(spa_ctx* c, const float* B, bool B_dev, int64_t N, double
     rc = settle_stream(c, st);
     if (rc != SPA_OK) return rc;
     MoveArgs a = move_args(c, nullptr);
-    if (B_dev && particles_in_place(B, N, p, ll_dev ? ll : nullptr, sizeof(double) * (size_t)N)) {
+    if (B_dev && reads_in_place(c, memory_facts(B), B, N, ll_dev ? ll : nullptr, sizeof(double) * (size_t)N)) {
         a.beta = const_cast<float*>(B);  // packed with noise = 0: read only
     } else {
         CK(cudaMemcpyAsync(w.beta, B, sizeof(float) * (size_t)(N * p),
@@ -2132,8 +2163,9 @@ static int grad_impl(spa_ctx* c, const float* B, bool dev, int64_t N, double cs,
         q.c = c;
         q.st = st;
         MoveArgs a = move_args(c, nullptr);
-        if (dev && particles_in_place(B, N, p, grad, sizeof(float) * (size_t)(N * p)) &&
-            particles_in_place(B, N, p, ll, sizeof(double) * (size_t)N)) {
+        const MemoryFacts mf = dev ? memory_facts(B) : MemoryFacts();
+        if (reads_in_place(c, mf, B, N, grad, sizeof(float) * (size_t)(N * p)) &&
+            reads_in_place(c, mf, B, N, ll, sizeof(double) * (size_t)N)) {
             a.beta = const_cast<float*>(B);  // packed with noise = 0: read only
         } else {
             CK(cudaMemcpyAsync(w.beta, B, sizeof(float) * (size_t)(N * p),

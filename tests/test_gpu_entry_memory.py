@@ -1,0 +1,58 @@
+"""The device entry points and the caller's memory and streams: particles read where they lie or
+copied first, and work of the context that another stream has to wait for."""
+import numpy as np
+import pytest
+
+import oracle
+from paper_1106_0322_gb300 import synth
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def spa():
+    import __graft_entry__
+
+    __graft_entry__.build()
+    import paper_1106_0322_gb300 as mod
+
+    return mod
+
+
+# Read in place: an aligned base, and outputs elsewhere. Copied first: a base off by one float where
+# rows are read 16 bytes at a time (p % 4 == 0), and an output inside the particles' memory.
+@pytest.mark.parametrize("precision", ["split_bf16", "fp32"])
+@pytest.mark.parametrize("n,p,N", [(300, 20, 130), (300, 21, 130), (129, 64, 1)])
+def test_particles_copied_first_give_the_values_of_those_read_in_place(spa, precision, n, p, N):
+    import torch
+
+    reg = synth.make_region(n, p, 0.9, (0.4,), seed=1900 + n + p)
+    B = torch.from_numpy(synth.random_particles(N, p, 0.1, seed=p)).cuda()
+    st = torch.cuda.Stream()
+    with spa.Region(reg.G, reg.y, 1.0, config=spa.make_config(precision=precision)) as r:
+
+        def evaluate(b, ll, g):
+            out = torch.full((N,), float("nan"), dtype=torch.float64, device="cuda")
+            torch.cuda.synchronize()
+            r.loglik_device(b, out, st.cuda_stream)
+            r.grad_device(b, 0.7, ll, g, st.cuda_stream)
+            return out.cpu().numpy(), ll.cpu().numpy(), g.cpu().numpy()
+
+        ll, g = torch.empty(N, dtype=torch.float64, device="cuda"), torch.empty((N, p), device="cuda")
+        want = evaluate(B, ll, g)
+        assert np.allclose(want[0], oracle.loglik(reg.G, reg.y, B.cpu().numpy().astype(np.float64)), rtol=1e-3)
+        off = torch.empty(N * p + 1, device="cuda")[1:].view(N, p)
+        assert off.data_ptr() % 16 == 4
+        off.copy_(B)
+        for a, b in zip(want, evaluate(off, ll, g)):
+            assert np.array_equal(a, b)
+        # the gradient written over the particles it is of
+        over = B.clone()
+        for a, b in zip(want[1:], evaluate(over, ll, over)[1:]):
+            assert np.array_equal(a, b)
+        # the log-likelihood written into their first rows
+        room = torch.empty(max(N * p, 2 * N), device="cuda")
+        room[: N * p] = B.view(-1)
+        torch.cuda.synchronize()
+        r.loglik_device(room[: N * p].view(N, p), room.view(torch.float64)[:N], st.cuda_stream)
+        assert np.array_equal(room.view(torch.float64)[:N].cpu().numpy(), want[0])

@@ -1,0 +1,54 @@
+"""Host-side decisions of the entry points (csrc/spa_host_rules.h), compiled with the host compiler
+alone: no GPU, and none of the calls that they guard."""
+import os
+import shutil
+import subprocess
+
+import pytest
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+CSRC = os.path.join(ROOT, "paper_1106_0322_gb300", "csrc")
+
+
+def _run(tmp_path, body):
+    """Compile and run a C++ main() of CHECK(condition) lines; a failed one is reported."""
+    cxx = shutil.which("g++") or shutil.which("c++")
+    if not cxx:
+        pytest.skip("no host C++ compiler")
+    src, exe = tmp_path / "rules.cpp", tmp_path / "rules"
+    src.write_text('#include "spa_host_rules.h"\n#include <cstdio>\nstatic int bad = 0;\n'
+                   '#define CHECK(x) do { if (!(x)) { std::printf("%s\\n", #x); ++bad; } } while (0)\n'
+                   "using namespace spa;\nint main() {\n" + body + "\nreturn bad != 0; }\n")
+    subprocess.run([cxx, "-std=c++17", "-Wall", "-I", CSRC, str(src), "-o", str(exe)], check=True)
+    r = subprocess.run([str(exe)], capture_output=True, text=True)
+    assert r.returncode == 0, r.stdout
+
+
+def test_particles_are_read_in_place_only_inside_an_allocation_of_the_contexts_device(tmp_path):
+    """Device 0 holds [4096, 4096 + 6400): 100 particles of 16 coordinates fit it exactly."""
+    _run(tmp_path, """
+    MemoryFacts m; m.device = true; m.ordinal = 0; m.begin = 4096; m.bytes = 6400;
+    MemoryFacts other = m; other.ordinal = 1;
+    MemoryFacts host = m; host.device = false;
+    const MemoryFacts unknown;
+    CHECK(particles_in_place(m, 0, 4096, 100, 16, 0, 0));
+    CHECK(!particles_in_place(other, 0, 4096, 100, 16, 0, 0));
+    CHECK(particles_in_place(other, 1, 4096, 100, 16, 0, 0));
+    CHECK(!particles_in_place(host, 0, 4096, 100, 16, 0, 0));
+    CHECK(!particles_in_place(unknown, 0, 4096, 100, 16, 0, 0));
+    // past either end of the allocation
+    CHECK(!particles_in_place(m, 0, 4096, 101, 16, 0, 0));
+    CHECK(!particles_in_place(m, 0, 4112, 100, 16, 0, 0));
+    CHECK(particles_in_place(m, 0, 4112, 99, 16, 0, 0));
+    CHECK(!particles_in_place(m, 0, 4080, 10, 16, 0, 0));
+    // 16-byte rows for p % 4 == 0, 4-byte elements otherwise
+    CHECK(!particles_in_place(m, 0, 4100, 10, 16, 0, 0));
+    CHECK(particles_in_place(m, 0, 4100, 10, 15, 0, 0));
+    CHECK(!particles_in_place(m, 0, 4098, 10, 15, 0, 0));
+    // outputs that overlap: before, across, inside, behind
+    CHECK(particles_in_place(m, 0, 4896, 10, 16, 4096, 800));
+    CHECK(!particles_in_place(m, 0, 4896, 10, 16, 4096, 801));
+    CHECK(!particles_in_place(m, 0, 4896, 10, 16, 4900, 8));
+    CHECK(!particles_in_place(m, 0, 4896, 10, 16, 5535, 8));
+    CHECK(particles_in_place(m, 0, 4896, 10, 16, 5536, 8));
+    """)
