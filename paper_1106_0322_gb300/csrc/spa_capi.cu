@@ -214,9 +214,15 @@ struct spa_ctx {
     uint64_t wait_ns = 0;      // limit of the tensor-core kernels' bounded waits (0: the default)
     int tile_cfg = -1;         // likelihood tile configuration fixed by spa_set_tile_config (-1: tuned)
     int fault = 0;             // faults injected into the current sweep graph (SPA_FAULT)
-    bool own_busy = true;      // work may still run on own_stream (nothing waited for it yet)
+    OwnStream own;             // whether work may still run on own_stream
 
-    cudaStream_t stream() const { return cfg.stream ? static_cast<cudaStream_t>(cfg.stream) : own_stream; }
+    // The configured stream or the context's own, to put work on.
+    cudaStream_t stream()
+    {
+        const cudaStream_t st = cfg.stream ? static_cast<cudaStream_t>(cfg.stream) : own_stream;
+        own.handed_out(st);
+        return st;
+    }
 };
 
 namespace {
@@ -284,18 +290,21 @@ int read_error_word(spa_ctx* c, cudaStream_t st)
         CK(cudaMemsetAsync(c->d_err, 0, sizeof(uint32_t), st), "reset error word");
         CK(cudaStreamSynchronize(st), "stream synchronize");
     }
-    if (st == c->stream()) c->own_busy = false;
+    c->own.waited_for(st);
     return map_device_error(c, e);
 }
 int read_error_word(spa_ctx* c) { return read_error_word(c, c->stream()); }
 
-// Before an entry point works on a caller's stream: the context's stream is done with the
-// workspace. Its own stream needs the wait only if something was left running on it.
+// Before an entry point works on stream st: the context's other streams are done with the workspace,
+// its own where something may have been left running on it, the configured one always.
 int settle_stream(spa_ctx* c, cudaStream_t st)
 {
-    if (st == c->stream() || (!c->cfg.stream && !c->own_busy)) return SPA_OK;
-    CK(cudaStreamSynchronize(c->stream()), "sync context stream");
-    c->own_busy = false;
+    if (c->own.holds_up(st)) {
+        CK(cudaStreamSynchronize(c->own_stream), "sync the context's own stream");
+        c->own.waited_for(c->own_stream);
+    }
+    if (c->cfg.stream && st != c->cfg.stream)
+        CK(cudaStreamSynchronize(static_cast<cudaStream_t>(c->cfg.stream)), "sync the configured stream");
     return SPA_OK;
 }
 
@@ -552,7 +561,6 @@ int ensure_workspace(spa_ctx* c, int64_t N)
 {
     Workspace& w = c->ws;
     if (w.N == N) return SPA_OK;
-    c->own_busy = true;
     drop_graph(c);
     free_workspace(w);
     const int64_t p = c->p;
@@ -605,7 +613,6 @@ int ensure_adjoint_buffers(spa_ctx* c)
 {
     Workspace& w = c->ws;
     if (w.R) return SPA_OK;
-    c->own_busy = true;
     const AdjPlan a = adj_plan((int)c->p, c->n, w.N_pad, c->num_sms);
     const TcPlan plan = tc_plan(c->n, (int)c->p, w.N_pad, c->num_sms);
     cudaError_t e = dalloc(&w.R, (size_t)(w.N_pad * 2 * a.n_r));
@@ -650,7 +657,6 @@ int ensure_site_store(spa_ctx* c)
 {
     const int64_t count = site_xs_floats(c->n, c->p);
     if (count == 0 || c->XS) return SPA_OK;
-    c->own_busy = true;
     cudaError_t e = dalloc(&c->XS, (size_t)count);
     if (e != cudaSuccess) return cuda_fail(c, e, "single-coordinate store");
     CK(launch_store_xsite(c->XT2, c->n, c->p, c->XS, c->stream()), "store X for the single-coordinate kernel");
@@ -1617,6 +1623,7 @@ int spa_create(const int8_t* G, const uint8_t* y, int64_t n, int64_t p, double n
     c->pr.de = std::isinf(nu) ? 1 : 0;
     c->pr.a = c->pr.de ? 1.0f : (float)nu;
     cudaError_t e = cudaStreamCreateWithFlags(&c->own_stream, cudaStreamNonBlocking);
+    c->own.handle = c->own_stream;
     if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&c->side_stream, cudaStreamNonBlocking);
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&c->ev_fork, cudaEventDisableTiming);
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&c->ev_keys, cudaEventDisableTiming);
@@ -1752,7 +1759,6 @@ static int run_common(spa_ctx* c, const double* sched, bool sched_on_device, int
         if (rc != SPA_OK) return rc;
     }
     cudaStream_t st = c->stream();
-    c->own_busy = true;
     CK(cudaMemcpyAsync(c->rb.sched, sched, sizeof(double) * (size_t)T,
                        sched_on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, st),
        "copy schedule");
@@ -1975,7 +1981,6 @@ int spa_loglik_repeat(spa_ctx* c, int64_t N, int32_t reps, void* stream)
     if (!c) return fail(nullptr, SPA_EINVAL, "ctx is NULL");
     if (c->ws.N != N || N < 1 || reps < 0) return fail(c, SPA_EINVAL, "no workspace of N particles");
     cudaStream_t st = stream ? static_cast<cudaStream_t>(stream) : c->stream();
-    c->own_busy = true;
     Workspace& w = c->ws;
     for (int32_t k = 0; k < reps; ++k) {
         if (c->cfg.precision == SPA_PREC_SPLIT_BF16) {
@@ -1998,7 +2003,6 @@ int spa_grad_repeat(spa_ctx* c, int64_t N, int32_t reps, void* stream)
     Enq q;
     q.c = c;
     q.st = stream ? static_cast<cudaStream_t>(stream) : c->stream();
-    c->own_busy = true;
     Workspace& w = c->ws;
     for (int32_t k = 0; k < reps && q.e == cudaSuccess; ++k) enq_grad_tc(q, w.gl_p, w.beta_p, 0.0, w.N);
     if (q.e != cudaSuccess) return cuda_fail(c, q.e, "gradient kernels");

@@ -30,4 +30,21 @@ inline bool particles_in_place(const MemoryFacts& m, int ctx_device, uintptr_t b
     return out == 0 || out + out_bytes <= b || b + bytes <= out;
 }
 
+// Whether work may still run on a context's own stream, which a call on another stream has to wait for
+// because both use the context's buffers. Busy from the moment the stream is handed out to be worked
+// on, whatever becomes of the call, until the host has waited for that very stream.
+struct OwnStream {
+    const void* handle = nullptr;
+    bool busy = true;
+    void handed_out(const void* stream)
+    {
+        if (stream == handle) busy = true;
+    }
+    void waited_for(const void* stream)
+    {
+        if (stream == handle) busy = false;
+    }
+    bool holds_up(const void* stream) const { return busy && stream != handle; }
+};
+
 }  // namespace spa

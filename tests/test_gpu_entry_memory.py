@@ -56,3 +56,37 @@ def test_particles_copied_first_give_the_values_of_those_read_in_place(spa, prec
         torch.cuda.synchronize()
         r.loglik_device(room[: N * p].view(N, p), room.view(torch.float64)[:N], st.cuda_stream)
         assert np.array_equal(room.view(torch.float64)[:N].cpu().numpy(), want[0])
+
+
+def test_a_call_on_another_stream_waits_for_a_sweep_left_running(spa):
+    """A sweep is left running on the context's own stream; a call on a configured stream ends in
+    between and waits for that one only; then a caller's stream uses the same workspace."""
+    import torch
+
+    n, p, N, T, M = 1500, 100, 4096, 60, 5
+    reg = synth.make_region(n, p, 0.9, (0.4,), seed=2000)
+    sched = synth.geometric_schedule(T)
+    sched_d = torch.from_numpy(sched).cuda()
+    B = torch.from_numpy(synth.random_particles(N, p, 0.1, seed=3)).cuda()
+    ll = torch.empty(N, dtype=torch.float64, device="cuda")
+    ess = torch.empty(T, dtype=torch.float64, device="cuda")
+    conf, user = torch.cuda.Stream(), torch.cuda.Stream()
+    torch.cuda.synchronize()
+    with spa.Region(reg.G, reg.y, 1.0) as r:
+        want = r.run(sched, N, M, 7)
+        r.loglik_device(B, ll, user.cuda_stream)
+        alone = ll.cpu().numpy()
+        own_cfg, conf_cfg = r.config(), r.config()
+        conf_cfg.stream = conf.cuda_stream
+        for between in (False, True):
+            ll.fill_(float("nan"))
+            torch.cuda.synchronize()
+            r.run_device(sched_d, N, M, 7, {"ess": ess})
+            if between:
+                r.set_config(conf_cfg)
+                r.sync()
+                r.set_config(own_cfg)
+            r.loglik_device(B, ll, user.cuda_stream)
+            assert np.array_equal(ll.cpu().numpy(), alone)
+            r.sync()
+            assert np.array_equal(ess.cpu().numpy(), want["ess"])

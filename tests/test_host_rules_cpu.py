@@ -52,3 +52,39 @@ def test_particles_are_read_in_place_only_inside_an_allocation_of_the_contexts_d
     CHECK(!particles_in_place(m, 0, 4896, 10, 16, 5535, 8));
     CHECK(particles_in_place(m, 0, 4896, 10, 16, 5536, 8));
     """)
+
+
+def test_own_stream_is_waited_for_until_the_host_has_waited_for_that_very_stream(tmp_path):
+    """Handles 1 (the context's own), 2 (a configured one), 3 (a caller's)."""
+    _run(tmp_path, """
+    const void *own = (void*)1, *conf = (void*)2, *user = (void*)3;
+    OwnStream s; s.handle = own;
+    CHECK(s.holds_up(user) && !s.holds_up(own));  // nothing has waited for it yet
+    s.waited_for(own);
+    CHECK(!s.holds_up(user));
+    // a sweep enqueued on the own stream, then a call on a configured stream that waits for that one only
+    s.handed_out(own);
+    s.handed_out(conf);
+    s.waited_for(conf);
+    CHECK(s.holds_up(user) && s.holds_up(conf));
+    s.waited_for(user);
+    CHECK(s.holds_up(user));
+    s.waited_for(own);
+    CHECK(!s.holds_up(user) && !s.holds_up(conf));
+    // a call that took the stream and returned early: nobody has waited
+    s.handed_out(own);
+    CHECK(s.holds_up(user));
+    """)
+
+
+def test_every_use_of_the_contexts_stream_hands_it_out():
+    """No code of the runtime reads own_stream past stream(), except to create, wait for or destroy it."""
+    import re
+
+    src = open(os.path.join(CSRC, "spa_capi.cu")).read()
+    lines = [ln for ln in src.splitlines() if "own_stream" in re.sub(r"//.*", "", ln)]
+    allowed = (r"cudaStream_t own_stream = nullptr", r": own_stream;", r"cudaStreamCreateWithFlags\(&c->own_stream",
+               r"own\.handle = c->own_stream", r"cudaStreamSynchronize\(c->own_stream\)", r"waited_for\(c->own_stream\)",
+               r"cudaStreamDestroy\(c->own_stream\)", r"launch_step_constants\(.*c->own_stream\)")
+    for ln in lines:
+        assert any(re.search(a, ln) for a in allowed), ln
