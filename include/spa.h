@@ -75,7 +75,8 @@ typedef struct spa_config {
     double site_sd;          /* SITE: proposal sd of one coordinate (0.5: the paper's variance 0.25) */
     int32_t map_path;        /* nonzero: record each step's particle of highest posterior density,
                                 for spa_map_path after the run (default 0) */
-    void* stream;            /* cudaStream_t to run on; NULL: the context's own stream */
+    void* stream;            /* cudaStream_t to run on; NULL: the context's own stream. Setting
+                                another waits for the sweep left running on this one */
 } spa_config;
 
 /* Per-scale outputs of a sweep, caller-allocated (any pointer may be NULL to skip it).

@@ -215,6 +215,8 @@ struct spa_ctx {
     int tile_cfg = -1;         // likelihood tile configuration fixed by spa_set_tile_config (-1: tuned)
     int fault = 0;             // faults injected into the current sweep graph (SPA_FAULT)
     OwnStream own;             // whether work may still run on own_stream
+    cudaEvent_t ev_left = nullptr;  // behind the work left running on the configured stream, if `left`
+    bool left = false;
 
     // The configured stream or the context's own, to put work on.
     cudaStream_t stream()
@@ -291,6 +293,7 @@ int read_error_word(spa_ctx* c, cudaStream_t st)
         CK(cudaStreamSynchronize(st), "stream synchronize");
     }
     c->own.waited_for(st);
+    if (st == c->cfg.stream) c->left = false;
     return map_device_error(c, e);
 }
 int read_error_word(spa_ctx* c) { return read_error_word(c, c->stream()); }
@@ -337,6 +340,32 @@ MemoryFacts memory_facts(const void* ptr)
     m.begin = (uintptr_t)begin;
     m.bytes = bytes;
     return m;
+}
+
+// The call returns with work running on stream st. (A caller's configured stream may be destroyed with
+// work on it, so that is waited for by an event of the context's.)
+int leave_running(spa_ctx* c, cudaStream_t st)
+{
+    if (!c->cfg.stream || st != c->cfg.stream) return SPA_OK;
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    CK(cudaStreamIsCapturing(st, &cap), "capture status");
+    if (cap != cudaStreamCaptureStatusNone) return SPA_OK;  // nothing runs yet
+    if (!c->ev_left) CK(cudaEventCreateWithFlags(&c->ev_left, cudaEventDisableTiming), "event creation");
+    CK(cudaEventRecord(c->ev_left, st), "event record");
+    c->left = true;
+    return SPA_OK;
+}
+
+// The context is to work on another stream than until now: the work left on that one comes first.
+int change_stream(spa_ctx* c)
+{
+    if (c->own.busy) {
+        CK(cudaStreamSynchronize(c->own_stream), "sync the context's own stream");
+        c->own.waited_for(c->own_stream);
+    }
+    if (c->left) CK(cudaEventSynchronize(c->ev_left), "sync the configured stream");
+    c->left = false;
+    return SPA_OK;
 }
 
 // Whether the likelihood entry points can read the caller's device particles where they lie, given
@@ -1223,6 +1252,7 @@ void destroy(spa_ctx* c)
     if (c->ev_fork) cudaEventDestroy(c->ev_fork);
     if (c->ev_keys) cudaEventDestroy(c->ev_keys);
     if (c->ev_join) cudaEventDestroy(c->ev_join);
+    if (c->ev_left) cudaEventDestroy(c->ev_left);
     if (c->side_stream) cudaStreamDestroy(c->side_stream);
     if (c->own_stream) cudaStreamDestroy(c->own_stream);
     delete c;
@@ -1683,6 +1713,8 @@ int spa_set_config(spa_ctx* c, const spa_config* k)
     if (!c || !k) return fail(c, SPA_EINVAL, "NULL argument");
     int rc = validate_config(c, *k);
     if (rc != SPA_OK) return rc;
+    if (k->stream != c->cfg.stream) rc = change_stream(c);
+    if (rc != SPA_OK) return rc;
     if (std::memcmp(&c->cfg, k, sizeof(spa_config)) != 0) drop_graph(c);
     c->cfg = *k;
     return SPA_OK;
@@ -1840,7 +1872,7 @@ int spa_run_device(spa_ctx* c, const double* sched, int64_t T, int64_t N, int32_
         CK(d2d(out->accept_rate, r.accrate, sizeof(double) * (size_t)T), "copy acceptance");
         CK(d2d(out->resampled, r.res, (size_t)T), "copy resampled");
     }
-    return SPA_OK;
+    return leave_running(c, c->stream());
 }
 
 int spa_sync(spa_ctx* c)
@@ -1991,7 +2023,7 @@ int spa_loglik_repeat(spa_ctx* c, int64_t N, int32_t reps, void* stream)
             CK(launch_loglik_simt(w.beta_p, c->Xf, c->y, N, c->n, (int)c->p, w.partial, w.N_pad, c->num_sms, st), "loglik simt");
         }
     }
-    return SPA_OK;
+    return leave_running(c, st);
 }
 
 int spa_grad_repeat(spa_ctx* c, int64_t N, int32_t reps, void* stream)
@@ -2006,7 +2038,7 @@ int spa_grad_repeat(spa_ctx* c, int64_t N, int32_t reps, void* stream)
     Workspace& w = c->ws;
     for (int32_t k = 0; k < reps && q.e == cudaSuccess; ++k) enq_grad_tc(q, w.gl_p, w.beta_p, 0.0, w.N);
     if (q.e != cudaSuccess) return cuda_fail(c, q.e, "gradient kernels");
-    return SPA_OK;
+    return leave_running(c, q.st);
 }
 
 static MapData map_data(spa_ctx* c)

@@ -90,3 +90,29 @@ def test_a_call_on_another_stream_waits_for_a_sweep_left_running(spa):
             assert np.array_equal(ll.cpu().numpy(), alone)
             r.sync()
             assert np.array_equal(ess.cpu().numpy(), want["ess"])
+
+
+def test_a_changed_stream_waits_for_a_sweep_left_on_the_one_before(spa):
+    """Own stream to a configured one, from that to another, and back to the own one, each with a
+    sweep left running on the stream before; the sweeps share the workspace and the captured graph's
+    buffers."""
+    import torch
+
+    n, p, N, T, M = 1500, 100, 4096, 60, 5
+    reg = synth.make_region(n, p, 0.9, (0.4,), seed=2100)
+    sched = synth.geometric_schedule(T)
+    sched_d = torch.from_numpy(sched).cuda()
+    streams = [0, torch.cuda.Stream().cuda_stream, torch.cuda.Stream().cuda_stream, 0]
+    ess = [torch.empty(T, dtype=torch.float64, device="cuda") for _ in streams]
+    torch.cuda.synchronize()
+    with spa.Region(reg.G, reg.y, 1.0) as r:
+        want = [r.run(sched, N, M, 20 + k)["ess"] for k in range(len(streams))]
+        for k, s in enumerate(streams):
+            cfg = r.config()
+            cfg.stream = s or None
+            r.set_config(cfg)
+            r.run_device(sched_d, N, M, 20 + k, {"ess": ess[k]})
+        r.sync()
+    torch.cuda.synchronize()
+    for k in range(len(streams)):
+        assert np.array_equal(ess[k].cpu().numpy(), want[k])

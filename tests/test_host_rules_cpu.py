@@ -88,3 +88,15 @@ def test_every_use_of_the_contexts_stream_hands_it_out():
                r"cudaStreamDestroy\(c->own_stream\)", r"launch_step_constants\(.*c->own_stream\)")
     for ln in lines:
         assert any(re.search(a, ln) for a in allowed), ln
+
+
+def test_set_config_waits_before_the_stream_changes():
+    """Read from the source: the wait stands before the new configuration is taken over, and a sweep
+    that is left running on a configured stream is marked by an event."""
+    import re
+
+    src = re.sub(r"//[^\n]*", "", open(os.path.join(CSRC, "spa_capi.cu")).read())
+    body = src[src.index("int spa_set_config("):src.index("int spa_get_config(")]
+    assert re.search(r"if \(k->stream != c->cfg\.stream\) rc = change_stream\(c\);", body[:body.index("c->cfg = *k")])
+    run = src[src.index("int spa_run_device("):src.index("int spa_sync(")]
+    assert "return leave_running(" in run
