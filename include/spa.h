@@ -144,8 +144,9 @@ int spa_run(spa_ctx* ctx, const double* scale_schedule, int64_t T, int64_t N,
  * call only enqueues the sweep on the configured stream (no host synchronisation).
  * Inside the sweep each step's summaries run on a second stream owned by the context and
  * are joined back before the sweep's last kernel. Work enqueued on the configured stream
- * after the call therefore sees the whole sweep, outputs included. Device-side errors are
- * reported by the next spa_sync(). */
+ * after the call therefore sees the whole sweep, outputs included. With no configured stream
+ * the sweep runs after the work queued so far on the legacy default stream. Device-side errors
+ * are reported by the next spa_sync(). */
 int spa_run_device(spa_ctx* ctx, const double* scale_schedule_device, int64_t T, int64_t N,
                    int32_t moves_per_step, uint64_t seed, spa_result* out_device);
 
@@ -329,7 +330,9 @@ int spa_map_path_given(spa_ctx* ctx, const double* sched, const float* best, int
  * (Section 2, standardised X of Section 3) for N particles B (N*p floats), with the
  * context's precision: split-BF16 tcgen05 or plain FP32. ll_out: N doubles.
  * Split-BF16 bound: |err| <= (2^-15 + (2p+2) 2^-23) * sum_i (sum_j |g_ij bt_j| + |o|)
- *   + 2^-20 n + 2^-21 sum_i softplus(eta_i), with bt_j = beta_j/s_j, o = -sum_j m_j bt_j. */
+ *   + 2^-20 n + 2^-21 sum_i softplus(eta_i), with bt_j = beta_j/s_j, o = -sum_j m_j bt_j.
+ * spa_loglik_device and spa_grad_device work on `stream` and return when they are done. NULL:
+ * the context's stream, after the work queued so far on the legacy default stream. */
 int spa_loglik(spa_ctx* ctx, const float* B, int64_t N, double* ll_out);
 int spa_loglik_device(spa_ctx* ctx, const float* B_device, int64_t N, double* ll_device,
                       void* stream);

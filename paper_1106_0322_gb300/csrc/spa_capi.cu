@@ -217,6 +217,7 @@ struct spa_ctx {
     OwnStream own;             // whether work may still run on own_stream
     cudaEvent_t ev_left = nullptr;  // behind the work left running on the configured stream, if `left`
     bool left = false;
+    cudaEvent_t ev_default = nullptr;  // behind the default stream's work (follow_default_stream)
 
     // The configured stream or the context's own, to put work on.
     cudaStream_t stream()
@@ -340,6 +341,21 @@ MemoryFacts memory_facts(const void* ptr)
     m.begin = (uintptr_t)begin;
     m.bytes = bytes;
     return m;
+}
+
+// A device entry point given NULL (spa_run_device: configured with it), which is also the handle of the
+// legacy default stream (torch's default one), works on the context's stream st. That is not ordered with the default stream, so the
+// work queued there (what fills the particles, or still reads the output's memory) comes first.
+int follow_default_stream(spa_ctx* c, cudaStream_t st)
+{
+    const cudaError_t q = cudaStreamQuery(cudaStreamLegacy);
+    if (q == cudaSuccess) return SPA_OK;  // nothing queued: the query alone, no event
+    (void)cudaGetLastError();             // "not ready" is no error
+    if (q != cudaErrorNotReady) return cuda_fail(c, q, "query the default stream");
+    if (!c->ev_default) CK(cudaEventCreateWithFlags(&c->ev_default, cudaEventDisableTiming), "event creation");
+    CK(cudaEventRecord(c->ev_default, cudaStreamLegacy), "event record");
+    CK(cudaStreamWaitEvent(st, c->ev_default, 0), "wait for the default stream");
+    return SPA_OK;
 }
 
 // The call returns with work running on stream st. (A caller's configured stream may be destroyed with
@@ -1253,6 +1269,7 @@ void destroy(spa_ctx* c)
     if (c->ev_keys) cudaEventDestroy(c->ev_keys);
     if (c->ev_join) cudaEventDestroy(c->ev_join);
     if (c->ev_left) cudaEventDestroy(c->ev_left);
+    if (c->ev_default) cudaEventDestroy(c->ev_default);
     if (c->side_stream) cudaStreamDestroy(c->side_stream);
     if (c->own_stream) cudaStreamDestroy(c->own_stream);
     delete c;
@@ -1791,6 +1808,10 @@ static int run_common(spa_ctx* c, const double* sched, bool sched_on_device, int
         if (rc != SPA_OK) return rc;
     }
     cudaStream_t st = c->stream();
+    if (sched_on_device && !c->cfg.stream) {
+        rc = follow_default_stream(c, st);
+        if (rc != SPA_OK) return rc;
+    }
     CK(cudaMemcpyAsync(c->rb.sched, sched, sizeof(double) * (size_t)T,
                        sched_on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, st),
        "copy schedule");
@@ -1986,6 +2007,7 @@ static int loglik_impl(spa_ctx* c, const float* B, bool B_dev, int64_t N, double
     const int64_t p = c->p;
     const bool tc = c->cfg.precision == SPA_PREC_SPLIT_BF16;
     rc = settle_stream(c, st);
+    if (rc == SPA_OK && B_dev && !st_user) rc = follow_default_stream(c, st);
     if (rc != SPA_OK) return rc;
     MoveArgs a = move_args(c, nullptr);
     if (B_dev && reads_in_place(c, memory_facts(B), B, N, ll_dev ? ll : nullptr, sizeof(double) * (size_t)N)) {
@@ -2194,6 +2216,7 @@ static int grad_impl(spa_ctx* c, const float* B, bool dev, int64_t N, double cs,
         }
         cudaStream_t st = st_user ? st_user : c->stream();
         rc = settle_stream(c, st);
+        if (rc == SPA_OK && dev && !st_user) rc = follow_default_stream(c, st);
         if (rc != SPA_OK) return rc;
         Enq q;
         q.c = c;
@@ -2226,6 +2249,7 @@ static int grad_impl(spa_ctx* c, const float* B, bool dev, int64_t N, double cs,
     }
     cudaStream_t st = st_user ? st_user : c->stream();
     rc = settle_stream(c, st);
+    if (rc == SPA_OK && dev && !st_user) rc = follow_default_stream(c, st);
     if (rc != SPA_OK) return rc;
     CK(cudaMemcpyAsync(w.beta, B, sizeof(float) * (size_t)(N * p), dev ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, st),
        "copy B");

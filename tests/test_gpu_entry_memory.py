@@ -116,3 +116,59 @@ def test_a_changed_stream_waits_for_a_sweep_left_on_the_one_before(spa):
     torch.cuda.synchronize()
     for k in range(len(streams)):
         assert np.array_equal(ess[k].cpu().numpy(), want[k])
+
+
+# Work queued on torch's default stream just before the call: 20 ms of it, then the update of the
+# particles that the call is to see.
+@pytest.mark.parametrize("precision", ["split_bf16", "fp32"])
+def test_calls_without_a_stream_see_what_the_default_stream_has_queued(spa, precision):
+    import torch
+
+    n, p, N = 500, 40, 2000
+    reg = synth.make_region(n, p, 0.9, (0.4,), seed=2200)
+    old, new = (torch.from_numpy(synth.random_particles(N, p, 0.1, seed=s)).cuda() for s in (1, 2))
+    ll, g = torch.empty(N, dtype=torch.float64, device="cuda"), torch.empty((N, p), device="cuda")
+
+    def queue(B):
+        torch.cuda.synchronize()
+        torch.cuda._sleep(40_000_000)
+        B.copy_(new)
+
+    with spa.Region(reg.G, reg.y, 1.0, config=spa.make_config(precision=precision)) as r:
+        want_ll, want_g = r.grad(new.cpu().numpy())
+        want = r.loglik(new.cpu().numpy())
+        B = old.clone()
+        queue(B)
+        r.loglik_device(B, ll)
+        assert np.array_equal(ll.cpu().numpy(), want)
+        B.copy_(old)
+        queue(B)
+        r.grad_device(B, 0.0, ll, g)
+        assert np.array_equal(ll.cpu().numpy(), want_ll) and np.array_equal(g.cpu().numpy(), want_g)
+        B = old.clone().requires_grad_(True)
+        with torch.no_grad():
+            queue(B)
+        out = spa.loglik_autograd(B, r)
+        torch.cuda._sleep(40_000_000)
+        (grad,) = torch.autograd.grad(out, B, torch.full_like(out, 2.0))
+        assert np.array_equal(out.detach().cpu().numpy(), want)
+        assert np.array_equal(grad.cpu().numpy(), 2.0 * want_g)
+        # a block of the output's memory that the default stream still reads when the call writes it
+        keep = torch.empty((N, p), device="cuda")
+        g.fill_(7.0)
+        torch.cuda.synchronize()
+        torch.cuda._sleep(40_000_000)
+        keep.copy_(g)
+        r.grad_device(new, 0.0, ll, g)
+        assert bool((keep == 7.0).all()) and np.array_equal(g.cpu().numpy(), want_g)
+        # a schedule that the default stream is still to write
+        sched = synth.geometric_schedule(5)
+        want_ess = r.run(sched, N, 1, 3)["ess"]
+        later, ess = torch.from_numpy(sched).cuda(), torch.empty(5, dtype=torch.float64, device="cuda")
+        sched_d = torch.full((5,), 0.5, dtype=torch.float64, device="cuda")
+        torch.cuda.synchronize()
+        torch.cuda._sleep(40_000_000)
+        sched_d.copy_(later)
+        r.run_device(sched_d, N, 1, 3, {"ess": ess})
+        r.sync()
+        assert np.array_equal(ess.cpu().numpy(), want_ess)

@@ -100,3 +100,20 @@ def test_set_config_waits_before_the_stream_changes():
     assert re.search(r"if \(k->stream != c->cfg\.stream\) rc = change_stream\(c\);", body[:body.index("c->cfg = *k")])
     run = src[src.index("int spa_run_device("):src.index("int spa_sync(")]
     assert "return leave_running(" in run
+
+
+def test_device_entry_points_follow_the_default_stream_when_given_its_handle():
+    """Read from the source: the legacy default stream's handle is NULL, which the entry points take
+    as the context's own (non-blocking) stream; each orders that behind the default stream."""
+    import re
+
+    src = re.sub(r"//[^\n]*", "", open(os.path.join(CSRC, "spa_capi.cu")).read())
+    loglik = src[src.index("static int loglik_impl("):src.index("int spa_loglik_repeat(")]
+    grad = src[src.index("static int grad_impl("):src.index("int spa_grad(")]
+    for body, dev in ((loglik, "B_dev"), (grad, "dev")):
+        settled = body.count("rc = settle_stream(c, st);")
+        assert settled >= 1
+        assert len(re.findall(r"if \(rc == SPA_OK && %s && !st_user\) rc = follow_default_stream\(c, st\);" % dev,
+                              body)) == settled
+    run = src[src.index("static int run_common("):src.index("int spa_run(")]
+    assert re.search(r"if \(sched_on_device && !c->cfg\.stream\) \{\s*rc = follow_default_stream\(c, st\);", run)
