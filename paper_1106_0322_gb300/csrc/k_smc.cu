@@ -33,21 +33,25 @@ __device__ __forceinline__ int64_t warp_global_id()
 // The log prior's coefficient of its term sum (prior_term, spa_device.cuh), FP64.
 __device__ __forceinline__ double prior_coef(PriorArgs pr, double c) { return pr.de ? -1.0 / c : -((double)pr.a + 1.0); }
 
-// The prior's gradient in MALA's drift. The drift can be any fixed function of the state:
-// the MH test evaluates the forward and reverse proposal densities with this same function,
-// so the fast quotient (within 2 ulp) keeps each step's kernel exactly pi_t-invariant.
-__device__ __forceinline__ float dlogprior(float b, float a1, float ac, float inv_c, int de)
+// MALA's drift is (h^2/2) D_j times the slope of the log posterior: g = grad l plus the prior's part,
+// -(a+1) sgn(b)/(a c + |b|) or, for the double exponential, -sgn(b)/c. The quotient is the product with
+// the approximate reciprocal (rcp.approx.ftz.f32, 1 ulp): the drift may be any fixed function of the
+// state. Every operation is rounded as written, so that the slope does not depend on how the compiler
+// joins it to the code around, which differs between the kernels. The forward density rounds the prior's
+// part before the sum, the reverse density (slope_reverse) adds it in one rounding: the two are within
+// 2^-24 of the prior's part of each other, which enters log alpha as the FP32 roundings of the two
+// residual sums do. One rounding in both would be the cleaner rule, but gives every sweep whose a + 1 is
+// not a power of two other bits.
+__device__ __forceinline__ float slope_sign(float b, float v) { return b > 0.0f ? -v : (b < 0.0f ? v : 0.0f); }
+__device__ __forceinline__ float slope_forward(float g, float b, float a1, float ac, float inv_c, int de)
 {
-    const float sg = (b > 0.0f) ? 1.0f : ((b < 0.0f) ? -1.0f : 0.0f);
-    return de ? -sg * inv_c : __fdividef(-a1 * sg, ac + fabsf(b));
+    return __fadd_rn(g, de ? __fmul_rn(slope_sign(b, 1.0f), inv_c)
+                           : __fmul_rn(slope_sign(b, a1), rcp_approx(__fadd_rn(ac, fabsf(b)))));
 }
-
-// g + dlogprior(b) as one multiply-add: what the sum of the two compiles to in the MALA kernels, written
-// out so that the reverse move's bits do not depend on the code around it.
-__device__ __forceinline__ float dlogpost(float g, float b, float a1, float ac, float inv_c, int de)
+__device__ __forceinline__ float slope_reverse(float g, float b, float a1, float ac, float inv_c, int de)
 {
-    const float sg = (b > 0.0f) ? 1.0f : ((b < 0.0f) ? -1.0f : 0.0f);
-    return de ? fmaf(-sg, inv_c, g) : fmaf(-a1 * sg, rcp_approx(ac + fabsf(b)), g);
+    return de ? __fmaf_rn(slope_sign(b, 1.0f), inv_c, g)
+              : __fmaf_rn(slope_sign(b, a1), rcp_approx(__fadd_rn(ac, fabsf(b))), g);
 }
 
 // ------------------------------------------------------------------- init (t = 0)
@@ -553,7 +557,7 @@ __device__ __forceinline__ FSum mala_reverse(const MoveArgs& a, int64_t i, int p
             const float4 Dv = ldg4(a.sigma + j0), iD = ldg4(a.inv_D + j0);
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
-                const float drift = h2 * comp(Dv, k) * dlogpost(comp(gg, k), comp(x1, k), a1, ac, inv_c, de);
+                const float drift = h2 * comp(Dv, k) * slope_reverse(comp(gg, k), comp(x1, k), a1, ac, inv_c, de);
                 const float d = (comp(x0, k) - comp(x1, k)) - drift;
                 bwd.add(d * d * comp(iD, k));
             }
@@ -567,7 +571,7 @@ __device__ __forceinline__ FSum mala_reverse(const MoveArgs& a, int64_t i, int p
                 const int j = j0 + 32 * k;
                 if (j >= p) break;
                 g1[j] = g4[k];
-                const float drift = h2 * a.sigma[j] * dlogpost(g4[k], b1[j], a1, ac, inv_c, de);
+                const float drift = h2 * a.sigma[j] * slope_reverse(g4[k], b1[j], a1, ac, inv_c, de);
                 const float d = (b0[j] - b1[j]) - drift;
                 bwd.add(d * d * a.inv_D[j]);
             }
@@ -577,7 +581,7 @@ __device__ __forceinline__ FSum mala_reverse(const MoveArgs& a, int64_t i, int p
     } else {
         const float* g = a.gl_p + i * p;
         for (int j = lane; j < p; j += 32) {
-            const float drift = h2 * a.sigma[j] * dlogpost(g[j], b1[j], a1, ac, inv_c, de);
+            const float drift = h2 * a.sigma[j] * slope_reverse(g[j], b1[j], a1, ac, inv_c, de);
             const float d = (b0[j] - b1[j]) - drift;
             bwd.add(d * d * a.inv_D[j]);
         }
@@ -667,7 +671,7 @@ __global__ void __launch_bounds__(BLOCK, 4) k_move_mala(MoveArgs a, int64_t N, i
 #pragma unroll
                 for (int k = 0; k < 4; ++k) {
                     const float b0 = comp(x0, k);
-                    const float drift = h2 * comp(Dv, k) * (comp(g0, k) + dlogprior(b0, a1, ac, inv_c, pr.de));
+                    const float drift = h2 * comp(Dv, k) * slope_forward(comp(g0, k), b0, a1, ac, inv_c, pr.de);
                     const float b = (b0 + drift) + h * comp(sD, k) * comp(z4, k);
                     const float d = (b - b0) - drift;
                     fw.add(d * d * comp(iD, k));
@@ -698,7 +702,7 @@ __global__ void __launch_bounds__(BLOCK, 4) k_move_mala(MoveArgs a, int64_t N, i
                         cur[j] = b0;
                         gcur[j] = g0;
                     }
-                    const float drift = h2 * D[j] * (g0 + dlogprior(b0, a1, ac, inv_c, pr.de));
+                    const float drift = h2 * D[j] * slope_forward(g0, b0, a1, ac, inv_c, pr.de);
                     const float b = (b0 + drift) + h * a.sqrt_D[j] * comp(z4, k);
                     dst[j] = b;
                     const float d = (b - b0) - drift;

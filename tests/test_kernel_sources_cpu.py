@@ -34,3 +34,17 @@ def test_mala_gradient_row_is_ordered_between_the_lanes_that_write_and_read_it()
     after_store = rev[store:]
     between = move[move.index("mala_reverse<") : move.index("gsrc[j]")]
     assert re.search(r"__syncwarp\(\)|__syncthreads\(\)", after_store + between)
+
+
+def test_mala_drift_is_rounded_as_written_in_both_densities():
+    """The slope in MALA's drift comes from functions whose every operation names its rounding, in the
+    reverse density and in the forward one, instead of from a sum that the compiler may contract."""
+    src = _code("k_smc.cu")
+    drifts = re.findall(r"const float drift = [^;]*;", src)
+    assert len(drifts) == 5
+    assert [bool(re.search(r"\* slope_reverse\([^;]*\);$", d)) for d in drifts] == [True] * 3 + [False] * 2
+    assert [bool(re.search(r"\* slope_forward\([^;]*\);$", d)) for d in drifts] == [False] * 3 + [True] * 2
+    for name in ("slope_forward(", "slope_reverse("):
+        body = _body(src, "__device__ __forceinline__ float " + name)
+        assert re.search(r"__f(maf|add)_rn\(", body)
+        assert not re.search(r"[^_a-z] [+*/-] |__fdividef", body)
