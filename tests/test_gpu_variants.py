@@ -182,3 +182,17 @@ def test_mala_decisions_do_not_depend_on_the_launches(spa, n, p):
             b.close()
             for k in one:
                 assert np.array_equal(one[k], two[k]), k
+
+
+@pytest.mark.parametrize("n,p,N", [(31, 1, 4096), (33, 2, 3001)])
+def test_site_kernel_of_the_smallest_regions_takes_the_oracles_decisions(spa, n, p, N):
+    """As above at sizes where a handful of flips cannot hide a wrong decision: of about 5000
+    decisions fewer than one is expected to lie within 1e-5 of its log U, two may flip."""
+    reg = synth.make_region(n, p, 0.9, (0.5,), seed=1200 + n)
+    sched = synth.geometric_schedule(2, -3.0, -2.0)
+    with spa.Region(reg.G, reg.y, 1.0, config=spa.make_config(move="site", init="resample_move")) as r:
+        g = r.run(sched, N, 1, 11)
+    o = oracle.run(reg.G, reg.y, 1.0, sched, N, 1, seed=11,
+                   cfg=oracle.make_config(move="site", init="mcmc"))
+    assert abs(g["accept_rate"][0] - o["accept_rate"][0]) <= 2.0 / (N * p) + 1e-12
+    assert np.max(np.abs(g["mean"][0] - o["mean"][0])) <= 2 * 2.0 / N + 1e-4
