@@ -345,13 +345,11 @@ MemoryFacts memory_facts(const void* ptr)
 
 // A device entry point given NULL (spa_run_device: configured with it), which is also the handle of the
 // legacy default stream (torch's default one), works on the context's stream st. That is not ordered with the default stream, so the
-// work queued there (what fills the particles, or still reads the output's memory) comes first.
+// work queued there (what fills the particles, or still reads the output's memory) comes first. The
+// event and the wait take 0.7 us of a 29 us call (n = 500, p = 50, N = 128); asking first whether the
+// stream is idle (cudaStreamQuery) took 2.
 int follow_default_stream(spa_ctx* c, cudaStream_t st)
 {
-    const cudaError_t q = cudaStreamQuery(cudaStreamLegacy);
-    if (q == cudaSuccess) return SPA_OK;  // nothing queued: the query alone, no event
-    (void)cudaGetLastError();             // "not ready" is no error
-    if (q != cudaErrorNotReady) return cuda_fail(c, q, "query the default stream");
     if (!c->ev_default) CK(cudaEventCreateWithFlags(&c->ev_default, cudaEventDisableTiming), "event creation");
     CK(cudaEventRecord(c->ev_default, cudaStreamLegacy), "event record");
     CK(cudaStreamWaitEvent(st, c->ev_default, 0), "wait for the default stream");
