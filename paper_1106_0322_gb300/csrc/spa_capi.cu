@@ -199,7 +199,8 @@ struct spa_ctx {
     CUtensorMap mapGT;
     int mapGT_BN = 0;
     uint32_t* d_err = nullptr;
-    uint32_t* h_err = nullptr;  // pinned: where the error word is copied to
+    uint32_t* h_err = nullptr;  // pinned (take_pinned_word): where the error word is copied to
+    unsigned long long h_err_owner = 0;
     Workspace ws;
     RunBufs rb;
     cudaGraphExec_t gexec = nullptr;
@@ -270,6 +271,34 @@ int check_device(spa_ctx* c)
         c->num_sms = prop.multiProcessorCount;
     }
     return SPA_OK;
+}
+
+// The words outlive the library's other statics: contexts may be destroyed while a process ends.
+PinnedWords& pinned_words()
+{
+    static PinnedWords* w = new PinnedWords();
+    return *w;
+}
+cudaError_t take_pinned_word(spa_ctx* c)
+{
+    cudaError_t e = cudaSuccess;
+    auto alloc = [&e](size_t bytes) {
+        void* b = nullptr;
+        e = cudaHostAlloc(&b, bytes, cudaHostAllocDefault);
+        return e == cudaSuccess ? b : nullptr;
+    };
+    c->h_err_owner = current_context_id();
+    c->h_err = c->h_err_owner ? pinned_words().take(c->h_err_owner, alloc) : static_cast<uint32_t*>(alloc(sizeof(uint32_t)));
+    return e;
+}
+void give_pinned_word(spa_ctx* c)
+{
+    auto free = [](void* b) { cudaFreeHost(b); };
+    if (c->h_err && c->h_err_owner)
+        pinned_words().give(c->h_err, c->h_err_owner, current_context_id(), free);
+    else if (c->h_err)
+        free(c->h_err);
+    c->h_err = nullptr;
 }
 
 int map_device_error(spa_ctx* c, uint32_t e)
@@ -1262,7 +1291,7 @@ void destroy(spa_ctx* c)
     dfree(c->G); dfree(c->y); dfree(c->sums); dfree(c->mean); dfree(c->sd); dfree(c->v); dfree(c->unit_c); dfree(c->unit_k);
     dfree(c->l2e_s); dfree(c->mean_f); dfree(c->colf); dfree(c->Xf); dfree(c->Gbf); dfree(c->d_err); dfree(c->GT); dfree(c->yv);
     dfree(c->ybits); dfree(c->XT2); dfree(c->XS); dfree(c->lip);
-    if (c->h_err) cudaFreeHost(c->h_err);
+    give_pinned_word(c);
     if (c->ev_fork) cudaEventDestroy(c->ev_fork);
     if (c->ev_keys) cudaEventDestroy(c->ev_keys);
     if (c->ev_join) cudaEventDestroy(c->ev_join);
@@ -1691,7 +1720,7 @@ int spa_create(const int8_t* G, const uint8_t* y, int64_t n, int64_t p, double n
     CA(ybits, c->ywords);
     CA(d_err, 1);
 #undef CA
-    if (e == cudaSuccess) e = cudaHostAlloc(reinterpret_cast<void**>(&c->h_err), sizeof(uint32_t), cudaHostAllocDefault);
+    if (e == cudaSuccess) e = take_pinned_word(c);
     if (e != cudaSuccess) {
         set_thread_error_str(std::string("device allocation: ") + cudaGetErrorString(e));
         destroy(c);

@@ -16,6 +16,8 @@ constexpr double LOG2E = 1.4426950408889634073599246810019;
 // Set the message spa_last_error(NULL) returns on this thread ("msg" followed by value
 // when value >= 0). Writes into fixed storage; never allocates.
 void set_thread_error(const char* msg, int64_t value = -1);
+// The unique ID of the calling thread's current CUDA context (0 if it cannot be read).
+unsigned long long current_context_id();
 
 // ----------------------------------------------------------- genotype store
 // Integer column sums of G (S1 = sum g, S2 = sum g^2, SY = sum y g) and the case count,

@@ -36,13 +36,21 @@ struct ScratchSlot {
 std::mutex g_mu;
 ScratchSlot g_scratch[MAX_DEVICES];
 
-typedef CUresult (*CtxGetCurrentFn)(CUcontext*);
-typedef CUresult (*CtxGetIdFn)(CUcontext, unsigned long long*);
-
-// The unique ID of the calling thread's current context (0 if it cannot be read). The
-// driver entry points are looked up through the runtime, so the library needs no -lcuda.
-unsigned long long current_context_id()
+int cuda_error(const char* what, cudaError_t e)
 {
+    char msg[256];
+    std::snprintf(msg, sizeof(msg), "spa_resample_systematic_noalloc: %s: %s", what, cudaGetErrorString(e));
+    spa::set_thread_error(msg);
+    return SPA_ECUDA;
+}
+
+}  // namespace
+
+// The driver entry points are looked up through the runtime, so the library needs no -lcuda.
+unsigned long long spa::current_context_id()
+{
+    typedef CUresult (*CtxGetCurrentFn)(CUcontext*);
+    typedef CUresult (*CtxGetIdFn)(CUcontext, unsigned long long*);
     static CtxGetCurrentFn get_current = nullptr;
     static CtxGetIdFn get_id = nullptr;
     static std::once_flag once;
@@ -63,16 +71,6 @@ unsigned long long current_context_id()
     if (get_current(&ctx) != CUDA_SUCCESS || !ctx || get_id(ctx, &id) != CUDA_SUCCESS) return 0;
     return id;
 }
-
-int cuda_error(const char* what, cudaError_t e)
-{
-    char msg[256];
-    std::snprintf(msg, sizeof(msg), "spa_resample_systematic_noalloc: %s: %s", what, cudaGetErrorString(e));
-    spa::set_thread_error(msg);
-    return SPA_ECUDA;
-}
-
-}  // namespace
 
 extern "C" int spa_resample_systematic_noalloc(const double* W_device, int64_t N, double u, int32_t* idx_device,
                                                void* stream)
@@ -109,7 +107,7 @@ extern "C" int spa_resample_systematic_noalloc(const double* W_device, int64_t N
     double* scratch = nullptr;
     {
         std::lock_guard<std::mutex> lock(g_mu);
-        const unsigned long long id = current_context_id();
+        const unsigned long long id = spa::current_context_id();
         ScratchSlot& s = g_scratch[dev];
         if (!s.ptr || id == 0 || s.ctx_id != id) {
             // First call on this device in this context: the array's name is only a host

@@ -16,10 +16,10 @@ def _run(tmp_path, body):
     if not cxx:
         pytest.skip("no host C++ compiler")
     src, exe = tmp_path / "rules.cpp", tmp_path / "rules"
-    src.write_text('#include "spa_host_rules.h"\n#include <cstdio>\nstatic int bad = 0;\n'
+    src.write_text('#include "spa_host_rules.h"\n#include <cstdio>\n#include <cstdlib>\n#include <thread>\nstatic int bad = 0;\n'
                    '#define CHECK(x) do { if (!(x)) { std::printf("%s\\n", #x); ++bad; } } while (0)\n'
                    "using namespace spa;\nint main() {\n" + body + "\nreturn bad != 0; }\n")
-    subprocess.run([cxx, "-std=c++17", "-Wall", "-I", CSRC, str(src), "-o", str(exe)], check=True)
+    subprocess.run([cxx, "-std=c++17", "-Wall", "-pthread", "-I", CSRC, str(src), "-o", str(exe)], check=True)
     r = subprocess.run([str(exe)], capture_output=True, text=True)
     assert r.returncode == 0, r.stdout
 
@@ -88,6 +88,52 @@ def test_every_use_of_the_contexts_stream_hands_it_out():
                r"cudaStreamDestroy\(c->own_stream\)", r"launch_step_constants\(.*c->own_stream\)")
     for ln in lines:
         assert any(re.search(a, ln) for a in allowed), ln
+
+
+def test_pinned_words_are_shared_by_page_given_back_and_kept_to_their_cuda_context(tmp_path):
+    _run(tmp_path, """
+    PinnedWords pool;
+    std::vector<void*> made, freed;
+    auto alloc = [&](size_t n) { made.push_back(std::aligned_alloc(4096, n)); return made.back(); };
+    auto release = [&](void* p) { freed.push_back(p); };
+    std::vector<uint32_t*> w;
+    for (int k = 0; k < 130; ++k) w.push_back(pool.take(7, alloc));
+    CHECK(made.size() == 3);  // 64 to a page
+    for (size_t a = 0; a < w.size(); ++a)
+        for (size_t b = 0; b < a; ++b) CHECK((w[a] > w[b] ? w[a] - w[b] : w[b] - w[a]) >= 16);
+    pool.give(w[3], 7, 7, release);
+    CHECK(pool.take(7, alloc) == w[3] && made.size() == 3);
+    // another CUDA context never gets words of this one's pages
+    uint32_t* other = pool.take(8, alloc);
+    CHECK(made.size() == 4 && other == made[3]);
+    // empty pages are freed, the last one kept for the next context
+    for (uint32_t* x : w) pool.give(x, 7, 7, release);
+    CHECK(freed.size() == 2 && pool.pages() == 2);
+    CHECK(pool.take(7, alloc) && made.size() == 4);
+    // given back from a thread in another CUDA context, or after a reset: nothing is freed there
+    uint32_t* one = pool.take(9, alloc);
+    std::vector<uint32_t*> nine;
+    for (int k = 0; k < 64; ++k) nine.push_back(pool.take(9, alloc));
+    for (uint32_t* x : nine) pool.give(x, 9, 8, release);
+    pool.give(one, 9, 0, release);
+    CHECK(freed.size() == 2);
+    // no memory: no word, and nothing is kept of the attempt
+    const size_t before = pool.pages();
+    CHECK(pool.take(10, [](size_t) { return (void*)nullptr; }) == nullptr && pool.pages() == before);
+    // two threads take and give words of one CUDA context
+    auto work = [&] {
+        for (int k = 0; k < 2000; ++k) {
+            uint32_t* x = pool.take(11, [](size_t n) { return std::aligned_alloc(4096, n); });
+            *x = (uint32_t)k;
+            if (*x != (uint32_t)k) ++bad;
+            pool.give(x, 11, 11, [](void* p) { std::free(p); });
+        }
+    };
+    std::thread t1(work), t2(work);
+    t1.join();
+    t2.join();
+    CHECK(pool.pages() == before + 1);
+    """)
 
 
 def test_set_config_waits_before_the_stream_changes():
