@@ -33,7 +33,7 @@ namespace spa {
 namespace {
 
 constexpr int MAP_THREADS = 512;
-constexpr int MAP_REG_P = 64;  // markers a thread can hold of its individual (load_x)
+constexpr int MAP_REG_P = 64;  // markers a thread can hold of its individual (map_em_block)
 constexpr int MAP_MAX_INNER = 4000;  // proximal-gradient steps per EM step
 
 __device__ __forceinline__ float block_sum_f(float v, float* red)

@@ -299,10 +299,10 @@ __device__ __forceinline__ void draw_accept_logu(const MhState& s, int64_t N, in
     s.lu[(int64_t)(m & 1u) * s.ld_lu + i] = logf(u01_open_f(u.x));
 }
 
-// Warp-cooperative MH test of particle i's pending proposal; `extra` is the MALA
-// q-correction. Lane 0 decides with the accept uniform of move m_prev (drawn by the kernel
-// that proposed it) and, on acceptance, moves the proposal's log-likelihood and log-prior
-// into the current state. Returns the decision on every lane.
+// MH test of particle i's pending proposal, by one lane: L is the proposal's log-likelihood, `extra`
+// the MALA q-correction. It decides with the accept uniform of move m_prev (drawn by the kernel that
+// proposed it) and, on acceptance, moves the proposal's log-likelihood and log-prior into the
+// current state.
 __device__ __forceinline__ bool mh_test(const MhState& s, const FSum& L, int64_t i, float coef, float extra, uint32_t m_prev,
                                         uint32_t* err)
 {
@@ -1096,7 +1096,8 @@ __global__ void k_mark_uniform(int64_t N, int t, double* ess_out, uint8_t* res_o
 // in index order, a running sum of the block totals, C_i = carry(block) + local_i. cum holds
 // N + ceil(N/256) + 1 doubles: the block-local running sums, then one carry per block, then u.
 // Three kernels spread it over the SMs: the local sums (a warp per block), the carries (one
-// warp, in block order), and the search, which forms C_i = carry + local_i as it reads it.
+// warp, in block order), and the search, which forms C_i = carry + local_i as it reads it. A sweep of
+// up to 64 blocks takes the local sums alone, the rest in its gather (k_resample_gather).
 // Every bit of C is that of additions in the definition's order (running_sums).
 constexpr int RS_BLOCK = 256;  // cumulative-sum block of the specified association order
 constexpr int RS_CHUNKS = 4;   // 256-blocks (warps) per CTA of the local pass

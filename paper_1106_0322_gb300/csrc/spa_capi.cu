@@ -1356,11 +1356,6 @@ void batch_free(spa_batch* b)
     delete b;
 }
 
-// Lock-step batching (SPA_BATCH_MODE=lockstep) needs every region's sweep to stop at the
-// same likelihood evaluations: the same T, N, M, move kind (random walk or MALA), start and
-// burn-in, all on the tensor cores. By default the batch is one graph branch per region: on
-// the 64-region batched workload that measures 1.84 s per batch against 2.26 s in lock step,
-// whose joins at every evaluation stop the regions' other kernels from overlapping.
 // The SMs each region's likelihood launches are sized for when a batch runs its regions as
 // graph branches side by side: shares in proportion to the regions' work, twice the GPU in all
 // (an eighth of it a region on average from 16 regions on). Smaller grids give each CTA more units
@@ -1390,6 +1385,11 @@ std::vector<int> batch_plan_sms(const spa_batch* b, const spa_batch_args* args)
     return sms;
 }
 
+// Lock-step batching (SPA_BATCH_MODE=lockstep) needs every region's sweep to stop at the
+// same likelihood evaluations: the same T, N, M, move kind (random walk or MALA), start and
+// burn-in, all on the tensor cores. By default the batch is one graph branch per region: on
+// the 64-region batched workload that measures 1.84 s per batch against 2.26 s in lock step,
+// whose joins at every evaluation stop the regions' other kernels from overlapping.
 bool batch_lockstep(spa_ctx* const* ctxs, int32_t R, const spa_batch_args* args)
 {
     const char* env = std::getenv("SPA_BATCH_MODE");
